@@ -219,8 +219,8 @@ def _guess_net():
     h = _silu(_silu(_features(cons) @ W1.T + b1) @ W2.T + b2)
     A = torch.cat([h, torch.ones_like(h[:, :1])], 1)
     y = _target(cons, prim[4])
-    G = A.T @ A + 1e-4 * torch.eye(65, dtype=torch.float64, device="cuda")
-    P[4416:] = torch.linalg.solve(G, A.T @ y)
+    G, r = (A.T @ A).cpu().numpy() + 1e-4 * np.eye(65), (A.T @ y).cpu().numpy()
+    P[4416:] = torch.from_numpy(np.linalg.solve(G, r)).cuda()
     return _Net(P)
 
 
