@@ -209,13 +209,13 @@ cudaError_t launch_stage_fp64_n5(int, int, const StageArgs &, long long, cudaStr
 cudaError_t launch_stage_fp64_n6(int, int, const StageArgs &, long long, cudaStream_t);
 cudaError_t launch_stage_fp64_n7(int, int, const StageArgs &, long long, cudaStream_t);
 cudaError_t launch_stage_fp64_n8(int, int, const StageArgs &, long long, cudaStream_t);
-cudaError_t launch_summaries_n2(const SummaryArgs &, long long, cudaStream_t);
-cudaError_t launch_summaries_n3(const SummaryArgs &, long long, cudaStream_t);
-cudaError_t launch_summaries_n4(const SummaryArgs &, long long, cudaStream_t);
-cudaError_t launch_summaries_n5(const SummaryArgs &, long long, cudaStream_t);
-cudaError_t launch_summaries_n6(const SummaryArgs &, long long, cudaStream_t);
-cudaError_t launch_summaries_n7(const SummaryArgs &, long long, cudaStream_t);
-cudaError_t launch_summaries_n8(const SummaryArgs &, long long, cudaStream_t);
+cudaError_t launch_summaries_n2(const SummaryArgs &, cudaStream_t);
+cudaError_t launch_summaries_n3(const SummaryArgs &, cudaStream_t);
+cudaError_t launch_summaries_n4(const SummaryArgs &, cudaStream_t);
+cudaError_t launch_summaries_n5(const SummaryArgs &, cudaStream_t);
+cudaError_t launch_summaries_n6(const SummaryArgs &, cudaStream_t);
+cudaError_t launch_summaries_n7(const SummaryArgs &, cudaStream_t);
+cudaError_t launch_summaries_n8(const SummaryArgs &, cudaStream_t);
 cudaError_t launch_limit_n2(const LimitArgs &, cudaStream_t);
 cudaError_t launch_limit_n3(const LimitArgs &, cudaStream_t);
 cudaError_t launch_limit_n4(const LimitArgs &, cudaStream_t);
@@ -238,16 +238,16 @@ cudaError_t launch_stage_fp64(int n, int system, int flux, const StageArgs &a, l
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_summaries(int n, const SummaryArgs &a, long long E, cudaStream_t s)
+cudaError_t launch_summaries(int n, const SummaryArgs &a, cudaStream_t s)
 {
     switch (n) {
-    case 2: return launch_summaries_n2(a, E, s);
-    case 3: return launch_summaries_n3(a, E, s);
-    case 4: return launch_summaries_n4(a, E, s);
-    case 5: return launch_summaries_n5(a, E, s);
-    case 6: return launch_summaries_n6(a, E, s);
-    case 7: return launch_summaries_n7(a, E, s);
-    case 8: return launch_summaries_n8(a, E, s);
+    case 2: return launch_summaries_n2(a, s);
+    case 3: return launch_summaries_n3(a, s);
+    case 4: return launch_summaries_n4(a, s);
+    case 5: return launch_summaries_n5(a, s);
+    case 6: return launch_summaries_n6(a, s);
+    case 7: return launch_summaries_n7(a, s);
+    case 8: return launch_summaries_n8(a, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -556,12 +556,24 @@ LimitArgs limit_args(const dg_mesh *m, double *U, unsigned char *troubled)
     for (int ax = 0; ax < 3; ++ax) {
         l.K[ax] = m->d.K[ax];
         l.dx[ax] = m->dx[ax];
+        l.tvb[ax] = m->d.tvb_M * m->dx[ax] * m->dx[ax];
+        l.h[ax] = m->dx[ax] / m->d.beta;
+        for (int i = 0; i < m->d.n; ++i) l.hx[ax][i] = 0.5 * m->dx[ax] * m->T.x[i];
     }
     l.limiter = m->d.limiter;
-    l.tvb_M = m->d.tvb_M;
-    l.beta = m->d.beta;
-    l.T = m->T;
     return l;
+}
+
+SummaryArgs summary_args(const dg_mesh *m, const double *U, double *S)
+{
+    SummaryArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.U = U;
+    a.S = S;
+    a.unphys = (m->d.system == 1) ? m->unphys : nullptr;
+    a.E = m->E;
+    a.T = m->T;
+    return a;
 }
 
 dg_status check_mesh(const dg_mesh *m)
@@ -946,8 +958,6 @@ dg_status dg_rk3_step(dg_mesh *m, double *U, double dt, double cfl, double *dt_u
     a.mode = 1;
     a.dt = dt;
     a.dt_ptr = cflmode ? m->dt : nullptr;
-    a.S = lim ? m->S : nullptr;
-    a.unphys = (lim && sr) ? m->unphys : nullptr;
     if (cflmode) DG_CUDA(cudaMemsetAsync(m->lam, 0, sizeof(unsigned long long), s));
 
     double *ins[3] = {U, m->W1, m->W2};
@@ -968,6 +978,7 @@ dg_status dg_rk3_step(dg_mesh *m, double *U, double dt, double cfl, double *dt_u
         a.ca = ca[st];
         a.cb = cb[st];
         DG_LAUNCH(m, s, PROF_STAGE, launch_stage_fp64(m->d.n, m->d.system, m->d.flux, a, m->E, s));
+        if (lim) DG_LAUNCH(m, s, PROF_LIMIT, launch_summaries(m->d.n, summary_args(m, outs[st], m->S), s));
         if (lim && m->d.limiter == DG_LIMITER_MRS) {
             DG_LAUNCH(m, s, PROF_LIMIT, launch_mrs(m, outs[st], st == 2 ? troubled : nullptr, s));
         } else if (lim) {
@@ -1041,12 +1052,7 @@ dg_status dg_limiter_summaries(dg_mesh *m, const double *U, double *S, void *str
 {
     if (dg_status s = check_mesh(m)) return s;
     if (!U || !S) return fail(DG_ERR_ARG, "U and S must not be NULL");
-    SummaryArgs sa;
-    sa.U = U;
-    sa.S = S;
-    sa.unphys = (m->d.system == 1) ? m->unphys : nullptr;
-    sa.T = m->T;
-    DG_CUDA(launch_summaries(m->d.n, sa, m->E, (cudaStream_t)stream));
+    DG_CUDA(launch_summaries(m->d.n, summary_args(m, U, S), (cudaStream_t)stream));
     return DG_OK;
 }
 
@@ -1059,12 +1065,7 @@ dg_status dg_limit(dg_mesh *m, double *U, unsigned char *troubled, void *stream)
         if (troubled) DG_CUDA(cudaMemsetAsync(troubled, 0, (size_t)m->E, s));
         return DG_OK;
     }
-    SummaryArgs sa;
-    sa.U = U;
-    sa.S = m->S;
-    sa.unphys = (m->d.system == 1) ? m->unphys : nullptr;
-    sa.T = m->T;
-    DG_CUDA(launch_summaries(m->d.n, sa, m->E, s));
+    DG_CUDA(launch_summaries(m->d.n, summary_args(m, U, m->S), s));
     if (m->d.limiter == DG_LIMITER_MRS) {
         DG_CUDA(launch_mrs(m, U, troubled, s));
         return DG_OK;

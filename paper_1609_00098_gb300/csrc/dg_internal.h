@@ -8,6 +8,7 @@
 namespace dg {
 
 constexpr int MAXN = 8;  // largest LGL node count per axis
+constexpr int kNumSMs = 152;
 
 __host__ __device__ constexpr int round_up32(int v) { return (v + 31) / 32 * 32; }
 
@@ -71,15 +72,12 @@ struct Tables {
     double row1[MAXN];      // Legendre P1 coefficient of the nodal interpolant: c1 = sum_i row1[i] u_i
 };
 
-// Per-launch arguments of the fused stage kernel (RHS of eq:411 + SSP-RK3 stage
-// + limiter summaries).
+// Per-launch arguments of the fused stage kernel (RHS of eq:411 + SSP-RK3 stage).
 struct StageArgs {
     const double *Us;      // state the RHS is evaluated on
     const double *Un;      // U^n (stages 2 and 3)
     const double *P;       // primitives (vx, vy, vz, p) of Us, [e][4][node]
     double *out;           // U_{s+1} (mode 1) or dU/dt (mode 0)
-    double *S;             // limiter summaries [e][5][10] of out, or nullptr
-    unsigned char *unphys; // SR: per-element unphysical flag of out, or nullptr
     const double *dt_ptr;  // device dt (CFL mode) or nullptr
     double dt;             // host dt when dt_ptr == nullptr
     double ca, cb;         // out = ca Un + cb (Us + dt R); first stage: out = Us + dt R
@@ -102,15 +100,18 @@ struct LimitArgs {
     long long E;
     int K[3];
     int limiter;
-    double tvb_M, beta;
     double dx[3];
-    Tables T;
+    double tvb[3];          // M dx^2
+    double h[3];            // dx / beta
+    double hx[3][MAXN];     // (dx/2) x_i
 };
 
 struct SummaryArgs {
     const double *U;
     double *S;
     unsigned char *unphys;  // SR: per-element unphysical flag of U, or nullptr
+    long long E;
+    int G;                  // elements per CTA (set by the launcher)
     Tables T;
 };
 
@@ -165,7 +166,7 @@ namespace dg {
 
 // Kernel launchers (defined in the .cu files).
 cudaError_t launch_stage_fp64(int n, int system, int flux, const StageArgs &a, long long E, cudaStream_t s);
-cudaError_t launch_summaries(int n, const SummaryArgs &a, long long E, cudaStream_t s);
+cudaError_t launch_summaries(int n, const SummaryArgs &a, cudaStream_t s);
 cudaError_t launch_limit(int n, const LimitArgs &a, cudaStream_t s);
 
 cudaError_t launch_primitives(const dg_mesh *m, const double *U, double *P, int fix, double *Ufix,

@@ -1,0 +1,271 @@
+// dg_intfp64.cuh -- IEEE binary64 multiplication, division and square root, round to
+// nearest even, on the integer ALU.
+//
+// This GPU issues an FP64 instruction from a warp once every 64 cycles per SM
+// sub-partition (0.5e12 lane operations/s over the chip, measured), while its integer
+// ALU retires more than a warp instruction every other cycle.  An FP64 multiply costs
+// about 28 integer instructions here, a division about 65 and a square root about 60
+// (the compiler's FP64 division and square root are each a sequence of FP64
+// instructions), so kernels bound by the FP64 pipe run these operations on the integer
+// ALU, beside the additions that stay on the FP64 pipe.  Measured on a line contraction
+// s += D F of length 6 (multiply and add rounded separately): 0.25e12 pairs/s with both
+// on the FP64 pipe, 0.50e12 with the multiplies here, which is the rate of the FP64
+// additions alone.
+//
+// Results are the correctly rounded ones, the same bits as the FP64 unit's.  The fast
+// paths cover normal operands with normal results; everything else (zeros, subnormals,
+// infinities, NaN, results outside the normal range) takes the FP64 instruction.
+//
+// Methods, from the definitions: the multiply forms the exact 128-bit product of the
+// two significands.  The division is long division in three digits with a reciprocal
+// estimate from below, an exact remainder after every digit, and one final correction;
+// a quotient of two 53-bit significands is never half-way between two 53-bit values,
+// so floor(2^53 q) decides the rounding.  The square root refines an estimate from
+// the exact remainder v - s^2 and corrects the last bit against it; a root is never
+// half-way either.
+#pragma once
+
+#include <cstdint>
+#include <cstring>
+#if !defined(__CUDACC__)
+#include <cmath>
+#define __host__
+#define __device__
+#define __forceinline__ inline
+#endif
+
+namespace dg {
+namespace ifp {
+
+__host__ __device__ __forceinline__ uint64_t dbits(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (uint64_t)__double_as_longlong(x);
+#else
+    uint64_t b;
+    std::memcpy(&b, &x, 8);
+    return b;
+#endif
+}
+
+__host__ __device__ __forceinline__ double bdbl(uint64_t b)
+{
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)b);
+#else
+    double x;
+    std::memcpy(&x, &b, 8);
+    return x;
+#endif
+}
+
+__host__ __device__ __forceinline__ uint32_t hi32(uint64_t b) { return (uint32_t)(b >> 32); }
+__host__ __device__ __forceinline__ uint32_t lo32(uint64_t b) { return (uint32_t)b; }
+__host__ __device__ __forceinline__ uint64_t mk64(uint32_t h, uint32_t l) { return ((uint64_t)h << 32) | l; }
+__host__ __device__ __forceinline__ uint64_t mulw(uint32_t a, uint32_t b) { return (uint64_t)a * b; }
+
+// 1/x and 1/sqrt(x) in FP32 to about 2^-22 (any estimate within 2^-21.5 does)
+__host__ __device__ __forceinline__ float rcp_est(float x)
+{
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+#else
+    return 1.0f / x;
+#endif
+}
+
+__host__ __device__ __forceinline__ float rsqrt_est(float x)
+{
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+#else
+    return 1.0f / std::sqrt(x);
+#endif
+}
+
+__host__ __device__ __forceinline__ uint32_t fbits(float x)
+{
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(x);
+#else
+    uint32_t b;
+    std::memcpy(&b, &x, 4);
+    return b;
+#endif
+}
+
+__host__ __device__ __forceinline__ float bflt(uint32_t b)
+{
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(b);
+#else
+    float x;
+    std::memcpy(&x, &b, 4);
+    return x;
+#endif
+}
+
+__host__ __device__ __forceinline__ double native_mul(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    return __dmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+
+// ---------------------------------------------------------------------------
+// A factor prepared for products: the 53-bit significand shifted left by 11 (top bit
+// set; zero for a zero) in h:l, and in e the high word's sign and exponent fields.
+struct Factor {
+    uint32_t h, l, e;
+};
+
+__host__ __device__ __forceinline__ Factor factor(double x)
+{
+    const uint64_t b = dbits(x);
+    const uint32_t H = hi32(b), L = lo32(b);
+    Factor f;
+    f.h = (H << 11) | (L >> 21) | 0x80000000u;
+    f.l = L << 11;
+    f.e = H & 0xfff00000u;
+    if ((H & 0x7ff00000u) == 0u) f.h = f.l = 0u;  // zero (subnormals are excluded by factor_ok)
+    return f;
+}
+
+// Whether a factor is in the range the products below are exact for: zero, or an
+// exponent field in [E - span, E + span] around the bias (no product of two such
+// factors over- or underflows for span <= 500).
+__host__ __device__ __forceinline__ bool factor_ok(double x, uint32_t span = 500u)
+{
+    const uint64_t b = dbits(x);
+    const uint32_t ef = (hi32(b) >> 20) & 0x7ffu;
+    return ef - (1023u - span) <= 2u * span || (b << 1) == 0u;
+}
+
+// RN(f d) for two factors that factor_ok accepts.
+__host__ __device__ __forceinline__ double mul(const Factor &f, const Factor &d)
+{
+    const uint64_t p0 = mulw(f.l, d.l);
+    const uint64_t p1 = mulw(f.h, d.l) + hi32(p0);
+    const uint64_t p2 = mulw(f.l, d.h) + lo32(p1);
+    const uint64_t T = mulw(f.h, d.h) + hi32(p1) + hi32(p2);  // top 64 bits of the product
+    const uint32_t th = hi32(T);
+    const uint32_t n = th >> 31;  // 1: the product of the significands is >= 2
+    const uint64_t m = T >> (10 + n);
+    // the bits below the 53 kept, those of the lower 64 folded into the lowest one
+    // (the lowest bit is below the rounding position either way)
+    const uint32_t r = (lo32(T) & (n ? 0x7ffu : 0x3ffu)) | ((lo32(p2) | lo32(p0)) ? 1u : 0u);
+    const uint32_t up = r + (lo32(m) & 1u) > (n ? 0x400u : 0x200u) ? 1u : 0u;
+    // exponent field minus 1 (the significand's leading bit adds it back; a rounding
+    // carry into 2^53 raises the exponent by itself)
+    const uint32_t ex = (f.e & 0x7ff00000u) + (d.e & 0x7ff00000u) - (1024u << 20) + (n << 20);
+    uint64_t bits = mk64(ex, 0u) + m + up;
+    if (th == 0u) bits = 0u;
+    return bdbl(bits | mk64((f.e ^ d.e) & 0x80000000u, 0u));
+}
+
+// RN(a b).
+__host__ __device__ __forceinline__ double mul(double a, double b)
+{
+    if (factor_ok(a) & factor_ok(b)) return mul(factor(a), factor(b));
+    return native_mul(a, b);
+}
+
+// ---------------------------------------------------------------------------
+// RN(a / b): significands A, B in [2^52, 2^53); A doubled if below B, so that the
+// quotient is in [1, 2).  r = 2^84 / B from below, within 2^-20 relative.  Digits of 18,
+// 18 and 17 bits: q = floor-ish(rem 2^k / B), never above the true digit and below it
+// by less than 2, rem exact (modulo 2^64, always below 2^54).
+__host__ __device__ __forceinline__ double div(double a, double b)
+{
+    const uint64_t ab = dbits(a), bb = dbits(b);
+    const uint32_t ah = hi32(ab), bh = hi32(bb);
+    const uint32_t ea = (ah >> 20) & 0x7ffu, eb = (bh >> 20) & 0x7ffu;
+    // both in the middle of the exponent range: normal operands, normal quotient
+    if (((ea - 523u) <= 1000u) & ((eb - 523u) <= 1000u)) {
+        const uint32_t Bh = (bh & 0xfffffu) | 0x100000u, Bl = lo32(bb);
+        const uint64_t B = mk64(Bh, Bl);
+        uint64_t rem = mk64((ah & 0xfffffu) | 0x100000u, lo32(ab));
+        uint32_t ex = ea - eb + 1022u;  // exponent field minus 1
+        if (rem < B) {
+            rem <<= 1;
+            ex -= 1u;
+        }
+        // reciprocal of B's significand rounded up to FP32, y in [0.5, 1), as 2^32 y less
+        // 2^10 (more than the estimate's error): r <= 2^84 / B
+        const float y = rcp_est(bflt(0x3f800001u + ((Bh & 0xfffffu) << 3) + (Bl >> 29)));
+        const uint32_t r = (fbits(y) << 8) + 0x7ffffc00u;
+        const uint32_t nl = 0u - Bl, nh = ~Bh + (Bl == 0u ? 1u : 0u);  // -B
+        const uint32_t q1 = hi32(mulw((uint32_t)(rem >> 22), r)) >> 12;
+        rem <<= 18;
+        rem += mulw(q1, nl) + mk64(q1 * nh, 0u);
+        const uint32_t q2 = hi32(mulw((uint32_t)(rem >> 22), r)) >> 12;
+        rem <<= 18;
+        rem += mulw(q2, nl) + mk64(q2 * nh, 0u);
+        const uint32_t q3 = hi32(mulw((uint32_t)(rem >> 22), r)) >> 13;
+        rem <<= 17;
+        rem += mulw(q3, nl) + mk64(q3 * nh, 0u);
+        uint64_t Q = ((uint64_t)q1 << 35) + ((uint64_t)q2 << 17) + q3;  // floor(2^53 A/B), or one below
+        Q += rem >= B ? 2u : 1u;                                        // corrected, plus the rounding 1
+        return bdbl(mk64(ex << 20, 0u) + (Q >> 1) | mk64((ah ^ bh) & 0x80000000u, 0u));
+    }
+#ifdef __CUDA_ARCH__
+    return __ddiv_rn(a, b);
+#else
+    return a / b;
+#endif
+}
+
+// ---------------------------------------------------------------------------
+// RN(sqrt(x)): v = x scaled by an even power of two into [1, 4), V = 2^52 v.  With
+// y ~ 1/sqrt(v) (FP32): S1 = 2^24 sqrt(v) from y, the exact remainder V - S1^2 2^4
+// gives the next bits through y/2, twice; then floor(2^53 sqrt v) is fixed against the
+// exact remainder.
+__host__ __device__ __forceinline__ double root(double x)
+{
+    const uint64_t xb = dbits(x);
+    const uint32_t xh = hi32(xb);
+    if ((xh >> 20) - 1u <= 2045u) {  // positive and normal
+        const uint32_t ef = xh >> 20, odd = (ef & 1u) ^ 1u;  // odd power of two: v in [2, 4)
+        const uint64_t V = mk64((xh & 0xfffffu) | 0x100000u, lo32(xb)) << odd;  // 2^52 v
+        // FP32 copy of v (truncated) and 1/sqrt
+        const float vf = bflt(((127u + odd) << 23) + ((xh & 0xfffffu) << 3) + (lo32(xb) >> 29));
+        const float y = rsqrt_est(vf);                  // in (0.5, 1]
+        const float s = vf * y;                          // sqrt(v), in [1, 2), to 2^-21
+        const uint32_t yi = (uint32_t)(int32_t)(y * 1073741824.0f);  // 2^30 y
+        const uint32_t S1 = (uint32_t)(int32_t)(s * 16777216.0f);    // 2^24 sqrt(v) + d, |d| < 16
+        // remainder R1 = 2^48 v - S1^2, times 2^4 (V = 2^52 v): |R1 2^4| < 2^34
+        const int64_t R1 = (int64_t)V - (int64_t)(mulw(S1, S1) << 4);
+        // next 22 bits: R1 2^22 / (2 S1) = (R1 2^4) 2^18 / 2^25 / (S1 2^-24) = (R1 2^4) y 2^-7
+        const int32_t t1 = (int32_t)(R1 >> 3);                       // |t1| < 2^31
+        const int32_t d1 = (int32_t)(((int64_t)t1 * (int64_t)yi) >> 34);
+        const uint64_t S2 = ((uint64_t)S1 << 22) + (int64_t)d1;      // 2^46 sqrt(v), within 2^5
+        // remainder R2 = 2^92 v - S2^2 = V 2^40 - S2^2 (modulo 2^64; |R2| < 2^53)
+        const uint32_t s2h = hi32(S2), s2l = lo32(S2);
+        const uint64_t sq = mulw(s2l, s2l) + mk64(2u * s2h * s2l, 0u);  // S2^2 modulo 2^64
+        const int64_t R2 = (int64_t)((V << 40) - sq);
+        // next 7 bits: R2 2^7 / (2 S2) = R2 2^6 2^-46 y = (R2 2^-22) (2^30 y) 2^-48
+        const int32_t t2 = (int32_t)(R2 >> 22);
+        const int32_t d2 = (int32_t)(((int64_t)t2 * (int64_t)yi) >> 48);
+        uint64_t F = (S2 << 7) + (int64_t)d2;                        // 2^53 sqrt(v), within 1
+        // exact: 2^106 v - F^2 = V 2^54 - F^2 modulo 2^64 (|.| < 2^57)
+        const uint32_t fh = hi32(F), fl = lo32(F);
+        int64_t R = (int64_t)((V << 54) - (mulw(fl, fl) + mk64(2u * fh * fl, 0u)));
+        F += R < 0 ? 0u : (R > (int64_t)(2u * F) ? 2u : 1u);  // floor + 1 (the rounding)
+        const uint32_t ex = (ef - odd + 1023u) >> 1;
+        return bdbl(mk64((ex - 1u) << 20, 0u) + (F >> 1));
+    }
+#ifdef __CUDA_ARCH__
+    return __dsqrt_rn(x);
+#else
+    return std::sqrt(x);
+#endif
+}
+
+}  // namespace ifp
+}  // namespace dg

@@ -270,18 +270,45 @@ __device__ __forceinline__ unsigned sr_fix(double d_atm, double tau_atm, double 
     return ch;
 }
 
-// minmod of three slopes (eq:MinMod) and the TVB-bounded m_B (eq:MinModB).
-__device__ __forceinline__ double minmod3(double a1, double a2, double a3)
+// Sign tests, minmod (eq:MinMod) and magnitude comparisons of doubles done on
+// their bit patterns, on the integer ALU instead of the FP64 pipe (which bounds
+// the limiter kernels).  They decide exactly as the floating-point forms, NaN included:
+// - a double is > 0 iff its bits, read as a signed integer, lie in (0, +inf];
+// - it is < 0 iff its sign bit is set and its magnitude bits lie in (0, inf]
+//   (-0 is not negative);
+// - doubles of one sign are ordered like their bits, reversed for negatives, so
+//   among three positive or three negative doubles the one closest to 0 (the
+//   minmod pick) has the smallest bit pattern as a signed integer;
+// - |x| > c and |x| <= c for a finite c >= 0 compare the magnitude bits with c's.
+constexpr long long kMagBits = 0x7fffffffffffffffLL;
+constexpr long long kInfBits = 0x7ff0000000000000LL;
+
+__device__ __forceinline__ bool bits_pos(long long b) { return b > 0 && b <= kInfBits; }
+__device__ __forceinline__ bool bits_neg(long long b)
 {
-    if (a1 > 0.0 && a2 > 0.0 && a3 > 0.0) return fmin(a1, fmin(a2, a3));
-    if (a1 < 0.0 && a2 < 0.0 && a3 < 0.0) return fmax(a1, fmax(a2, a3));
-    return 0.0;
+    const long long m = b & kMagBits;
+    return b < 0 && m != 0 && m <= kInfBits;
 }
 
-__device__ __forceinline__ double minmodB(double a1, double a2, double a3, double M, double h)
+__device__ __forceinline__ double minmod3_bits(double a1, double a2, double a3)
 {
-    if (fabs(a1) <= M * h * h) return a1;
-    return minmod3(a1, a2, a3);
+    const long long b1 = __double_as_longlong(a1), b2 = __double_as_longlong(a2), b3 = __double_as_longlong(a3);
+    const bool pos = bits_pos(b1) & bits_pos(b2) & bits_pos(b3);
+    const bool neg = bits_neg(b1) & bits_neg(b2) & bits_neg(b3);
+    return (pos | neg) ? __longlong_as_double(min(b1, min(b2, b3))) : 0.0;
+}
+
+// |x| > c, for finite c >= 0
+__device__ __forceinline__ bool abs_gt(double x, double c)
+{
+    const long long m = __double_as_longlong(x) & kMagBits;
+    return m > __double_as_longlong(c) && m <= kInfBits;
+}
+
+// |x| <= c, for finite c >= 0
+__device__ __forceinline__ bool abs_le(double x, double c)
+{
+    return (__double_as_longlong(x) & kMagBits) <= __double_as_longlong(c);
 }
 
 }  // namespace dg

@@ -1,8 +1,8 @@
 // dg_stage_fp64.cuh -- FP64 element kernels of the DG stage (templated on the
 // number of LGL nodes per axis NP):
-//   k_stage_fp64  : volume term + lifted surface term of eq:411, the SSP-RK3
-//                   stage combination (Sec. 3.4) and the limiter summaries;
-//   k_summaries   : the limiter summaries alone;
+//   k_stage_fp64  : volume term + lifted surface term of eq:411 and the SSP-RK3
+//                   stage combination (Sec. 3.4);
+//   k_summaries   : the limiter summaries;
 //   k_limit       : the MinModN / MinMod decision and linear replacement (Sec. 3.3).
 // One CTA per element, one thread per node; the element's fluxes live in shared
 // memory for the three tensor-product contractions (eq:405).  This file is
@@ -12,60 +12,10 @@
 #pragma once
 
 #include "dg_internal.h"
+#include "dg_intfp64.cuh"
 #include "dg_physics.cuh"
 
 namespace dg {
-
-// Mean over the face nodes of axis `a` at index ia along a, weighted by the LGL
-// weights of the two other axes (divided by the reference face area 4).
-template <int NP>
-__device__ __forceinline__ double face_mean(const double *Uv, const double *sW, int a, int ia)
-{
-    const int b = (a + 1) % 3, c = (a + 2) % 3;
-    double s = 0.0;
-    for (int t1 = 0; t1 < NP; ++t1)
-        for (int t0 = 0; t0 < NP; ++t0) {
-            int id[3];
-            id[a] = ia;
-            id[b] = t0;
-            id[c] = t1;
-            s = s + sW[t0] * sW[t1] * Uv[id[0] + NP * (id[1] + NP * id[2])];
-        }
-    return s / 4.0;
-}
-
-// Limiter summaries of one element from its state in shared memory:
-// S[v][0] cell mean (LGL quadrature / 8), S[v][1+2a], S[v][2+2a] lower / upper
-// face means along a, S[v][7+a] Legendre P1 coefficient along a of the mean over
-// the other axes.  The block's threads produce the 50 entries, strided.
-template <int NP>
-__device__ __forceinline__ void element_summaries(const double *sU, const double *sW, const double *sRow1,
-                                                  double *Sout, int t)
-{
-    constexpr int NN = NP * NP * NP;
-    for (int id = t; id < 50; id += blockDim.x) {
-    const int v = id / 10, kind = id % 10;
-    const double *Uv = sU + v * NN;
-    double r;
-    if (kind == 0) {
-        double s = 0.0;
-        for (int k = 0; k < NP; ++k)
-            for (int j = 0; j < NP; ++j)
-                for (int i = 0; i < NP; ++i)
-                    s = s + sW[i] * sW[j] * sW[k] * Uv[i + NP * (j + NP * k)];
-        r = s / 8.0;
-    } else if (kind <= 6) {
-        const int a = (kind - 1) / 2;
-        r = face_mean<NP>(Uv, sW, a, ((kind - 1) % 2) ? NP - 1 : 0);
-    } else {
-        const int a = kind - 7;
-        double c1 = 0.0;
-        for (int ia = 0; ia < NP; ++ia) c1 = c1 + sRow1[ia] * face_mean<NP>(Uv, sW, a, ia);
-        r = c1;
-    }
-    Sout[v * 10 + kind] = r;
-    }
-}
 
 template <int NP, int SYS, int FLX>
 __global__ void __launch_bounds__(round_up32(NP *NP *NP)) k_stage_fp64(const StageArgs a)
@@ -75,16 +25,11 @@ __global__ void __launch_bounds__(round_up32(NP *NP *NP)) k_stage_fp64(const Sta
     double *sF = smem_stage;            // fluxes F^a_v per node [3][5][NN]; later the new state
     double *sR = smem_stage + 15 * NN;  // right-hand side per node [5][NN]
     __shared__ double sD[NP * NP];
-    __shared__ double sW[NP], sRow1[NP];
     __shared__ long long sNb[6];
 
     const int t = threadIdx.x;
     const long long e = blockIdx.x;
     for (int i = t; i < NP * NP; i += blockDim.x) sD[i] = a.T.D[i];
-    if (t < NP) {
-        sW[t] = a.T.w[t];
-        sRow1[t] = a.T.row1[t];
-    }
     if (t < 6) sNb[t] = SYS == 0 ? elem_neighbour_bc(e, a.K, t >> 1, (t & 1) ? 1 : -1, a.gh)
                                  : elem_neighbour(e, a.K, t >> 1, (t & 1) ? 1 : -1);
 
@@ -173,10 +118,8 @@ __global__ void __launch_bounds__(round_up32(NP *NP *NP)) k_stage_fp64(const Sta
     }
 
     // stage combination (or the bare RHS)
-    bool bad = false;
     if (t < NN) {
         const double dt = a.dt_ptr ? *a.dt_ptr : a.dt;
-        double un[5];
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
             const double R = sR[v * NN + t];
@@ -188,94 +131,183 @@ __global__ void __launch_bounds__(round_up32(NP *NP *NP)) k_stage_fp64(const Sta
                 val = a.first ? y : a.ca * a.Un[(e * 5 + v) * NN + t] + a.cb * y;
             }
             a.out[(e * 5 + v) * NN + t] = val;
-            sF[v * NN + t] = val;
-            un[v] = val;
         }
-        if (SYS == 1) bad = sr_unphysical(un);
     }
-    if (a.S == nullptr) return;
-    const int anybad = __syncthreads_or(bad);
-    element_summaries<NP>(sF, sW, sRow1, a.S + e * 50, t);
-    if (SYS == 1 && t == 0 && a.unphys) a.unphys[e] = anybad ? 1 : 0;
 }
+
+// w x for a quadrature weight w (prepared factor f of the double fd) and a state value x.
+__device__ __forceinline__ double weighted(const ifp::Factor &f, double fd, double x)
+{
+    return ifp::factor_ok(x) ? ifp::mul(ifp::factor(x), f) : fd * x;
+}
+
+// Limiter summaries S[e][v][10] of a.G consecutive elements per CTA: [0] the cell mean
+// (LGL quadrature / 8), [1+2a], [2+2a] the lower / upper face means along a, [7+a] the
+// Legendre P1 coefficient along a of the mean over the other axes.  Every sum runs
+// sequentially over its nodes in a fixed order, so the parallelism is over sums: warp
+// 0 takes the cell means (n^3 terms each, one lane per element and variable), the other
+// warps the 15 n plane means per element (n^2 terms each), of which the face means are
+// the first and last and the P1 coefficients the weighted sums.
+//
+// FP64-pipe bound.  The terms' products run on the integer ALU, and the weight products
+// are formed once per CTA.  Several elements share a CTA because a warp-wide FP64
+// instruction costs the same with 5 or 30 lanes active; one element per CTA, every
+// summary summing its own nodes, took two thirds of the FP64 stage's time.
+template <int NP>
+struct SumShape {
+    static constexpr int NN = NP * NP * NP;
+    static constexpr int G = NP <= 6 ? 6 : 3;  // most elements per CTA (5 G lanes of warp 0)
+    static constexpr int THREADS = 192;
+    // per element: U[5][NN] and plane means [15 NP]; per CTA: weight products
+    static constexpr size_t ELEM = sizeof(double) * (5 * NN + 15 * NP);
+    static constexpr size_t TAB = (sizeof(double) + sizeof(ifp::Factor)) * (NN + NP * NP) + 8;
+    __host__ __device__ static size_t smem(int g) { return ELEM * g + TAB; }
+};
 
 template <int NP>
-__global__ void __launch_bounds__(round_up32(NP *NP *NP)) k_summaries(const SummaryArgs a)
+__global__ void __launch_bounds__(SumShape<NP>::THREADS) k_summaries(const __grid_constant__ SummaryArgs a)
 {
-    constexpr int NN = NP * NP * NP;
-    __shared__ double sU[5 * NN];
-    __shared__ double sW[NP], sRow1[NP];
-    const int t = threadIdx.x;
-    const long long e = blockIdx.x;
-    if (t < NP) {
-        sW[t] = a.T.w[t];
-        sRow1[t] = a.T.row1[t];
+    constexpr int NN = NP * NP * NP, N2 = NP * NP;
+    extern __shared__ double smem_sum[];
+    const int G = a.G, t = threadIdx.x;
+    const long long e0 = (long long)blockIdx.x * G;
+    const int ne = a.E - e0 < G ? (int)(a.E - e0) : G;
+    double *sU = smem_sum;                 // [G][5][NN]
+    double *sQ = sU + (size_t)G * 5 * NN;  // [G][3 axes][NP][5]
+    double *sW3 = sQ + (size_t)G * 15 * NP, *sW2 = sW3 + NN;
+    ifp::Factor *sF3 = reinterpret_cast<ifp::Factor *>(sW2 + N2), *sF2 = sF3 + NN;
+    __shared__ double sMean[SumShape<NP>::G][5];
+    __shared__ int sBad[SumShape<NP>::G];
+
+    const double *Ug = a.U + e0 * 5 * NN;
+    for (int i = t; i < ne * 5 * NN; i += blockDim.x) sU[i] = Ug[i];
+    if (t < SumShape<NP>::G) sBad[t] = 0;
+    for (int q = t; q < NN; q += blockDim.x) {
+        const double w2 = a.T.w[q % NP] * a.T.w[(q / NP) % NP];
+        const double w3 = w2 * a.T.w[q / N2];
+        sW3[q] = w3;
+        sF3[q] = ifp::factor(w3);
+        if (q < N2) {
+            sW2[q] = w2;
+            sF2[q] = ifp::factor(w2);
+        }
     }
-    bool bad = false;
-    if (t < NN) {
-        double u[5];
-        for (int v = 0; v < 5; ++v) sU[v * NN + t] = u[v] = a.U[(e * 5 + v) * NN + t];
-        bad = sr_unphysical(u);
+    __syncthreads();
+
+    if (a.unphys)
+        for (int i = t; i < ne * NN; i += blockDim.x) {
+            const int el = i / NN;
+            const double *p = sU + (size_t)el * 5 * NN + (i - el * NN);
+            const double u[5] = {p[0], p[NN], p[2 * NN], p[3 * NN], p[4 * NN]};
+            if (sr_unphysical(u)) sBad[el] = 1;
+        }
+    if (t < 32) {
+        for (int r = t; r < ne * 5; r += 32) {
+            const double *Uv = sU + (size_t)r * NN;
+            double s = 0.0;
+            for (int q = 0; q < NN; ++q) s = s + weighted(sF3[q], sW3[q], Uv[q]);
+            sMean[r / 5][r % 5] = s * 0.125;
+        }
+    } else {
+        for (int r = t - 32; r < ne * 15 * NP; r += SumShape<NP>::THREADS - 32) {
+            const int v = r % 5, ia = (r / 5) % NP, ax = (r / (5 * NP)) % 3, el = r / (15 * NP);
+            // nodes with index ia along ax; t0 runs along the next axis, t1 along the one after
+            const int sa = ax == 0 ? 1 : ax == 1 ? NP : N2, sb = ax == 0 ? NP : ax == 1 ? N2 : 1;
+            const int sc = ax == 0 ? N2 : ax == 1 ? 1 : NP;
+            const double *Uv = sU + (size_t)(el * 5 + v) * NN + ia * sa;
+            double s = 0.0;
+            for (int t1 = 0; t1 < NP; ++t1)
+#pragma unroll
+                for (int t0 = 0; t0 < NP; ++t0)
+                    s = s + weighted(sF2[t0 + NP * t1], sW2[t0 + NP * t1], Uv[t0 * sb + t1 * sc]);
+            sQ[((el * 3 + ax) * NP + ia) * 5 + v] = s * 0.25;
+        }
     }
-    const int anybad = __syncthreads_or(bad);
-    element_summaries<NP>(sU, sW, sRow1, a.S + e * 50, t);
-    if (t == 0 && a.unphys) a.unphys[e] = anybad ? 1 : 0;
+    __syncthreads();
+    for (int r = t; r < ne * 50; r += blockDim.x) {
+        // kind-major: neighbouring lanes on one kind
+        const int el = r % ne, v = (r / ne) % 5, kind = r / (5 * ne);
+        double val;
+        if (kind == 0) {
+            val = sMean[el][v];
+        } else if (kind <= 6) {
+            const int ax = (kind - 1) / 2, ia = ((kind - 1) % 2) ? NP - 1 : 0;
+            val = sQ[((el * 3 + ax) * NP + ia) * 5 + v];
+        } else {
+            const double *Q = sQ + (el * 3 + kind - 7) * NP * 5 + v;
+            val = 0.0;
+#pragma unroll
+            for (int ia = 0; ia < NP; ++ia) val = val + ifp::mul(a.T.row1[ia], Q[ia * 5]);
+        }
+        a.S[(e0 + el) * 50 + v * 10 + kind] = val;
+    }
+    if (t < ne && a.unphys) a.unphys[e0 + t] = sBad[t] ? 1 : 0;
 }
 
-// One warp per element.  Lanes 0..4 decide for one conserved variable each:
-// MinModN tests the six face conditions of Sec. 3.3.2 (tolerance 1e-8, M = 0);
-// MinMod always limits; SR elements with an unphysical node limit every
+// Two elements per warp: lane 16 h + 3 v + ax decides variable v along axis ax of
+// element 2 w + h.  MinModN tests the six face conditions of Sec. 3.3.2 (tolerance
+// 1e-8, M = 0); MinMod always limits; SR elements with an unphysical node limit every
 // variable.  A limited variable becomes U0 + sum_a m_B(U_a, dU+/(dx/beta),
-// dU-/(dx/beta); M)(x_a - x_a0) (eq:MinModSol) at every node.
+// dU-/(dx/beta); M)(x_a - x_a0) (eq:MinModSol) at every node, the terms added one
+// after another.  The terms depend on one node index each and the first two partial
+// sums on two, so they are formed once per (variable, index) and (variable, plane
+// point): one FP64 addition per node is left of nine operations.
 template <int NP>
-__global__ void __launch_bounds__(256) k_limit(const LimitArgs a)
+__global__ void __launch_bounds__(128) k_limit(const __grid_constant__ LimitArgs a)
 {
-    constexpr int NN = NP * NP * NP;
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= a.E) return;
-    const long long e = warp;
+    constexpr int NN = NP * NP * NP, N2 = NP * NP;
+    __shared__ double sSl[4][32], sM0[4][32];  // per warp: slopes and means by lane
+    __shared__ double sP[4][15 * NP];          // [v][ax][i] slope terms
+    __shared__ double sAB[4][5 * N2];          // [v][j][i] mean + x term + y term
+    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5, half = lane >> 4, h = lane & 15;
+    const long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+    const bool live = e < a.E;
     int flag = 0;
-    double sl[3] = {0.0, 0.0, 0.0};
-    double U0 = 0.0;
-    if (lane < 5) {
-        const int v = lane;
+    double slope = 0.0, U0 = 0.0;
+    if (live && h < 15) {
+        const int v = h / 3, ax = h % 3;
         const double *Se = a.S + (e * 5 + v) * 10;
         U0 = Se[0];
+        const double dm = U0 - a.S[(elem_neighbour(e, a.K, ax, -1) * 5 + v) * 10];
+        const double dp = a.S[(elem_neighbour(e, a.K, ax, +1) * 5 + v) * 10] - U0;
         flag = (a.limiter == 2);
-        for (int ax = 0; ax < 3; ++ax) {
-            const double U0m = a.S[(elem_neighbour(e, a.K, ax, -1) * 5 + v) * 10];
-            const double U0p = a.S[(elem_neighbour(e, a.K, ax, +1) * 5 + v) * 10];
+        if (a.limiter == 1) {
             const double ulo = Se[1 + 2 * ax], uhi = Se[2 + 2 * ax];
-            if (a.limiter == 1) {
-                const double vl = U0 - minmodB(U0 - ulo, U0 - U0m, U0p - U0, 0.0, a.dx[ax]);
-                const double vr = U0 + minmodB(uhi - U0, U0 - U0m, U0p - U0, 0.0, a.dx[ax]);
-                if (fabs(vl - ulo) > 1e-8 || fabs(vr - uhi) > 1e-8) flag = 1;
-            }
-            const double h = a.dx[ax] / a.beta;
-            sl[ax] = minmodB(2.0 * Se[7 + ax] / a.dx[ax], (U0p - U0) / h, (U0 - U0m) / h, a.tvb_M, a.dx[ax]);
+            const double vl = U0 - minmod3_bits(U0 - ulo, dm, dp);
+            const double vr = U0 + minmod3_bits(uhi - U0, dm, dp);
+            if (abs_gt(vl - ulo, 1e-8) || abs_gt(vr - uhi, 1e-8)) flag = 1;
         }
+        const double s1 = ifp::div(2.0 * Se[7 + ax], a.dx[ax]);
+        slope = abs_le(s1, a.tvb[ax]) ? s1 : minmod3_bits(s1, ifp::div(dp, a.h[ax]), ifp::div(dm, a.h[ax]));
     }
-    unsigned mask = __ballot_sync(0xffffffffu, flag) & 0x1fu;
-    if (a.unphys && a.unphys[e]) mask = 0x1fu;
-    if (lane == 0 && a.troubled) a.troubled[e] = (unsigned char)mask;
-    if (!mask) return;
-    double hx[NP];
+    const unsigned fb = __ballot_sync(0xffffffffu, flag) >> (16 * half);
+    unsigned mask = 0;
 #pragma unroll
-    for (int i = 0; i < NP; ++i) hx[i] = a.T.x[i];
-    for (int v = 0; v < 5; ++v) {
-        const double m0 = __shfl_sync(0xffffffffu, U0, v);
-        const double s0 = __shfl_sync(0xffffffffu, sl[0], v);
-        const double s1 = __shfl_sync(0xffffffffu, sl[1], v);
-        const double s2 = __shfl_sync(0xffffffffu, sl[2], v);
-        if (!(mask & (1u << v))) continue;
-        for (int q = lane; q < NN; q += 32) {
-            const int i = q % NP, j = (q / NP) % NP, k = q / (NP * NP);
-            double val = m0;
-            val = val + s0 * (0.5 * a.dx[0] * hx[i]);
-            val = val + s1 * (0.5 * a.dx[1] * hx[j]);
-            val = val + s2 * (0.5 * a.dx[2] * hx[k]);
-            a.U[(e * 5 + v) * NN + q] = val;
+    for (int v = 0; v < 5; ++v)
+        if ((fb >> (3 * v)) & 7u) mask |= 1u << v;
+    if (live && a.unphys && a.unphys[e]) mask = 0x1fu;
+    if (live && h == 0 && a.troubled) a.troubled[e] = (unsigned char)mask;
+    sSl[wl][lane] = slope;
+    sM0[wl][lane] = U0;
+    for (int hh = 0; hh < 2; ++hh) {
+        const unsigned mk = __shfl_sync(0xffffffffu, mask, 16 * hh);
+        const long long eh = __shfl_sync(0xffffffffu, e, 16 * hh);
+        if (!mk) continue;
+        __syncwarp();
+        for (int r = lane; r < 15 * NP; r += 32) {
+            const int va = r / NP;  // 3 v + ax
+            sP[wl][r] = ifp::mul(sSl[wl][16 * hh + va], a.hx[va % 3][r % NP]);
+        }
+        __syncwarp();
+        for (int r = lane; r < 5 * N2; r += 32) {
+            const int v = r / N2, i = r % NP, j = (r / NP) % NP;
+            sAB[wl][r] = (sM0[wl][16 * hh + 3 * v] + sP[wl][(3 * v) * NP + i]) + sP[wl][(3 * v + 1) * NP + j];
+        }
+        __syncwarp();
+        for (int v = 0; v < 5; ++v) {
+            if (!(mk & (1u << v))) continue;
+            double *Uv = a.U + (eh * 5 + v) * NN;
+            for (int q = lane; q < NN; q += 32) Uv[q] = sAB[wl][v * N2 + q % N2] + sP[wl][(3 * v + 2) * NP + q / N2];
         }
     }
 }
@@ -301,17 +333,26 @@ cudaError_t launch_stage_np(int system, int flux, const StageArgs &a, long long 
 }
 
 template <int NP>
-cudaError_t launch_summaries_np(const SummaryArgs &a, long long E, cudaStream_t s)
+cudaError_t launch_summaries_np(const SummaryArgs &args, cudaStream_t s)
 {
-    k_summaries<NP><<<(unsigned)E, round_up32(NP * NP * NP), 0, s>>>(a);
+    SummaryArgs a = args;
+    // few elements: fewer per CTA, so that every SM gets some
+    const long long per = (a.E + kNumSMs - 1) / kNumSMs;
+    a.G = per < 1 ? 1 : per < SumShape<NP>::G ? (int)per : SumShape<NP>::G;
+    const size_t smem = SumShape<NP>::smem(a.G);
+    if (smem > 48 * 1024) {
+        const cudaError_t err =
+            cudaFuncSetAttribute(k_summaries<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (err != cudaSuccess) return err;
+    }
+    k_summaries<NP><<<(unsigned)((a.E + a.G - 1) / a.G), SumShape<NP>::THREADS, smem, s>>>(a);
     return cudaGetLastError();
 }
 
 template <int NP>
 cudaError_t launch_limit_np(const LimitArgs &a, cudaStream_t s)
 {
-    const long long threads = a.E * 32;
-    k_limit<NP><<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(a);
+    k_limit<NP><<<(unsigned)((a.E + 7) / 8), 128, 0, s>>>(a);  // 8 elements per CTA
     return cudaGetLastError();
 }
 
@@ -324,9 +365,9 @@ cudaError_t launch_limit_np(const LimitArgs &a, cudaStream_t s)
     {                                                                                                 \
         return launch_stage_np<NP>(system, flux, a, E, s);                                            \
     }                                                                                                 \
-    cudaError_t launch_summaries_n##NP(const SummaryArgs &a, long long E, cudaStream_t s)             \
+    cudaError_t launch_summaries_n##NP(const SummaryArgs &a, cudaStream_t s)                          \
     {                                                                                                 \
-        return launch_summaries_np<NP>(a, E, s);                                                      \
+        return launch_summaries_np<NP>(a, s);                                                         \
     }                                                                                                 \
     cudaError_t launch_limit_n##NP(const LimitArgs &a, cudaStream_t s) { return launch_limit_np<NP>(a, s); } \
     }

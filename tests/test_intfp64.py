@@ -1,0 +1,65 @@
+"""The integer-ALU binary64 operations (csrc/dg_intfp64.cuh), compiled for the host, against
+IEEE hardware: the same bits for products, quotients and square roots, special values included."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1609_00098_gb300", "csrc")
+SRC = """
+#include "dg_intfp64.cuh"
+using namespace dg::ifp;
+extern "C" void run(long n, const double *a, const double *b, double *m, double *d, double *r)
+{
+    for (long i = 0; i < n; ++i) {
+        m[i] = mul(a[i], b[i]);
+        d[i] = div(a[i], b[i]);
+        r[i] = root(a[i]);
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("intfp64")
+    src, so = str(d / "t.cpp"), str(d / "t.so")
+    with open(src, "w") as f:
+        f.write(SRC)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC, src, "-o", so],
+                   check=True)
+    return ctypes.CDLL(so)
+
+
+def _operands(kind):
+    r = np.random.RandomState(3)
+    n = 400000
+    bits = r.randint(0, 1 << 62, n, dtype=np.int64).astype(np.uint64) * np.uint64(4) + np.uint64(1)
+    mant = bits & np.uint64((1 << 52) - 1)
+    if kind == "sparse":      # significands with few bits at either end: exact results, carries, halves
+        k = r.randint(0, 52, n).astype(np.uint64)
+        mant = np.where(r.rand(n) < 0.5, mant >> k << k, mant | ((np.uint64(1) << k) - np.uint64(1)))
+    exp = r.randint(0, 2048, n) if kind == "any" else r.randint(960, 1087, n)
+    sign = r.randint(0, 2, n).astype(np.uint64) << np.uint64(63)
+    x = (sign | (exp.astype(np.uint64) << np.uint64(52)) | mant).view(np.float64)
+    if kind == "special":
+        sp = np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, 2.2250738585072014e-308, 1.7976931348623157e308,
+                       1.0, -1.0, 2.0, 0.5, 1.0 + 2.0 ** -52, 2.0 - 2.0 ** -52])
+        x = sp[r.randint(0, len(sp), n)]
+    return x
+
+
+@pytest.mark.parametrize("ka", ["near", "sparse", "any", "special"])
+@pytest.mark.parametrize("kb", ["near", "sparse", "any", "special"])
+def test_same_bits(lib, ka, kb):
+    a, b = _operands(ka), np.roll(_operands(kb), 7)
+    m, d, s = (np.empty_like(a) for _ in range(3))
+    p = [x.ctypes.data_as(ctypes.c_void_p) for x in (a, b, m, d, s)]
+    lib.run(ctypes.c_long(len(a)), *p)
+    with np.errstate(all="ignore"):
+        for got, ref in ((m, a * b), (d, a / b), (s, np.sqrt(a))):
+            nan = np.isnan(ref)
+            assert np.array_equal(np.isnan(got), nan)
+            assert np.array_equal(got[~nan].view(np.uint64), ref[~nan].view(np.uint64))
