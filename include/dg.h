@@ -221,14 +221,14 @@ dg_status dg_c2p_net_train(dg_c2p_net *net, long long count, const double *cons,
  * cannot call cudaMalloc -- device memory owned by another allocator, or loops that
  * cannot afford the device synchronisation of cudaMalloc/cudaFree).  Same kernels
  * and result as dg_rhs on a mesh made from `desc` (FP64 only), but the node
- * primitives live in a static device array of DG_RHS_STATIC_MAX_NODES nodes
- * (4 doubles each, 4 MiB, held by every GPU that loads the library until exit)
- * and nothing is allocated.  U and dUdt are caller-owned device arrays in state
+ * primitives and the face fluxes live in static device arrays for
+ * DG_RHS_STATIC_MAX_NODES nodes (4 and up to 7.5 doubles each, 11.5 MiB, held by
+ * every GPU that loads the library until exit) and nothing is allocated.  U and dUdt are caller-owned device arrays in state
  * layout.  DG_ERR_ARG if the mesh has more than DG_RHS_STATIC_MAX_NODES nodes or
- * the descriptor is invalid.  The first call on a device looks up the array's
- * device address; make that first call before any stream capture.  The array is
- * shared by all calls and keeps the last call's contents; calls that overlap on
- * the GPU race on it.  A node without a physical primitive state gives non-finite
+ * the descriptor is invalid.  The first call on a device looks up the arrays'
+ * device addresses; make that first call before any stream capture.  The arrays are
+ * shared by all calls and keep the last call's contents; calls that overlap on
+ * the GPU race on them.  A node without a physical primitive state gives non-finite
  * values in dUdt. */
 #define DG_RHS_STATIC_MAX_NODES 131072
 /* (periodic meshes only: DG_ERR_ARG for analytic boundaries) */

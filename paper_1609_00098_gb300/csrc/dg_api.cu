@@ -202,13 +202,13 @@ void lgl_tables(int n, Tables &T)
     for (int i = 0; i < n; ++i) T.row1[i] = M[1][n + i];
 }
 
-cudaError_t launch_stage_fp64_n2(int, int, const StageArgs &, long long, cudaStream_t);
-cudaError_t launch_stage_fp64_n3(int, int, const StageArgs &, long long, cudaStream_t);
-cudaError_t launch_stage_fp64_n4(int, int, const StageArgs &, long long, cudaStream_t);
-cudaError_t launch_stage_fp64_n5(int, int, const StageArgs &, long long, cudaStream_t);
-cudaError_t launch_stage_fp64_n6(int, int, const StageArgs &, long long, cudaStream_t);
-cudaError_t launch_stage_fp64_n7(int, int, const StageArgs &, long long, cudaStream_t);
-cudaError_t launch_stage_fp64_n8(int, int, const StageArgs &, long long, cudaStream_t);
+cudaError_t launch_stage_fp64_n2(const StageArgs &, cudaStream_t);
+cudaError_t launch_stage_fp64_n3(const StageArgs &, cudaStream_t);
+cudaError_t launch_stage_fp64_n4(const StageArgs &, cudaStream_t);
+cudaError_t launch_stage_fp64_n5(const StageArgs &, cudaStream_t);
+cudaError_t launch_stage_fp64_n6(const StageArgs &, cudaStream_t);
+cudaError_t launch_stage_fp64_n7(const StageArgs &, cudaStream_t);
+cudaError_t launch_stage_fp64_n8(const StageArgs &, cudaStream_t);
 cudaError_t launch_summaries_n2(const SummaryArgs &, cudaStream_t);
 cudaError_t launch_summaries_n3(const SummaryArgs &, cudaStream_t);
 cudaError_t launch_summaries_n4(const SummaryArgs &, cudaStream_t);
@@ -224,16 +224,16 @@ cudaError_t launch_limit_n6(const LimitArgs &, cudaStream_t);
 cudaError_t launch_limit_n7(const LimitArgs &, cudaStream_t);
 cudaError_t launch_limit_n8(const LimitArgs &, cudaStream_t);
 
-cudaError_t launch_stage_fp64(int n, int system, int flux, const StageArgs &a, long long E, cudaStream_t s)
+cudaError_t launch_stage_fp64(int n, const StageArgs &a, cudaStream_t s)
 {
     switch (n) {
-    case 2: return launch_stage_fp64_n2(system, flux, a, E, s);
-    case 3: return launch_stage_fp64_n3(system, flux, a, E, s);
-    case 4: return launch_stage_fp64_n4(system, flux, a, E, s);
-    case 5: return launch_stage_fp64_n5(system, flux, a, E, s);
-    case 6: return launch_stage_fp64_n6(system, flux, a, E, s);
-    case 7: return launch_stage_fp64_n7(system, flux, a, E, s);
-    case 8: return launch_stage_fp64_n8(system, flux, a, E, s);
+    case 2: return launch_stage_fp64_n2(a, s);
+    case 3: return launch_stage_fp64_n3(a, s);
+    case 4: return launch_stage_fp64_n4(a, s);
+    case 5: return launch_stage_fp64_n5(a, s);
+    case 6: return launch_stage_fp64_n6(a, s);
+    case 7: return launch_stage_fp64_n7(a, s);
+    case 8: return launch_stage_fp64_n8(a, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -538,10 +538,28 @@ StageArgs stage_args(const dg_mesh *m)
         a.lift0[ax] = a.g[ax] / m->T.w[0];
         a.liftN[ax] = a.g[ax] / m->T.w[m->d.n - 1];
     }
-    a.gamma = m->d.gamma;
+    a.E = m->E;
+    a.P = m->P;
+    a.Fs = m->Fs;
     a.gh = m->gh;
     a.T = m->T;
     return a;
+}
+
+FaceArgs face_args(const dg_mesh *m, const double *Us)
+{
+    FaceArgs f;
+    std::memset(&f, 0, sizeof(f));
+    f.Us = Us;
+    f.P = m->P;
+    f.Fs = m->Fs;
+    f.E = m->E;
+    f.nghost = m->nghost;
+    for (int ax = 0; ax < 3; ++ax) f.K[ax] = m->d.K[ax];
+    f.n = m->d.n;
+    f.gh = m->gh;
+    f.gamma = m->d.gamma;
+    return f;
 }
 
 LimitArgs limit_args(const dg_mesh *m, double *U, unsigned char *troubled)
@@ -608,6 +626,7 @@ void free_scratch(dg_mesh *m)
     cudaFree(m->pfull);
     for (int i = 0; i < 3; ++i) cudaFree(m->abL[i]);
     cudaFree(m->P);
+    cudaFree(m->Fs);
     cudaFree(m->S);
     cudaFree(m->mrsT);
     cudaFree(m->t);
@@ -709,6 +728,7 @@ dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out)
         if (st == cudaSuccess) st = cudaMemset(gU, 0, sizeof(double) * (size_t)m->nghost * 5 * m->nn);
         if (st == cudaSuccess) st = cudaMemset(gP, 0, sizeof(double) * (size_t)m->nghost * 4 * m->nn);
     }
+    if (!mixed) st = st ? st : cudaMalloc(&m->Fs, sizeof(double) * (size_t)(3 * E + m->nghost) * 5 * d->n * d->n);
     st = st ? st : cudaMalloc(&m->unphys, (size_t)E);
     st = st ? st : cudaMalloc(&m->lam, sizeof(unsigned long long));
     st = st ? st : cudaMalloc(&m->dt, sizeof(double));
@@ -806,10 +826,10 @@ dg_status dg_rhs(dg_mesh *m, const double *U, double *dUdt, void *stream)
     StageArgs a = stage_args(m);
     a.Us = U;
     a.Un = U;
-    a.P = m->P;
     a.out = dUdt;
     a.mode = 0;
-    DG_LAUNCH(m, s, PROF_STAGE, launch_stage_fp64(m->d.n, m->d.system, m->d.flux, a, m->E, s));
+    DG_LAUNCH(m, s, PROF_STAGE, launch_face_fp64(m->d.system, m->d.flux, face_args(m, U), s));
+    DG_LAUNCH(m, s, PROF_STAGE, launch_stage_fp64(m->d.n, a, s));
     return DG_OK;
 }
 
@@ -954,7 +974,6 @@ dg_status dg_rk3_step(dg_mesh *m, double *U, double dt, double cfl, double *dt_u
     const bool sr = m->d.system == 1;
     const bool lim = m->d.limiter != 0;
     StageArgs a = stage_args(m);
-    a.P = m->P;
     a.mode = 1;
     a.dt = dt;
     a.dt_ptr = cflmode ? m->dt : nullptr;
@@ -977,7 +996,8 @@ dg_status dg_rk3_step(dg_mesh *m, double *U, double dt, double cfl, double *dt_u
         a.first = st == 0;
         a.ca = ca[st];
         a.cb = cb[st];
-        DG_LAUNCH(m, s, PROF_STAGE, launch_stage_fp64(m->d.n, m->d.system, m->d.flux, a, m->E, s));
+        DG_LAUNCH(m, s, PROF_STAGE, launch_face_fp64(m->d.system, m->d.flux, face_args(m, ins[st]), s));
+        DG_LAUNCH(m, s, PROF_STAGE, launch_stage_fp64(m->d.n, a, s));
         if (lim) DG_LAUNCH(m, s, PROF_LIMIT, launch_summaries(m->d.n, summary_args(m, outs[st], m->S), s));
         if (lim && m->d.limiter == DG_LIMITER_MRS) {
             DG_LAUNCH(m, s, PROF_LIMIT, launch_mrs(m, outs[st], st == 2 ? troubled : nullptr, s));

@@ -77,6 +77,8 @@ struct StageArgs {
     const double *Us;      // state the RHS is evaluated on
     const double *Un;      // U^n (stages 2 and 3)
     const double *P;       // primitives (vx, vy, vz, p) of Us, [e][4][node]
+    const double *Fs;      // numerical fluxes of Us at the face points (FaceArgs)
+    long long E;
     double *out;           // U_{s+1} (mode 1) or dU/dt (mode 0)
     const double *dt_ptr;  // device dt (CFL mode) or nullptr
     double dt;             // host dt when dt_ptr == nullptr
@@ -85,11 +87,22 @@ struct StageArgs {
     int mode;              // 0 write RHS, 1 stage update
     int K[3];
     Ghosts gh;             // analytic boundaries (mask 0: periodic)
-    double gamma;
     double g[3];           // 2/dx_a
     double lift0[3];       // (2/dx_a)/w_0
     double liftN[3];       // (2/dx_a)/w_N
     Tables T;
+};
+
+// Numerical fluxes of the FP64 path, one evaluation per face point.
+struct FaceArgs {
+    const double *Us;
+    const double *P;
+    double *Fs;            // [3 E + nghost][5][n^2]: face a E + e below e along a, upper ghost faces after
+    long long E, nghost;
+    int K[3];
+    int n;
+    Ghosts gh;
+    double gamma;
 };
 
 struct LimitArgs {
@@ -128,6 +141,7 @@ struct dg_mesh {
     // library-owned device scratch
     double *W1, *W2;         // stage states
     double *P;               // primitives [e][4][node]
+    double *Fs;              // FP64 path: numerical fluxes at the face points [3 E + nghost][5][n^2]
     double *S;               // limiter summaries [e][5][10]
     unsigned char *unphys;   // per-element SR flags (bit 0: an unphysical node; mixed path bit 1: a node needs the fix)
     unsigned long long *lam; // max wave speed (bit pattern of a non-negative double)
@@ -165,7 +179,8 @@ struct dg_mesh {
 namespace dg {
 
 // Kernel launchers (defined in the .cu files).
-cudaError_t launch_stage_fp64(int n, int system, int flux, const StageArgs &a, long long E, cudaStream_t s);
+cudaError_t launch_face_fp64(int system, int flux, const FaceArgs &a, cudaStream_t s);
+cudaError_t launch_stage_fp64(int n, const StageArgs &a, cudaStream_t s);
 cudaError_t launch_summaries(int n, const SummaryArgs &a, cudaStream_t s);
 cudaError_t launch_limit(int n, const LimitArgs &a, cudaStream_t s);
 

@@ -27,8 +27,8 @@
 
 #include <cstdint>
 #include <cstring>
-#if !defined(__CUDACC__)
 #include <cmath>
+#if !defined(__CUDACC__)
 #define __host__
 #define __device__
 #define __forceinline__ inline
@@ -169,57 +169,84 @@ __host__ __device__ __forceinline__ double mul(const Factor &f, const Factor &d)
     return bdbl(bits | mk64((f.e ^ d.e) & 0x80000000u, 0u));
 }
 
-// RN(a b).
+// RN(a b).  (The fast result is formed first and replaced where an operand is out of
+// range: the factors of an operand used several times are then prepared once.)
 __host__ __device__ __forceinline__ double mul(double a, double b)
 {
-    if (factor_ok(a) & factor_ok(b)) return mul(factor(a), factor(b));
-    return native_mul(a, b);
+    double r = mul(factor(a), factor(b));
+    if (!(factor_ok(a) & factor_ok(b))) r = native_mul(a, b);
+    return r;
 }
 
 // ---------------------------------------------------------------------------
 // RN(a / b): significands A, B in [2^52, 2^53); A doubled if below B, so that the
 // quotient is in [1, 2).  r = 2^84 / B from below, within 2^-20 relative.  Digits of 18,
 // 18 and 17 bits: q = floor-ish(rem 2^k / B), never above the true digit and below it
-// by less than 2, rem exact (modulo 2^64, always below 2^54).
-__host__ __device__ __forceinline__ double div(double a, double b)
+// by less than 2, rem exact (modulo 2^64, always below 2^54).  Several quotients by one
+// divisor share its part.
+struct Divisor {
+    double b;
+    uint64_t B;
+    uint32_t nl, nh;  // -B
+    uint32_t r;
+    uint32_t h;       // high word of b
+};
+
+__host__ __device__ __forceinline__ Divisor divisor(double b)
 {
-    const uint64_t ab = dbits(a), bb = dbits(b);
-    const uint32_t ah = hi32(ab), bh = hi32(bb);
-    const uint32_t ea = (ah >> 20) & 0x7ffu, eb = (bh >> 20) & 0x7ffu;
-    // both in the middle of the exponent range: normal operands, normal quotient
-    if (((ea - 523u) <= 1000u) & ((eb - 523u) <= 1000u)) {
-        const uint32_t Bh = (bh & 0xfffffu) | 0x100000u, Bl = lo32(bb);
-        const uint64_t B = mk64(Bh, Bl);
-        uint64_t rem = mk64((ah & 0xfffffu) | 0x100000u, lo32(ab));
-        uint32_t ex = ea - eb + 1022u;  // exponent field minus 1
-        if (rem < B) {
-            rem <<= 1;
-            ex -= 1u;
-        }
-        // reciprocal of B's significand rounded up to FP32, y in [0.5, 1), as 2^32 y less
-        // 2^10 (more than the estimate's error): r <= 2^84 / B
-        const float y = rcp_est(bflt(0x3f800001u + ((Bh & 0xfffffu) << 3) + (Bl >> 29)));
-        const uint32_t r = (fbits(y) << 8) + 0x7ffffc00u;
-        const uint32_t nl = 0u - Bl, nh = ~Bh + (Bl == 0u ? 1u : 0u);  // -B
-        const uint32_t q1 = hi32(mulw((uint32_t)(rem >> 22), r)) >> 12;
-        rem <<= 18;
-        rem += mulw(q1, nl) + mk64(q1 * nh, 0u);
-        const uint32_t q2 = hi32(mulw((uint32_t)(rem >> 22), r)) >> 12;
-        rem <<= 18;
-        rem += mulw(q2, nl) + mk64(q2 * nh, 0u);
-        const uint32_t q3 = hi32(mulw((uint32_t)(rem >> 22), r)) >> 13;
-        rem <<= 17;
-        rem += mulw(q3, nl) + mk64(q3 * nh, 0u);
-        uint64_t Q = ((uint64_t)q1 << 35) + ((uint64_t)q2 << 17) + q3;  // floor(2^53 A/B), or one below
-        Q += rem >= B ? 2u : 1u;                                        // corrected, plus the rounding 1
-        return bdbl(mk64(ex << 20, 0u) + (Q >> 1) | mk64((ah ^ bh) & 0x80000000u, 0u));
-    }
-#ifdef __CUDA_ARCH__
-    return __ddiv_rn(a, b);
-#else
-    return a / b;
-#endif
+    Divisor d;
+    const uint64_t bb = dbits(b);
+    d.b = b;
+    d.h = hi32(bb);
+    const uint32_t Bh = (d.h & 0xfffffu) | 0x100000u, Bl = lo32(bb);
+    d.B = mk64(Bh, Bl);
+    // reciprocal of B's significand rounded up to FP32, y in [0.5, 1), as 2^32 y less
+    // 2^10 (more than the estimate's error): r <= 2^84 / B
+    const float y = rcp_est(bflt(0x3f800001u + ((Bh & 0xfffffu) << 3) + (Bl >> 29)));
+    d.r = (fbits(y) << 8) + 0x7ffffc00u;
+    d.nl = 0u - Bl;
+    d.nh = ~Bh + (Bl == 0u ? 1u : 0u);
+    return d;
 }
+
+__host__ __device__ __forceinline__ double div(double a, const Divisor &d)
+{
+    const uint64_t ab = dbits(a);
+    const uint32_t ah = hi32(ab);
+    const uint32_t ea = (ah >> 20) & 0x7ffu, eb = (d.h >> 20) & 0x7ffu;
+    const bool zero = (ab << 1) == 0u;
+    uint64_t rem = mk64((ah & 0xfffffu) | 0x100000u, lo32(ab));
+    uint32_t ex = ea - eb + 1022u;  // exponent field minus 1
+    if (rem < d.B) {
+        rem <<= 1;
+        ex -= 1u;
+    }
+    const uint32_t q1 = hi32(mulw((uint32_t)(rem >> 22), d.r)) >> 12;
+    rem <<= 18;
+    rem += mulw(q1, d.nl) + mk64(q1 * d.nh, 0u);
+    const uint32_t q2 = hi32(mulw((uint32_t)(rem >> 22), d.r)) >> 12;
+    rem <<= 18;
+    rem += mulw(q2, d.nl) + mk64(q2 * d.nh, 0u);
+    const uint32_t q3 = hi32(mulw((uint32_t)(rem >> 22), d.r)) >> 13;
+    rem <<= 17;
+    rem += mulw(q3, d.nl) + mk64(q3 * d.nh, 0u);
+    uint64_t Q = ((uint64_t)q1 << 35) + ((uint64_t)q2 << 17) + q3;  // floor(2^53 A/B), or one below
+    Q += rem >= d.B ? 2u : 1u;                                      // corrected, plus the rounding 1
+    uint64_t bits = mk64(ex << 20, 0u) + (Q >> 1);
+    if (zero) bits = 0u;
+    double r = bdbl(bits | mk64((ah ^ d.h) & 0x80000000u, 0u));
+    // both in the middle of the exponent range (normal operands, normal quotient), or 0 / b
+    if (!((((ea - 523u) <= 1000u) | zero) & ((eb - 523u) <= 1000u))) {
+#ifdef __CUDA_ARCH__
+        r = __ddiv_rn(a, d.b);
+#else
+        r = a / d.b;
+#endif
+    }
+    return r;
+}
+
+__host__ __device__ __forceinline__ double div(double a, double b) { return div(a, divisor(b)); }
 
 // ---------------------------------------------------------------------------
 // RN(sqrt(x)): v = x scaled by an even power of two into [1, 4), V = 2^52 v.  With
@@ -230,41 +257,70 @@ __host__ __device__ __forceinline__ double root(double x)
 {
     const uint64_t xb = dbits(x);
     const uint32_t xh = hi32(xb);
-    if ((xh >> 20) - 1u <= 2045u) {  // positive and normal
-        const uint32_t ef = xh >> 20, odd = (ef & 1u) ^ 1u;  // odd power of two: v in [2, 4)
-        const uint64_t V = mk64((xh & 0xfffffu) | 0x100000u, lo32(xb)) << odd;  // 2^52 v
-        // FP32 copy of v (truncated) and 1/sqrt
-        const float vf = bflt(((127u + odd) << 23) + ((xh & 0xfffffu) << 3) + (lo32(xb) >> 29));
-        const float y = rsqrt_est(vf);                  // in (0.5, 1]
-        const float s = vf * y;                          // sqrt(v), in [1, 2), to 2^-21
-        const uint32_t yi = (uint32_t)(int32_t)(y * 1073741824.0f);  // 2^30 y
-        const uint32_t S1 = (uint32_t)(int32_t)(s * 16777216.0f);    // 2^24 sqrt(v) + d, |d| < 16
-        // remainder R1 = 2^48 v - S1^2, times 2^4 (V = 2^52 v): |R1 2^4| < 2^34
-        const int64_t R1 = (int64_t)V - (int64_t)(mulw(S1, S1) << 4);
-        // next 22 bits: R1 2^22 / (2 S1) = (R1 2^4) 2^18 / 2^25 / (S1 2^-24) = (R1 2^4) y 2^-7
-        const int32_t t1 = (int32_t)(R1 >> 3);                       // |t1| < 2^31
-        const int32_t d1 = (int32_t)(((int64_t)t1 * (int64_t)yi) >> 34);
-        const uint64_t S2 = ((uint64_t)S1 << 22) + (int64_t)d1;      // 2^46 sqrt(v), within 2^5
-        // remainder R2 = 2^92 v - S2^2 = V 2^40 - S2^2 (modulo 2^64; |R2| < 2^53)
-        const uint32_t s2h = hi32(S2), s2l = lo32(S2);
-        const uint64_t sq = mulw(s2l, s2l) + mk64(2u * s2h * s2l, 0u);  // S2^2 modulo 2^64
-        const int64_t R2 = (int64_t)((V << 40) - sq);
-        // next 7 bits: R2 2^7 / (2 S2) = R2 2^6 2^-46 y = (R2 2^-22) (2^30 y) 2^-48
-        const int32_t t2 = (int32_t)(R2 >> 22);
-        const int32_t d2 = (int32_t)(((int64_t)t2 * (int64_t)yi) >> 48);
-        uint64_t F = (S2 << 7) + (int64_t)d2;                        // 2^53 sqrt(v), within 1
-        // exact: 2^106 v - F^2 = V 2^54 - F^2 modulo 2^64 (|.| < 2^57)
-        const uint32_t fh = hi32(F), fl = lo32(F);
-        int64_t R = (int64_t)((V << 54) - (mulw(fl, fl) + mk64(2u * fh * fl, 0u)));
-        F += R < 0 ? 0u : (R > (int64_t)(2u * F) ? 2u : 1u);  // floor + 1 (the rounding)
-        const uint32_t ex = (ef - odd + 1023u) >> 1;
-        return bdbl(mk64((ex - 1u) << 20, 0u) + (F >> 1));
-    }
+    const uint32_t ef = xh >> 20, odd = (ef & 1u) ^ 1u;  // odd power of two: v in [2, 4)
+    const uint64_t V = mk64((xh & 0xfffffu) | 0x100000u, lo32(xb)) << odd;  // 2^52 v
+    // FP32 copy of v (truncated) and 1/sqrt
+    const float vf = bflt(((127u + odd) << 23) + ((xh & 0xfffffu) << 3) + (lo32(xb) >> 29));
+    const float y = rsqrt_est(vf);                  // in (0.5, 1]
+    const float s = vf * y;                          // sqrt(v), in [1, 2), to 2^-21
+    const uint32_t yi = (uint32_t)(int32_t)(y * 1073741824.0f);  // 2^30 y
+    const uint32_t S1 = (uint32_t)(int32_t)(s * 16777216.0f);    // 2^24 sqrt(v) + d, |d| < 16
+    // remainder R1 = 2^48 v - S1^2, times 2^4 (V = 2^52 v): |R1 2^4| < 2^34
+    const int64_t R1 = (int64_t)V - (int64_t)(mulw(S1, S1) << 4);
+    // next 22 bits: R1 2^22 / (2 S1) = (R1 2^4) 2^18 / 2^25 / (S1 2^-24) = (R1 2^4) y 2^-7
+    const int32_t t1 = (int32_t)(R1 >> 3);                       // |t1| < 2^31
+    const int32_t d1 = (int32_t)(((int64_t)t1 * (int64_t)yi) >> 34);
+    const uint64_t S2 = ((uint64_t)S1 << 22) + (int64_t)d1;      // 2^46 sqrt(v), within 2^5
+    // remainder R2 = 2^92 v - S2^2 = V 2^40 - S2^2 (modulo 2^64; |R2| < 2^53)
+    const uint32_t s2h = hi32(S2), s2l = lo32(S2);
+    const uint64_t sq = mulw(s2l, s2l) + mk64(2u * s2h * s2l, 0u);  // S2^2 modulo 2^64
+    const int64_t R2 = (int64_t)((V << 40) - sq);
+    // next 7 bits: R2 2^7 / (2 S2) = R2 2^6 2^-46 y = (R2 2^-22) (2^30 y) 2^-48
+    const int32_t t2 = (int32_t)(R2 >> 22);
+    const int32_t d2 = (int32_t)(((int64_t)t2 * (int64_t)yi) >> 48);
+    uint64_t F = (S2 << 7) + (int64_t)d2;                        // 2^53 sqrt(v), within 1
+    // exact: 2^106 v - F^2 = V 2^54 - F^2 modulo 2^64 (|.| < 2^57)
+    const uint32_t fh = hi32(F), fl = lo32(F);
+    int64_t R = (int64_t)((V << 54) - (mulw(fl, fl) + mk64(2u * fh * fl, 0u)));
+    F += R < 0 ? 0u : (R > (int64_t)(2u * F) ? 2u : 1u);  // floor + 1 (the rounding)
+    const uint32_t ex = (ef - odd + 1023u) >> 1;
+    double r = bdbl(mk64((ex - 1u) << 20, 0u) + (F >> 1));
+    if (!((xh >> 20) - 1u <= 2045u)) {  // not positive and normal
 #ifdef __CUDA_ARCH__
-    return __dsqrt_rn(x);
+        r = __dsqrt_rn(x);
 #else
-    return std::sqrt(x);
+        r = std::sqrt(x);
 #endif
+    }
+    return r;
+}
+
+// ---------------------------------------------------------------------------
+// fmin / fmax by comparing the bit patterns (negatives ordered in reverse); a NaN
+// operand takes the FP64 instruction.
+__host__ __device__ __forceinline__ int64_t order_key(double x)
+{
+    const int64_t b = (int64_t)dbits(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+
+__host__ __device__ __forceinline__ bool maybe_nan(double x)
+{
+    return (hi32(dbits(x)) & 0x7fffffffu) >= 0x7ff00000u;
+}
+
+__host__ __device__ __forceinline__ double least(double a, double b)
+{
+    double r = order_key(a) < order_key(b) ? a : b;
+    if (maybe_nan(a) | maybe_nan(b)) r = fmin(a, b);
+    return r;
+}
+
+__host__ __device__ __forceinline__ double greatest(double a, double b)
+{
+    double r = order_key(a) > order_key(b) ? a : b;
+    if (maybe_nan(a) | maybe_nan(b)) r = fmax(a, b);
+    return r;
 }
 
 }  // namespace ifp

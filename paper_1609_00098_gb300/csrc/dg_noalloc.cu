@@ -6,8 +6,8 @@
 // memory, so a cudaMalloc would fail or fragment it), or time-critical loops
 // where the implicit device synchronisation of cudaMalloc / cudaFree is not
 // acceptable.  dg_rhs needs a dg_mesh, whose creation allocates the library's
-// scratch; this entry point instead keeps its one scratch buffer (the node
-// primitives) in a file-scope static device array of fixed size, takes the mesh
+// scratch; this entry point instead keeps its scratch (the node primitives and the
+// face fluxes) in file-scope static device arrays of fixed size, takes the mesh
 // descriptor directly, and allocates nothing.  The caller still owns U and dUdt.
 //
 // The array is global to the process on each device that loads the library and
@@ -24,13 +24,16 @@ constexpr long long kStaticMaxNodes = DG_RHS_STATIC_MAX_NODES;
 
 // Node primitives (vx, vy, vz, p), [e][4][node]; overwritten in full by each call.
 static __device__ __align__(256) double g_static_P[4 * kStaticMaxNodes];
+// Numerical fluxes at the face points, [3 E][5][n^2]: 15 / n doubles per node.
+static __device__ __align__(256) double g_static_F[15 * kStaticMaxNodes / 2];
 // Device status word of the primitive recovery; cleared at the start of each call.
 static __device__ __align__(256) unsigned int g_static_err;
 
-// Device addresses of the two arrays, looked up once per device with that device
+// Device addresses of the arrays, looked up once per device with that device
 // current (in host code the symbols are host-side stand-ins, not device addresses).
 struct StaticSlots {
     double *P = nullptr;
+    double *F = nullptr;
     unsigned int *err = nullptr;
     bool ready = false;
 };
@@ -45,6 +48,8 @@ dg_status static_slots(int dev, StaticSlots &out)
     StaticSlots &s = g_slots[dev];
     if (!s.ready) {
         cudaError_t e = cudaGetSymbolAddress((void **)&s.P, g_static_P);
+        if (e != cudaSuccess) return dg::set_error(DG_ERR_CUDA, cudaGetErrorString(e));
+        e = cudaGetSymbolAddress((void **)&s.F, g_static_F);
         if (e != cudaSuccess) return dg::set_error(DG_ERR_CUDA, cudaGetErrorString(e));
         e = cudaGetSymbolAddress((void **)&s.err, g_static_err);
         if (e != cudaSuccess) return dg::set_error(DG_ERR_CUDA, cudaGetErrorString(e));
@@ -97,24 +102,32 @@ extern "C" dg_status dg_rhs_static(const dg_mesh_desc *d, const double *U, doubl
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e = cudaMemsetAsync(slots.err, 0, sizeof(unsigned int), s);
     if (e == cudaSuccess) e = launch_primitives(&m, U, slots.P, 0, nullptr, nullptr, s);
-    if (e == cudaSuccess) {
-        StageArgs a;
-        std::memset(&a, 0, sizeof(a));
-        for (int ax = 0; ax < 3; ++ax) {
-            a.K[ax] = d->K[ax];
-            a.g[ax] = 2.0 / m.dx[ax];
-            a.lift0[ax] = a.g[ax] / m.T.w[0];
-            a.liftN[ax] = a.g[ax] / m.T.w[d->n - 1];
-        }
-        a.gamma = d->gamma;
-        a.T = m.T;
-        a.Us = U;
-        a.Un = U;
-        a.P = slots.P;
-        a.out = dUdt;
-        a.mode = 0;
-        e = launch_stage_fp64(d->n, d->system, d->flux, a, E, s);
+    FaceArgs f;
+    std::memset(&f, 0, sizeof(f));
+    f.Us = U;
+    f.P = slots.P;
+    f.Fs = slots.F;
+    f.E = E;
+    f.n = d->n;
+    f.gamma = d->gamma;
+    StageArgs a;
+    std::memset(&a, 0, sizeof(a));
+    for (int ax = 0; ax < 3; ++ax) {
+        f.K[ax] = a.K[ax] = d->K[ax];
+        a.g[ax] = 2.0 / m.dx[ax];
+        a.lift0[ax] = a.g[ax] / m.T.w[0];
+        a.liftN[ax] = a.g[ax] / m.T.w[d->n - 1];
     }
+    a.T = m.T;
+    a.Us = U;
+    a.Un = U;
+    a.P = slots.P;
+    a.Fs = slots.F;
+    a.E = E;
+    a.out = dUdt;
+    a.mode = 0;
+    if (e == cudaSuccess) e = launch_face_fp64(d->system, d->flux, f, s);
+    if (e == cudaSuccess) e = launch_stage_fp64(d->n, a, s);
     if (e != cudaSuccess) return set_error(DG_ERR_CUDA, cudaGetErrorString(e));
     return DG_OK;
 }

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "dg_intfp64.cuh"
+
 namespace dg {
 
 // Status bits of the per-mesh device status word.
@@ -15,11 +17,11 @@ enum : unsigned { ERRBIT_C2P = 1u, ERRBIT_UNPHYSICAL = 2u, ERRBIT_TIMEOUT = 4u }
 // Newtonian Euler: U = [rho, rho v_i, E], E = rho eps + rho v^2/2, p = (g-1) rho eps.
 __device__ __forceinline__ void ne_primitives(double g, const double u[5], double P[4])
 {
-    const double inv = 1.0 / u[0];
-    P[0] = u[1] * inv;
-    P[1] = u[2] * inv;
-    P[2] = u[3] * inv;
-    P[3] = (g - 1.0) * (u[4] - 0.5 * (u[1] * P[0] + u[2] * P[1] + u[3] * P[2]));
+    const double inv = ifp::div(1.0, u[0]);
+    P[0] = ifp::mul(u[1], inv);
+    P[1] = ifp::mul(u[2], inv);
+    P[2] = ifp::mul(u[3], inv);
+    P[3] = ifp::mul(g - 1.0, u[4] - 0.5 * (ifp::mul(u[1], P[0]) + ifp::mul(u[2], P[1]) + ifp::mul(u[3], P[2])));
 }
 
 // ---------------------------------------------------------------------------
@@ -123,17 +125,24 @@ __device__ __forceinline__ int node_primitives(double g, const double u[5], doub
 }
 
 // ---------------------------------------------------------------------------
+// The face kernel takes the axis at run time: components by selection (indexing a
+// register array with a runtime value would move it to local memory).
+__device__ __forceinline__ double pick_axis(int a, double x, double y, double z) { return a == 0 ? x : (a == 1 ? y : z); }
+
 // Physical flux along axis a, common to both systems with alpha = 1, beta = 0:
 // F = [U0 v_a, S_i v_a + p delta_ia, (U4 + p) v_a].
 __device__ __forceinline__ void flux_axis(const double u[5], const double P[4], int a, double F[5])
 {
-    const double va = P[a], p = P[3];
-    F[0] = u[0] * va;
-    F[1] = u[1] * va;
-    F[2] = u[2] * va;
-    F[3] = u[3] * va;
-    F[1 + a] = F[1 + a] + p;
-    F[4] = (u[4] + p) * va;
+    const double va = pick_axis(a, P[0], P[1], P[2]), p = P[3];
+    F[0] = ifp::mul(u[0], va);
+    F[1] = ifp::mul(u[1], va);
+    F[2] = ifp::mul(u[2], va);
+    F[3] = ifp::mul(u[3], va);
+    const double fn = pick_axis(a, F[1], F[2], F[3]) + p;
+    if (a == 0) F[1] = fn;
+    else if (a == 1) F[2] = fn;
+    else F[3] = fn;
+    F[4] = ifp::mul(u[4] + p, va);
 }
 
 // Extreme characteristic speeds along axis a (eq:CharDecomp).
@@ -141,27 +150,27 @@ template <int SYS>
 __device__ __forceinline__ void speeds_axis(double g, const double u[5], const double P[4], int a,
                                             double &lmin, double &lmax)
 {
-    const double va = P[a], p = P[3];
+    const double va = pick_axis(a, P[0], P[1], P[2]), p = P[3];
     if (SYS == 0) {
-        const double c = sqrt(g * p / u[0]);
+        const double c = ifp::root(ifp::div(ifp::mul(g, p), u[0]));
         lmin = va - c;
         lmax = va + c;
         return;
     }
-    const double v2 = P[0] * P[0] + P[1] * P[1] + P[2] * P[2];
-    const double rhoh = (u[4] + u[0] + p) * (1.0 - v2);
-    const double cs2 = g * p / rhoh;
-    const double cs = sqrt(cs2);
-    double disc = (1.0 - v2) * (1.0 - v2 * cs2 - va * va * (1.0 - cs2));
+    const double v2 = ifp::mul(P[0], P[0]) + ifp::mul(P[1], P[1]) + ifp::mul(P[2], P[2]);
+    const double w2i = 1.0 - v2;
+    const double cs2 = ifp::div(ifp::mul(g, p), ifp::mul(u[4] + u[0] + p, w2i));
+    const double om = 1.0 - cs2;
+    const double den = 1.0 - ifp::mul(v2, cs2);
+    double disc = ifp::mul(w2i, den - ifp::mul(ifp::mul(va, va), om));
     if (disc < 0.0) disc = 0.0;
-    const double root = cs * sqrt(disc);
-    const double den = 1.0 - v2 * cs2;
-    lmin = (va * (1.0 - cs2) - root) / den;
-    lmax = (va * (1.0 - cs2) + root) / den;
+    const double rt = ifp::mul(ifp::root(cs2), ifp::root(disc));
+    const double vo = ifp::mul(va, om);
+    const ifp::Divisor dd = ifp::divisor(den);
+    lmin = ifp::div(vo - rt, dd);
+    lmax = ifp::div(vo + rt, dd);
 }
 
-// Numerical flux along +e_a between the lower state L and the upper state R:
-// FLX = 0 local Lax-Friedrichs (eq:LLF), 1 HLL with Davis speeds (eq:HLL).
 // Roe dissipation D = sum_i alpha_i |lambda_i| e_i of eq:Roe for the Newtonian
 // ideal gas (Sec. 3.2.3): the flux Jacobian along e_a at the Roe averages
 // (eq:RoeAverages) of the velocity and of h = (E + p)/rho, eigenvalues u_n - c,
@@ -170,44 +179,51 @@ __device__ __forceinline__ void speeds_axis(double g, const double u[5], const d
 __device__ __forceinline__ void roe_dissipation(double g, int a, const double uL[5], const double PL[4],
                                                 const double uR[5], const double PR[4], double D[5])
 {
-    const double sl = sqrt(uL[0]), sr = sqrt(uR[0]);
-    const double wsum = sl + sr;
+    using ifp::mul;
+    const double sl = ifp::root(uL[0]), sr = ifp::root(uR[0]);
+    const ifp::Divisor wsum = ifp::divisor(sl + sr);
     double vh[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) vh[i] = (sl * PL[i] + sr * PR[i]) / wsum;
-    const double hL = (uL[4] + PL[3]) / uL[0], hR = (uR[4] + PR[3]) / uR[0];
-    const double hh = (sl * hL + sr * hR) / wsum;
-    const double q2 = vh[0] * vh[0] + vh[1] * vh[1] + vh[2] * vh[2];
-    const double c2 = (g - 1.0) * (hh - 0.5 * q2);
-    const double c = sqrt(c2);
-    const int b = (a + 1) % 3, d = (a + 2) % 3;
-    const double un = vh[a], ut1 = vh[b], ut2 = vh[d];
-    const double j1 = uR[0] - uL[0], jn = uR[1 + a] - uL[1 + a];
-    const double jt1 = uR[1 + b] - uL[1 + b], jt2 = uR[1 + d] - uL[1 + d], j5 = uR[4] - uL[4];
-    const double al3 = jt1 - ut1 * j1;
-    const double al4 = jt2 - ut2 * j1;
-    const double j5b = j5 - al3 * ut1 - al4 * ut2;
-    const double al2 = (g - 1.0) / c2 * (j1 * (hh - un * un) + un * jn - j5b);
-    const double al1 = (j1 * (un + c) - jn - c * al2) / (2.0 * c);
+    for (int i = 0; i < 3; ++i) vh[i] = ifp::div(mul(sl, PL[i]) + mul(sr, PR[i]), wsum);
+    const double hL = ifp::div(uL[4] + PL[3], uL[0]), hR = ifp::div(uR[4] + PR[3], uR[0]);
+    const double hh = ifp::div(mul(sl, hL) + mul(sr, hR), wsum);
+    const double q2 = mul(vh[0], vh[0]) + mul(vh[1], vh[1]) + mul(vh[2], vh[2]);
+    const double c2 = mul(g - 1.0, hh - 0.5 * q2);
+    const double c = ifp::root(c2);
+    const double un = pick_axis(a, vh[0], vh[1], vh[2]), ut1 = pick_axis(a, vh[1], vh[2], vh[0]);
+    const double ut2 = pick_axis(a, vh[2], vh[0], vh[1]);
+    const double jx = uR[1] - uL[1], jy = uR[2] - uL[2], jz = uR[3] - uL[3];
+    const double j1 = uR[0] - uL[0], jn = pick_axis(a, jx, jy, jz);
+    const double jt1 = pick_axis(a, jy, jz, jx), jt2 = pick_axis(a, jz, jx, jy), j5 = uR[4] - uL[4];
+    const double al3 = jt1 - mul(ut1, j1);
+    const double al4 = jt2 - mul(ut2, j1);
+    const double j5b = j5 - mul(al3, ut1) - mul(al4, ut2);
+    const double al2 = mul(ifp::div(g - 1.0, c2), mul(j1, hh - mul(un, un)) + mul(un, jn) - j5b);
+    const double al1 = ifp::div(mul(j1, un + c) - jn - mul(c, al2), 2.0 * c);
     const double al5 = j1 - (al1 + al2);
-    const double w1 = fabs(un - c) * al1, w2 = fabs(un) * al2, w5 = fabs(un + c) * al5;
-    const double w3 = fabs(un) * al3, w4 = fabs(un) * al4;
-    D[0] = w1 + w2 + w5;
-    D[1 + a] = w1 * (un - c) + w2 * un + w5 * (un + c);
-    D[1 + b] = (w1 + w2 + w5) * ut1 + w3;
-    D[1 + d] = (w1 + w2 + w5) * ut2 + w4;
-    D[4] = w1 * (hh - un * c) + w2 * (0.5 * q2) + w3 * ut1 + w4 * ut2 + w5 * (hh + un * c);
+    const double w1 = mul(fabs(un - c), al1), w2 = mul(fabs(un), al2), w5 = mul(fabs(un + c), al5);
+    const double w3 = mul(fabs(un), al3), w4 = mul(fabs(un), al4);
+    const double w = w1 + w2 + w5;
+    const double dn = mul(w1, un - c) + mul(w2, un) + mul(w5, un + c);
+    const double d1 = mul(w, ut1) + w3, d2 = mul(w, ut2) + w4;
+    D[0] = w;
+    D[1] = pick_axis(a, dn, d2, d1);
+    D[2] = pick_axis(a, d1, dn, d2);
+    D[3] = pick_axis(a, d2, d1, dn);
+    D[4] = mul(w1, hh - mul(un, c)) + mul(w2, 0.5 * q2) + mul(w3, ut1) + mul(w4, ut2) + mul(w5, hh + mul(un, c));
 }
 
+// Numerical flux along +e_a between the lower state L and the upper state R:
+// FLX = 0 local Lax-Friedrichs (eq:LLF), 1 HLL with Davis speeds (eq:HLL), 2 Roe
+// (eq:Roe, Newtonian).
 template <int SYS, int FLX>
 __device__ __forceinline__ void num_flux(double g, int a, const double uL[5], const double PL[4],
-                                         const double uR[5], const double PR[4], double Fs[5],
-                                         double FL[5], double FR[5])
+                                         const double uR[5], const double PR[4], double Fs[5])
 {
-    double lminL, lmaxL, lminR, lmaxR;
+    double FL[5], FR[5], lminL, lmaxL, lminR, lmaxR;
     flux_axis(uL, PL, a, FL);
     flux_axis(uR, PR, a, FR);
-    if (FLX == 2) {  // Roe (Newtonian only)
+    if (FLX == 2) {
         double D[5];
         roe_dissipation(g, a, uL, PL, uR, PR, D);
 #pragma unroll
@@ -217,17 +233,20 @@ __device__ __forceinline__ void num_flux(double g, int a, const double uL[5], co
     speeds_axis<SYS>(g, uL, PL, a, lminL, lmaxL);
     speeds_axis<SYS>(g, uR, PR, a, lminR, lmaxR);
     if (FLX == 0) {
-        const double al = fmax(fmax(fabs(lminL), fabs(lmaxL)), fmax(fabs(lminR), fabs(lmaxR)));
+        const double al = ifp::greatest(ifp::greatest(fabs(lminL), fabs(lmaxL)), ifp::greatest(fabs(lminR), fabs(lmaxR)));
+        const double hal = 0.5 * al;
 #pragma unroll
-        for (int v = 0; v < 5; ++v) Fs[v] = 0.5 * (FL[v] + FR[v]) - 0.5 * al * (uR[v] - uL[v]);
+        for (int v = 0; v < 5; ++v) Fs[v] = 0.5 * (FL[v] + FR[v]) - ifp::mul(hal, uR[v] - uL[v]);
     } else {
-        const double cmin = fmin(fmin(lminL, lminR), 0.0);
-        const double cmax = fmax(fmax(lmaxL, lmaxR), 0.0);
+        const double cmin = ifp::least(ifp::least(lminL, lminR), 0.0);
+        const double cmax = ifp::greatest(ifp::greatest(lmaxL, lmaxR), 0.0);
         const double den = cmax - cmin;
         if (den > 0.0) {
+            const ifp::Divisor dd = ifp::divisor(den);
+            const double cc = ifp::div(ifp::mul(cmin, cmax), dd);
 #pragma unroll
             for (int v = 0; v < 5; ++v)
-                Fs[v] = (cmax * FL[v] - cmin * FR[v]) / den + (cmin * cmax / den) * (uR[v] - uL[v]);
+                Fs[v] = ifp::div(ifp::mul(cmax, FL[v]) - ifp::mul(cmin, FR[v]), dd) + ifp::mul(cc, uR[v] - uL[v]);
         } else {
 #pragma unroll
             for (int v = 0; v < 5; ++v) Fs[v] = 0.5 * (FL[v] + FR[v]);
@@ -244,7 +263,7 @@ __device__ __forceinline__ double max_speed(double g, const double u[5], const d
     for (int a = 0; a < 3; ++a) {
         double lo, hi;
         speeds_axis<SYS>(g, u, P, a, lo, hi);
-        s = fmax(s, fmax(fabs(lo), fabs(hi)));
+        s = ifp::greatest(s, ifp::greatest(fabs(lo), fabs(hi)));
     }
     return s;
 }

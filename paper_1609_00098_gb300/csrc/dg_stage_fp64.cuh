@@ -17,7 +17,7 @@
 
 namespace dg {
 
-template <int NP, int SYS, int FLX>
+template <int NP>
 __global__ void __launch_bounds__(round_up32(NP *NP *NP)) k_stage_fp64(const StageArgs a)
 {
     constexpr int NN = NP * NP * NP;
@@ -30,8 +30,11 @@ __global__ void __launch_bounds__(round_up32(NP *NP *NP)) k_stage_fp64(const Sta
     const int t = threadIdx.x;
     const long long e = blockIdx.x;
     for (int i = t; i < NP * NP; i += blockDim.x) sD[i] = a.T.D[i];
-    if (t < 6) sNb[t] = SYS == 0 ? elem_neighbour_bc(e, a.K, t >> 1, (t & 1) ? 1 : -1, a.gh)
-                                 : elem_neighbour(e, a.K, t >> 1, (t & 1) ? 1 : -1);
+    // index of the face at side t & 1 of axis t >> 1 (dg_face_fp64.cu)
+    if (t < 6) {
+        const long long en = (t & 1) ? elem_neighbour_bc(e, a.K, t >> 1, 1, a.gh) : e;
+        sNb[t] = en >= 0 ? (t >> 1) * a.E + en : 3 * a.E + (-1 - en);
+    }
 
     double u[5], P[4];
     if (t < NN) {
@@ -82,36 +85,21 @@ __global__ void __launch_bounds__(round_up32(NP *NP *NP)) k_stage_fp64(const Sta
             id[(ax + 1) % 3] = rem % NP;
             id[(ax + 2) % 3] = rem / NP;
             const int q = id[0] + NP * (id[1] + NP * id[2]);
-            id[ax] = side ? 0 : NP - 1;
-            const int qn = id[0] + NP * (id[1] + NP * id[2]);
-            long long en = sNb[2 * ax + side];
-            // a negative neighbour is a ghost holding the analytic exterior state
-            const double *Ub = a.Us, *Pb = a.P;
-            if (SYS == 0 && en < 0) {
-                Ub = a.gh.U;
-                Pb = a.gh.P;
-                en = -1 - en;
-            }
-            double uo[5], Po[4], un[5], Pn[4];
+            const double *Fs = a.Fs + sNb[2 * ax + side] * 5 * NP * NP + rem;
+            double uo[5], Po[4], Fo[5];
 #pragma unroll
-            for (int v = 0; v < 5; ++v) {
-                uo[v] = a.Us[(e * 5 + v) * NN + q];
-                un[v] = Ub[(en * 5 + v) * NN + qn];
-            }
+            for (int v = 0; v < 5; ++v) uo[v] = a.Us[(e * 5 + v) * NN + q];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                Po[c] = a.P[(e * 4 + c) * NN + q];
-                Pn[c] = Pb[(en * 4 + c) * NN + qn];
-            }
-            double Fs[5], FL[5], FR[5];
+            for (int c = 0; c < 4; ++c) Po[c] = a.P[(e * 4 + c) * NN + q];
+            flux_axis(uo, Po, ax, Fo);
             if (side) {
-                num_flux<SYS, FLX>(a.gamma, ax, uo, Po, un, Pn, Fs, FL, FR);
 #pragma unroll
-                for (int v = 0; v < 5; ++v) sR[v * NN + q] = sR[v * NN + q] - a.liftN[ax] * (Fs[v] - FL[v]);
+                for (int v = 0; v < 5; ++v)
+                    sR[v * NN + q] = sR[v * NN + q] - a.liftN[ax] * (Fs[v * NP * NP] - Fo[v]);
             } else {
-                num_flux<SYS, FLX>(a.gamma, ax, un, Pn, uo, Po, Fs, FL, FR);
 #pragma unroll
-                for (int v = 0; v < 5; ++v) sR[v * NN + q] = sR[v * NN + q] + a.lift0[ax] * (Fs[v] - FR[v]);
+                for (int v = 0; v < 5; ++v)
+                    sR[v * NN + q] = sR[v * NN + q] + a.lift0[ax] * (Fs[v * NP * NP] - Fo[v]);
             }
         }
         __syncthreads();
@@ -314,21 +302,15 @@ __global__ void __launch_bounds__(128) k_limit(const __grid_constant__ LimitArgs
 
 // Dispatch helpers instantiated once per NP in dg_stage_fp64_n*.cu.
 template <int NP>
-cudaError_t launch_stage_np(int system, int flux, const StageArgs &a, long long E, cudaStream_t s)
+cudaError_t launch_stage_np(const StageArgs &a, cudaStream_t s)
 {
-    const dim3 grid((unsigned)E), block(round_up32(NP * NP * NP));
+    const dim3 grid((unsigned)a.E), block(round_up32(NP * NP * NP));
     const size_t smem = sizeof(double) * 20 * NP * NP * NP;
-    void (*kern)(const StageArgs);
-    if (system == 0 && flux == 2) kern = k_stage_fp64<NP, 0, 2>;
-    else if (system == 0 && flux == 0) kern = k_stage_fp64<NP, 0, 0>;
-    else if (system == 0) kern = k_stage_fp64<NP, 0, 1>;
-    else if (flux == 0) kern = k_stage_fp64<NP, 1, 0>;
-    else kern = k_stage_fp64<NP, 1, 1>;
     if (smem > 48 * 1024) {
-        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t err = cudaFuncSetAttribute(k_stage_fp64<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (err != cudaSuccess) return err;
     }
-    kern<<<grid, block, smem, s>>>(a);
+    k_stage_fp64<NP><<<grid, block, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -360,10 +342,9 @@ cudaError_t launch_limit_np(const LimitArgs &a, cudaStream_t s)
 
 #define DG_INSTANTIATE_STAGE(NP)                                                                      \
     namespace dg {                                                                                    \
-    cudaError_t launch_stage_fp64_n##NP(int system, int flux, const StageArgs &a, long long E,         \
-                                        cudaStream_t s)                                               \
+    cudaError_t launch_stage_fp64_n##NP(const StageArgs &a, cudaStream_t s)                            \
     {                                                                                                 \
-        return launch_stage_np<NP>(system, flux, a, E, s);                                            \
+        return launch_stage_np<NP>(a, s);                                                             \
     }                                                                                                 \
     cudaError_t launch_summaries_n##NP(const SummaryArgs &a, cudaStream_t s)                          \
     {                                                                                                 \
