@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/dg.h"
+#include "dg_intfp64.cuh"
 
 namespace dg {
 
@@ -91,6 +92,7 @@ struct StageArgs {
     double lift0[3];       // (2/dx_a)/w_0
     double liftN[3];       // (2/dx_a)/w_N
     Tables T;
+    ifp::Factor DF[MAXN * MAXN];  // entries of D prepared for products (set by the launcher)
 };
 
 // Numerical fluxes of the FP64 path, one evaluation per face point.

@@ -4,10 +4,8 @@
 //                   stage combination (Sec. 3.4);
 //   k_summaries   : the limiter summaries;
 //   k_limit       : the MinModN / MinMod decision and linear replacement (Sec. 3.3).
-// One CTA per element, one thread per node; the element's fluxes live in shared
-// memory for the three tensor-product contractions (eq:405).  This file is
-// compiled without floating-point contraction and every sum runs in a fixed
-// order, so that the FP64 path reproduces a plain sequential evaluation of the
+// This file is compiled without floating-point contraction and every sum runs in a
+// fixed order, so that the FP64 path reproduces a plain sequential evaluation of the
 // same formulas operation for operation.
 #pragma once
 
@@ -17,108 +15,145 @@
 
 namespace dg {
 
+// Launch shape of k_stage_fp64: elements per CTA and threads, so that the 15 n^2 lines
+// of an element (the longest phase) fill the threads in whole rounds.
 template <int NP>
-__global__ void __launch_bounds__(round_up32(NP *NP *NP)) k_stage_fp64(const StageArgs a)
+struct StageShape64 {
+    static constexpr int NN = NP * NP * NP, N2 = NP * NP;
+    static constexpr int EPB = NP == 2 ? 4 : NP == 3 ? 2 : 1;
+    static constexpr int THREADS = NP == 2 || NP == 4 ? 256 : NP == 3 || NP == 6 ? 288 : NP == 8 ? 512 : 384;
+    static constexpr size_t SMEM = sizeof(double) * (15 * NN + 30 * N2) * EPB;
+};
+
+// One stage for EPB elements per CTA, in four phases:
+//   nodes   the fluxes F^a_v of the element (eq:411) into shared memory;
+//   faces   the stored numerical flux minus the element's own, times the lift factor,
+//           per face point and variable;
+//   lines   one thread per (axis, variable, line of n nodes): the n products and sums
+//           of eq:405 for the line's n nodes, in place;
+//   nodes   the three axes' sums combined, the lifts added (x, y, z in turn), and the
+//           stage update.
+// Every sum keeps the order of a sequential evaluation node by node (products and sums
+// rounded separately), so the results are its bits.
+//
+// FP64-pipe bound: the products run on the integer ALU, with the entries of D prepared
+// by the host and each line's flux values prepared once for n products, which leaves
+// the FP64 pipe n - 1 additions per node, axis and variable.  With products and sums
+// both on it and one thread per node, the contraction ran at half the rate (0.25e12
+// against 0.50e12 product-sum pairs/s).  Lines also give 15 n^2 threads' work where
+// nodes give n^3, which is what a mesh with fewer elements than SMs needs.
+template <int NP>
+__global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const __grid_constant__ StageArgs a)
 {
-    constexpr int NN = NP * NP * NP;
+    using SH = StageShape64<NP>;
+    constexpr int NN = SH::NN, N2 = SH::N2, EPB = SH::EPB;
     extern __shared__ double smem_stage[];
-    double *sF = smem_stage;            // fluxes F^a_v per node [3][5][NN]; later the new state
-    double *sR = smem_stage + 15 * NN;  // right-hand side per node [5][NN]
-    __shared__ double sD[NP * NP];
-    __shared__ long long sNb[6];
+    double *sF = smem_stage;                 // [EPB][3][5][NN] fluxes, then the lines' sums
+    double *sL = smem_stage + EPB * 15 * NN;  // [EPB][6][5][N2] lifted face terms
+    __shared__ long long sFace[EPB][6];       // index of the face at side s of axis a (2 a + s)
 
     const int t = threadIdx.x;
-    const long long e = blockIdx.x;
-    for (int i = t; i < NP * NP; i += blockDim.x) sD[i] = a.T.D[i];
-    // index of the face at side t & 1 of axis t >> 1 (dg_face_fp64.cu)
-    if (t < 6) {
-        const long long en = (t & 1) ? elem_neighbour_bc(e, a.K, t >> 1, 1, a.gh) : e;
-        sNb[t] = en >= 0 ? (t >> 1) * a.E + en : 3 * a.E + (-1 - en);
+    const long long e0 = (long long)blockIdx.x * EPB;
+    const int ne = EPB == 1 ? 1 : a.E - e0 < EPB ? (int)(a.E - e0) : EPB;
+    if (t < 6 * ne) {
+        const int ax = (t % 6) >> 1;
+        const long long e = e0 + t / 6;
+        const long long en = (t & 1) ? elem_neighbour_bc(e, a.K, ax, 1, a.gh) : e;
+        sFace[t / 6][t % 6] = en >= 0 ? ax * a.E + en : 3 * a.E + (-1 - en);
     }
-
-    double u[5], P[4];
-    if (t < NN) {
+    for (int r = t; r < ne * NN; r += SH::THREADS) {
+        const int el = EPB == 1 ? 0 : r / NN, q = r - el * NN;
+        double u[5], P[4];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) u[v] = a.Us[(e * 5 + v) * NN + t];
+        for (int v = 0; v < 5; ++v) u[v] = a.Us[((e0 + el) * 5 + v) * NN + q];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) P[c] = a.P[(e * 4 + c) * NN + t];
+        for (int c = 0; c < 4; ++c) P[c] = a.P[((e0 + el) * 4 + c) * NN + q];
 #pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
             double f[5];
             flux_axis(u, P, ax, f);
 #pragma unroll
-            for (int v = 0; v < 5; ++v) sF[(ax * 5 + v) * NN + t] = f[v];
+            for (int v = 0; v < 5; ++v) sF[(el * 15 + ax * 5 + v) * NN + q] = f[v];
         }
     }
     __syncthreads();
 
-    // volume term: -sum_a (2/dx_a) sum_l D_{i_a l} F^a_l
-    if (t < NN) {
-        const int i = t % NP, j = (t / NP) % NP, k = t / (NP * NP);
+    // lifted face terms: (2/dx_a)(F* - F)/w at the face's end of the axis
+    for (int r = t; r < ne * 30 * N2; r += SH::THREADS) {
+        const int el = EPB == 1 ? 0 : r / (30 * N2), rr = r - el * 30 * N2;
+        const int as = rr / (5 * N2), vr = rr - as * 5 * N2, v = vr / N2, p = vr - v * N2;
+        const int ax = as >> 1;
+        const int sa = ax == 0 ? 1 : ax == 1 ? NP : N2, sb = ax == 0 ? NP : ax == 1 ? N2 : 1;
+        const int sc = ax == 0 ? N2 : ax == 1 ? 1 : NP;
+        const int q = ((as & 1) ? NP - 1 : 0) * sa + (p % NP) * sb + (p / NP) * sc;
+        const double lift = (as & 1) ? (ax == 0 ? a.liftN[0] : ax == 1 ? a.liftN[1] : a.liftN[2])
+                                     : (ax == 0 ? a.lift0[0] : ax == 1 ? a.lift0[1] : a.lift0[2]);
+        sL[r] = ifp::mul(lift, a.Fs[sFace[el][as] * 5 * N2 + vr] - sF[(el * 15 + ax * 5 + v) * NN + q]);
+    }
+    __syncthreads();
+
+    // volume term: sum_l D_il F_l along every line, in place
+    for (int r = t; r < ne * 15 * N2; r += SH::THREADS) {
+        const int av = r / N2, c = r - av * N2;  // av = (el, axis, variable)
+        const int ax = (av % 15) / 5;
+        const int st = ax == 0 ? 1 : ax == 1 ? NP : N2;
+        double *F = sF + av * NN + (ax == 0 ? NP * c : ax == 1 ? c % NP + N2 * (c / NP) : c);
+        double f[NP], s[NP];
+        bool ok = true;
 #pragma unroll
-        for (int v = 0; v < 5; ++v) {
-            const double *Fx = sF + (0 * 5 + v) * NN;
-            const double *Fy = sF + (1 * 5 + v) * NN;
-            const double *Fz = sF + (2 * 5 + v) * NN;
-            double sx = 0.0, sy = 0.0, sz = 0.0;
+        for (int l = 0; l < NP; ++l) {
+            f[l] = F[l * st];
+            ok &= ifp::factor_ok(f[l]);
+        }
+        if (ok) {
 #pragma unroll
             for (int l = 0; l < NP; ++l) {
-                sx = sx + sD[i * NP + l] * Fx[l + NP * (j + NP * k)];
-                sy = sy + sD[j * NP + l] * Fy[i + NP * (l + NP * k)];
-                sz = sz + sD[k * NP + l] * Fz[i + NP * (j + NP * l)];
+                const ifp::Factor fl = ifp::factor(f[l]);
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                    const double p = ifp::mul(fl, a.DF[i * NP + l]);
+                    s[i] = l == 0 ? p : s[i] + p;
+                }
             }
-            double acc = a.g[0] * sx;
-            acc = acc + a.g[1] * sy;
-            acc = acc + a.g[2] * sz;
-            sR[v * NN + t] = -acc;
+        } else {  // values out of the products' range, infinities, NaN
+#pragma unroll
+            for (int l = 0; l < NP; ++l)
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                    const double p = a.T.D[i * NP + l] * f[l];
+                    s[i] = l == 0 ? p : s[i] + p;
+                }
         }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) F[i * st] = s[i];
     }
     __syncthreads();
 
-    // surface terms, one axis after another (within an axis no node is hit twice)
-    for (int ax = 0; ax < 3; ++ax) {
-        for (int fp = t; fp < 2 * NP * NP; fp += blockDim.x) {
-            const int side = fp / (NP * NP);
-            const int rem = fp % (NP * NP);
-            int id[3];
-            id[ax] = side ? NP - 1 : 0;
-            id[(ax + 1) % 3] = rem % NP;
-            id[(ax + 2) % 3] = rem / NP;
-            const int q = id[0] + NP * (id[1] + NP * id[2]);
-            const double *Fs = a.Fs + sNb[2 * ax + side] * 5 * NP * NP + rem;
-            double uo[5], Po[4], Fo[5];
-#pragma unroll
-            for (int v = 0; v < 5; ++v) uo[v] = a.Us[(e * 5 + v) * NN + q];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) Po[c] = a.P[(e * 4 + c) * NN + q];
-            flux_axis(uo, Po, ax, Fo);
-            if (side) {
-#pragma unroll
-                for (int v = 0; v < 5; ++v)
-                    sR[v * NN + q] = sR[v * NN + q] - a.liftN[ax] * (Fs[v * NP * NP] - Fo[v]);
-            } else {
-#pragma unroll
-                for (int v = 0; v < 5; ++v)
-                    sR[v * NN + q] = sR[v * NN + q] + a.lift0[ax] * (Fs[v * NP * NP] - Fo[v]);
-            }
-        }
-        __syncthreads();
-    }
-
-    // stage combination (or the bare RHS)
-    if (t < NN) {
-        const double dt = a.dt_ptr ? *a.dt_ptr : a.dt;
+    const double dt = a.dt_ptr ? *a.dt_ptr : a.dt;
+    for (int r = t; r < ne * NN; r += SH::THREADS) {
+        const int el = EPB == 1 ? 0 : r / NN, q = r - el * NN;
+        const int i = q % NP, j = (q / NP) % NP, k = q / N2;
+        const double *Fe = sF + el * 15 * NN + q, *Le = sL + el * 30 * N2;
+        // offset of the node's lifted terms on each axis, if it lies on a face
+        const bool fx = i == 0 || i == NP - 1, fy = j == 0 || j == NP - 1, fz = k == 0 || k == NP - 1;
+        const int ox = (i == 0 ? 0 : 5 * N2) + j + NP * k, oy = (j == 0 ? 10 * N2 : 15 * N2) + k + NP * i;
+        const int oz = (k == 0 ? 20 * N2 : 25 * N2) + i + NP * j;
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
-            const double R = sR[v * NN + t];
-            double val;
-            if (a.mode == 0) {
-                val = R;
-            } else {
-                const double y = u[v] + dt * R;
-                val = a.first ? y : a.ca * a.Un[(e * 5 + v) * NN + t] + a.cb * y;
+            double acc = ifp::mul(a.g[0], Fe[v * NN]);
+            acc = acc + ifp::mul(a.g[1], Fe[(5 + v) * NN]);
+            acc = acc + ifp::mul(a.g[2], Fe[(10 + v) * NN]);
+            double R = -acc;
+            if (fx) R = R + (i == 0 ? Le[ox + v * N2] : -Le[ox + v * N2]);
+            if (fy) R = R + (j == 0 ? Le[oy + v * N2] : -Le[oy + v * N2]);
+            if (fz) R = R + (k == 0 ? Le[oz + v * N2] : -Le[oz + v * N2]);
+            const long long ix = ((e0 + el) * 5 + v) * NN + q;
+            double val = R;
+            if (a.mode != 0) {
+                const double y = a.Us[ix] + ifp::mul(dt, R);
+                val = a.first ? y : ifp::mul(a.ca, a.Un[ix]) + ifp::mul(a.cb, y);
             }
-            a.out[(e * 5 + v) * NN + t] = val;
+            a.out[ix] = val;
         }
     }
 }
@@ -302,15 +337,17 @@ __global__ void __launch_bounds__(128) k_limit(const __grid_constant__ LimitArgs
 
 // Dispatch helpers instantiated once per NP in dg_stage_fp64_n*.cu.
 template <int NP>
-cudaError_t launch_stage_np(const StageArgs &a, cudaStream_t s)
+cudaError_t launch_stage_np(const StageArgs &args, cudaStream_t s)
 {
-    const dim3 grid((unsigned)a.E), block(round_up32(NP * NP * NP));
-    const size_t smem = sizeof(double) * 20 * NP * NP * NP;
-    if (smem > 48 * 1024) {
-        cudaError_t err = cudaFuncSetAttribute(k_stage_fp64<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    using SH = StageShape64<NP>;
+    StageArgs a = args;
+    for (int i = 0; i < NP * NP; ++i) a.DF[i] = ifp::factor(a.T.D[i]);
+    if (SH::SMEM > 48 * 1024) {
+        const cudaError_t err =
+            cudaFuncSetAttribute(k_stage_fp64<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM);
         if (err != cudaSuccess) return err;
     }
-    k_stage_fp64<NP><<<grid, block, smem, s>>>(a);
+    k_stage_fp64<NP><<<(unsigned)((a.E + SH::EPB - 1) / SH::EPB), SH::THREADS, SH::SMEM, s>>>(a);
     return cudaGetLastError();
 }
 
