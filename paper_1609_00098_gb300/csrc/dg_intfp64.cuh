@@ -37,10 +37,14 @@
 namespace dg {
 namespace ifp {
 
+// The bits of a double.  (Assembly on the device: given a plain cast the compiler turns
+// tests of these bits back into FP64 comparisons.)
 __host__ __device__ __forceinline__ uint64_t dbits(double x)
 {
 #ifdef __CUDA_ARCH__
-    return (uint64_t)__double_as_longlong(x);
+    uint32_t h, l;
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(l), "=r"(h) : "d"(x));
+    return ((uint64_t)h << 32) | l;
 #else
     uint64_t b;
     std::memcpy(&b, &x, 8);
@@ -109,12 +113,71 @@ __host__ __device__ __forceinline__ float bflt(uint32_t b)
 #endif
 }
 
+// The FP64 instructions of the rare paths.  Volatile assembly keeps them behind their
+// branches: left to itself the compiler computes the FP64 result every time and selects.
 __host__ __device__ __forceinline__ double native_mul(double a, double b)
 {
 #ifdef __CUDA_ARCH__
-    return __dmul_rn(a, b);
+    double r;
+    asm volatile("mul.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
+    return r;
 #else
     return a * b;
+#endif
+}
+
+__host__ __device__ __forceinline__ double native_add(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    double r;
+    asm volatile("add.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
+    return r;
+#else
+    return a + b;
+#endif
+}
+
+__host__ __device__ __forceinline__ double native_div(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    double r;
+    asm volatile("div.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
+    return r;
+#else
+    return a / b;
+#endif
+}
+
+__host__ __device__ __forceinline__ double native_root(double x)
+{
+#ifdef __CUDA_ARCH__
+    double r;
+    asm volatile("sqrt.rn.f64 %0, %1;" : "=d"(r) : "d"(x));
+    return r;
+#else
+    return std::sqrt(x);
+#endif
+}
+
+__host__ __device__ __forceinline__ double native_min(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    double r;
+    asm volatile("min.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
+    return r;
+#else
+    return std::fmin(a, b);
+#endif
+}
+
+__host__ __device__ __forceinline__ double native_max(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    double r;
+    asm volatile("max.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
+    return r;
+#else
+    return std::fmax(a, b);
 #endif
 }
 
@@ -138,35 +201,41 @@ __host__ __device__ __forceinline__ Factor factor(double x)
 }
 
 // Whether a factor is in the range the products below are exact for: zero, or an
-// exponent field in [E - span, E + span] around the bias (no product of two such
-// factors over- or underflows for span <= 500).
-__host__ __device__ __forceinline__ bool factor_ok(double x, uint32_t span = 500u)
+// exponent field within 500 of the bias (no product of two such factors over- or
+// underflows).
+__host__ __device__ __forceinline__ bool factor_ok(double x)
 {
     const uint64_t b = dbits(x);
-    const uint32_t ef = (hi32(b) >> 20) & 0x7ffu;
-    return ef - (1023u - span) <= 2u * span || (b << 1) == 0u;
+    const uint32_t m = hi32(b) << 1;  // exponent and significand, no sign
+    return (m - (523u << 21) < (1001u << 21)) | ((m | lo32(b)) == 0u);
 }
 
-// RN(f d) for two factors that factor_ok accepts.
-__host__ __device__ __forceinline__ double mul(const Factor &f, const Factor &d)
+// RN(f d) for two factors that factor_ok accepts, a zero product as +0.
+__host__ __device__ __forceinline__ double mul_unsigned_zero(const Factor &f, const Factor &d)
 {
     const uint64_t p0 = mulw(f.l, d.l);
     const uint64_t p1 = mulw(f.h, d.l) + hi32(p0);
     const uint64_t p2 = mulw(f.l, d.h) + lo32(p1);
-    const uint64_t T = mulw(f.h, d.h) + hi32(p1) + hi32(p2);  // top 64 bits of the product
+    uint64_t T = mulw(f.h, d.h) + hi32(p1) + hi32(p2);  // top 64 bits of the product
     const uint32_t th = hi32(T);
     const uint32_t n = th >> 31;  // 1: the product of the significands is >= 2
-    const uint64_t m = T >> (10 + n);
-    // the bits below the 53 kept, those of the lower 64 folded into the lowest one
-    // (the lowest bit is below the rounding position either way)
-    const uint32_t r = (lo32(T) & (n ? 0x7ffu : 0x3ffu)) | ((lo32(p2) | lo32(p0)) ? 1u : 0u);
-    const uint32_t up = r + (lo32(m) & 1u) > (n ? 0x400u : 0x200u) ? 1u : 0u;
-    // exponent field minus 1 (the significand's leading bit adds it back; a rounding
-    // carry into 2^53 raises the exponent by itself)
-    const uint32_t ex = (f.e & 0x7ff00000u) + (d.e & 0x7ff00000u) - (1024u << 20) + (n << 20);
-    uint64_t bits = mk64(ex, 0u) + m + up;
-    if (th == 0u) bits = 0u;
-    return bdbl(bits | mk64((f.e ^ d.e) & 0x80000000u, 0u));
+    // the bits of the lower 64 folded into the lowest one (below the rounding position)
+    const uint32_t rest = lo32(p2) | lo32(p0);
+    T |= rest != 0u ? 1u : 0u;
+    // to nearest even at bit 10 + n: half an ulp less one, plus the bit kept last (the
+    // top 64 bits of a product end at least 2^12 below 2^64, so nothing carries out)
+    T += (0x1ffu + (n << 9)) + ((uint32_t)(T >> (10 + n)) & 1u);
+    // sign and exponent fields of the product, the exponent less 1 (the significand's
+    // leading bit adds it back; a rounding carry into 2^53 raises it by itself)
+    const uint32_t e = f.e + (d.e - (1024u << 20)) + (n << 20);
+    return bdbl((T >> (10 + n)) + mk64(th == 0u ? 0u : e, 0u));
+}
+
+// RN(f d), the sign of a zero product included.
+__host__ __device__ __forceinline__ double mul(const Factor &f, const Factor &d)
+{
+    const uint64_t b = dbits(mul_unsigned_zero(f, d));
+    return bdbl(b | mk64((f.e ^ d.e) & 0x80000000u, 0u));
 }
 
 // RN(a b).  (The fast result is formed first and replaced where an operand is out of
@@ -214,7 +283,7 @@ __host__ __device__ __forceinline__ double div(double a, const Divisor &d)
     const uint64_t ab = dbits(a);
     const uint32_t ah = hi32(ab);
     const uint32_t ea = (ah >> 20) & 0x7ffu, eb = (d.h >> 20) & 0x7ffu;
-    const bool zero = (ab << 1) == 0u;
+    const bool zero = ((ah << 1) | lo32(ab)) == 0u;
     uint64_t rem = mk64((ah & 0xfffffu) | 0x100000u, lo32(ab));
     uint32_t ex = ea - eb + 1022u;  // exponent field minus 1
     if (rem < d.B) {
@@ -236,13 +305,7 @@ __host__ __device__ __forceinline__ double div(double a, const Divisor &d)
     if (zero) bits = 0u;
     double r = bdbl(bits | mk64((ah ^ d.h) & 0x80000000u, 0u));
     // both in the middle of the exponent range (normal operands, normal quotient), or 0 / b
-    if (!((((ea - 523u) <= 1000u) | zero) & ((eb - 523u) <= 1000u))) {
-#ifdef __CUDA_ARCH__
-        r = __ddiv_rn(a, d.b);
-#else
-        r = a / d.b;
-#endif
-    }
+    if (!((((ea - 523u) <= 1000u) | zero) & ((eb - 523u) <= 1000u))) r = native_div(a, d.b);
     return r;
 }
 
@@ -285,13 +348,7 @@ __host__ __device__ __forceinline__ double root(double x)
     F += R < 0 ? 0u : (R > (int64_t)(2u * F) ? 2u : 1u);  // floor + 1 (the rounding)
     const uint32_t ex = (ef - odd + 1023u) >> 1;
     double r = bdbl(mk64((ex - 1u) << 20, 0u) + (F >> 1));
-    if (!((xh >> 20) - 1u <= 2045u)) {  // not positive and normal
-#ifdef __CUDA_ARCH__
-        r = __dsqrt_rn(x);
-#else
-        r = std::sqrt(x);
-#endif
-    }
+    if (!((xh >> 20) - 1u <= 2045u)) r = native_root(x);  // not positive and normal
     return r;
 }
 
@@ -312,14 +369,14 @@ __host__ __device__ __forceinline__ bool maybe_nan(double x)
 __host__ __device__ __forceinline__ double least(double a, double b)
 {
     double r = order_key(a) < order_key(b) ? a : b;
-    if (maybe_nan(a) | maybe_nan(b)) r = fmin(a, b);
+    if (maybe_nan(a) | maybe_nan(b)) r = native_min(a, b);
     return r;
 }
 
 __host__ __device__ __forceinline__ double greatest(double a, double b)
 {
     double r = order_key(a) > order_key(b) ? a : b;
-    if (maybe_nan(a) | maybe_nan(b)) r = fmax(a, b);
+    if (maybe_nan(a) | maybe_nan(b)) r = native_max(a, b);
     return r;
 }
 

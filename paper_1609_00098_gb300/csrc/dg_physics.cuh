@@ -38,15 +38,18 @@ struct C2PEval {
     double f, df;
 };
 
-__device__ __forceinline__ C2PEval sr_c2p_eval(double g, double D, double s2, double tau, double p)
+// E = tau + D.  Six divisions and a square root bound an evaluation; they and the
+// products run on the integer ALU (dg_intfp64.cuh).
+__device__ __forceinline__ C2PEval sr_c2p_eval(double g, double D, double E, double s2, double tau, double p)
 {
     C2PEval r;
-    const double Ep = tau + D + p;
-    const double v2 = s2 / (Ep * Ep);
-    const double W = 1.0 / sqrt(1.0 - v2);
-    const double rhoeps = tau - v2 * (Ep - D * W / (W + 1.0));
-    r.f = p - (g - 1.0) * rhoeps;
-    r.df = 1.0 - (g - 1.0) * v2 * (1.0 - D * W / Ep);
+    const double Ep = E + p;
+    const double v2 = ifp::div(s2, ifp::mul(Ep, Ep));
+    const double W = ifp::div(1.0, ifp::root(1.0 - v2));
+    const double DW = ifp::mul(D, W);
+    const double rhoeps = tau - ifp::mul(v2, Ep - ifp::div(DW, W + 1.0));
+    r.f = p - ifp::mul(g - 1.0, rhoeps);
+    r.df = 1.0 - ifp::mul(ifp::mul(g - 1.0, v2), 1.0 - ifp::div(DW, Ep));
     return r;
 }
 
@@ -54,74 +57,6 @@ __device__ __forceinline__ bool sr_unphysical(const double u[5])
 {
     const double s2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
     return !(u[0] > 0.0) || !(u[4] > 0.0) || !(s2 < u[4] * (u[4] + 2.0 * u[0]));
-}
-
-// Returns 0 ok, 1 unphysical input, 2 no convergence.  prim = (rho, vx, vy, vz, p).
-// guess < 0 selects the standard guess (g-1) tau.
-__device__ __forceinline__ int sr_con2prim(double g, const double u[5], double guess, double prim[5],
-                                           int *iters)
-{
-    const double D = u[0], tau = u[4];
-    const double s2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
-    *iters = 0;
-    if (!(D > 0.0) || !(tau > 0.0) || !(s2 < tau * (tau + 2.0 * D))) {
-        for (int v = 0; v < 5; ++v) prim[v] = __longlong_as_double(0x7ff8000000000000LL);
-        return 1;
-    }
-    const double E = tau + D;
-    double plo = sqrt(s2) - E;
-    if (plo < 0.0) plo = 0.0;
-    double phi = (g - 1.0) * tau;
-    double p = (guess >= 0.0) ? guess : phi;
-    if (p < plo) p = plo;
-    if (p > phi) p = phi;
-    int status = 2;
-    bool lo_moved = false, hi_moved = false;  // an end still at its a-priori bound may be landed on
-    int it = 0;
-    for (; it < 200; ++it) {
-        const C2PEval r = sr_c2p_eval(g, D, s2, tau, p);
-        if (r.f == 0.0) { status = 0; break; }
-        if (r.f > 0.0) { phi = p; hi_moved = true; } else { plo = p; lo_moved = true; }
-        double pn = p - r.f / r.df;
-        if (!((pn > plo && pn < phi) || (pn == phi && !hi_moved) || (pn == plo && !lo_moved)))
-            pn = 0.5 * (plo + phi);
-        const double dp = fabs(pn - p);
-        p = pn;
-        if (dp <= 0x1p-48 * p) {
-            const C2PEval r2 = sr_c2p_eval(g, D, s2, tau, p);
-            p = p - r2.f / r2.df;
-            it += 1;
-            status = 0;
-            break;
-        }
-        if (phi - plo <= 0.0) { status = 0; break; }
-    }
-    *iters = it + 1;
-    const double Ep = E + p;
-    prim[0] = D * sqrt(1.0 - s2 / (Ep * Ep));
-    prim[1] = u[1] / Ep;
-    prim[2] = u[2] / Ep;
-    prim[3] = u[3] / Ep;
-    prim[4] = p;
-    return status;
-}
-
-// Flux-relevant primitives (vx, vy, vz, p) of either system; returns c2p status.
-template <int SYS>
-__device__ __forceinline__ int node_primitives(double g, const double u[5], double P[4])
-{
-    if (SYS == 0) {
-        ne_primitives(g, u, P);
-        return 0;
-    }
-    double pr[5];
-    int it;
-    const int st = sr_con2prim(g, u, -1.0, pr, &it);
-    P[0] = pr[1];
-    P[1] = pr[2];
-    P[2] = pr[3];
-    P[3] = pr[4];
-    return st;
 }
 
 // ---------------------------------------------------------------------------

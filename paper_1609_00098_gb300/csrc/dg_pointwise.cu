@@ -2,6 +2,7 @@
 // and the CFL wave-speed maximum, the SR fix alone, the CFL step, node
 // coordinates, primitive->conserved, and standalone con2prim.
 #include "dg_internal.h"
+#include "dg_con2prim_fp64.cuh"
 #include "dg_physics.cuh"
 
 namespace dg {
@@ -28,50 +29,105 @@ struct PrimArgs {
     double gamma, d_atm, tau_atm;
 };
 
-// One thread per node: (optional SR fix of the node in place), primitives
-// (vx, vy, vz, p) into P[e][c][node], and the block-reduced largest wave speed
-// folded into *lam with an integer atomicMax on the bit pattern (exact and
-// independent of order for non-negative doubles).
-template <int SYS>
-__global__ void __launch_bounds__(kThreads) k_primitives(const PrimArgs a)
+// Largest of the CTA's values into *lam with an integer atomicMax on the bit pattern
+// (exact and independent of order for non-negative doubles).
+template <int THREADS>
+__device__ __forceinline__ void block_max(double lmax, unsigned long long *lam)
+{
+    __shared__ double red[THREADS / 32];
+    for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lmax;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double m = red[0];
+        for (int w = 1; w < THREADS / 32; ++w) m = fmax(m, red[w]);
+        atomicMax(lam, (unsigned long long)__double_as_longlong(m));
+    }
+}
+
+// Newtonian primitives, one thread per node: (vx, vy, vz, p) into P[e][c][node], and
+// the largest wave speed into *lam.
+__global__ void __launch_bounds__(kThreads) k_primitives_ne(const PrimArgs a)
 {
     double lmax = 0.0;
-    unsigned errs = 0;
     for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < a.total;
          g += (long long)gridDim.x * blockDim.x) {
         const long long e = g / a.nn;
         const int q = (int)(g - e * a.nn);
-        double u[5];
+        double u[5], P[4];
 #pragma unroll
         for (int v = 0; v < 5; ++v) u[v] = a.U[(e * 5 + v) * a.nn + q];
-        if (SYS == 1 && a.Ufix) {
+        ne_primitives(a.gamma, u, P);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) a.P[(e * 4 + c) * a.nn + q] = P[c];
+        if (a.lam) lmax = ifp::greatest(lmax, max_speed<0>(a.gamma, u, P));
+    }
+    if (a.lam) block_max<kThreads>(lmax, a.lam);
+}
+
+// SR primitives by con2prim from the standard guess (c2p_warp), with the conserved fix
+// of the node in place first where a.Ufix is given, and the largest wave speed.
+struct PrimIO {
+    const PrimArgs &a;
+    double lmax;
+    unsigned errs;
+
+    __device__ __forceinline__ long long at(long long g, int rows, int row) const
+    {
+        const long long e = g / a.nn;
+        return (e * rows + row) * a.nn + (g - e * a.nn);
+    }
+    __device__ __forceinline__ void load(long long g, double u[5])
+    {
+        const long long b = at(g, 5, 0);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) u[v] = a.U[b + v * a.nn];
+        if (a.Ufix) {
             double f[5] = {u[0], u[1], u[2], u[3], u[4]};
             if (sr_fix(a.d_atm, a.tau_atm, f)) {
 #pragma unroll
                 for (int v = 0; v < 5; ++v) {
-                    if (f[v] != u[v]) a.Ufix[(e * 5 + v) * a.nn + q] = f[v];
+                    if (f[v] != u[v]) a.Ufix[b + v * a.nn] = f[v];
                     u[v] = f[v];
                 }
             }
         }
-        double P[4];
-        if (node_primitives<SYS>(a.gamma, u, P)) errs |= ERRBIT_C2P;
+    }
+    __device__ __forceinline__ double guess(long long) const { return -1.0; }
+    __device__ __forceinline__ void bad(long long g)
+    {
+        const long long b = at(g, 4, 0);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) a.P[(e * 4 + c) * a.nn + q] = P[c];
-        if (a.lam) lmax = fmax(lmax, max_speed<SYS>(a.gamma, u, P));
+        for (int c = 0; c < 4; ++c) a.P[b + c * a.nn] = __longlong_as_double(0x7ff8000000000000LL);
+        errs |= ERRBIT_C2P;
     }
-    if (errs) atomicOr(a.err, errs);
-    if (a.lam) {
-        __shared__ double red[kThreads / 32];
-        for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lmax;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double m = red[0];
-            for (int w = 1; w < kThreads / 32; ++w) m = fmax(m, red[w]);
-            atomicMax(a.lam, (unsigned long long)__double_as_longlong(m));
-        }
+    __device__ __forceinline__ void iterations(long long, int, int status)
+    {
+        if (status) errs |= ERRBIT_C2P;
     }
+    __device__ __forceinline__ void finish(long long g, double D, double, double E, double p)
+    {
+        const long long b = at(g, 4, 0), bu = at(g, 5, 0);
+        const ifp::Divisor Ep = ifp::divisor(E + p);
+        double u[5], P[4];
+        u[0] = D;
+#pragma unroll
+        for (int v = 1; v < 5; ++v) u[v] = a.U[bu + v * a.nn];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a.P[b + c * a.nn] = P[c] = ifp::div(u[1 + c], Ep);
+        a.P[b + 3 * a.nn] = P[3] = p;
+        if (a.lam) lmax = ifp::greatest(lmax, max_speed<1>(a.gamma, u, P));
+    }
+};
+
+__global__ void __launch_bounds__(kC2pThreads, 5) k_primitives_sr(const PrimArgs a)
+{
+    __shared__ C2pWarp Q[kC2pThreads / 32];
+    PrimIO io{a, 0.0, 0u};
+    const long long warp = ((long long)blockIdx.x * kC2pThreads + threadIdx.x) >> 5;
+    c2p_warp(io, Q[threadIdx.x >> 5], a.gamma, a.total, warp, (long long)gridDim.x * (kC2pThreads / 32));
+    if (io.errs) atomicOr(a.err, io.errs);
+    if (a.lam) block_max<kC2pThreads>(io.lmax, a.lam);
 }
 
 __global__ void __launch_bounds__(kThreads) k_fix(double *U, long long total, int nn, double d_atm, double tau_atm)
@@ -331,22 +387,52 @@ __global__ void __launch_bounds__(kThreads) k_prim2con(const double *prim, doubl
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_con2prim(long long count, double gamma, const double *cons,
-                                                       double *prim, const double *guess, int *iters,
-                                                       int *status)
-{
-    for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < count;
-         g += (long long)gridDim.x * blockDim.x) {
-        double u[5], pr[5];
+// Standalone con2prim: 5 rows of `count` in and out (they may be the same arrays: a
+// node's rows are written only after its last read).
+struct RowsIO {
+    long long count;
+    const double *cons;
+    double *prim;
+    const double *guesses;
+    int *iters, *status;
+
+    __device__ __forceinline__ void load(long long i, double u[5])
+    {
 #pragma unroll
-        for (int v = 0; v < 5; ++v) u[v] = cons[v * count + g];
-        int it;
-        const int st = sr_con2prim(gamma, u, guess ? guess[g] : -1.0, pr, &it);
-#pragma unroll
-        for (int v = 0; v < 5; ++v) prim[v * count + g] = pr[v];
-        if (iters) iters[g] = it;
-        if (status) status[g] = st;
+        for (int v = 0; v < 5; ++v) u[v] = cons[v * count + i];
     }
+    __device__ __forceinline__ double guess(long long i) const { return guesses ? guesses[i] : -1.0; }
+    __device__ __forceinline__ void bad(long long i)
+    {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) prim[v * count + i] = __longlong_as_double(0x7ff8000000000000LL);
+        if (iters) iters[i] = 0;
+        if (status) status[i] = 1;
+    }
+    __device__ __forceinline__ void iterations(long long i, int n, int st)
+    {
+        if (iters) iters[i] = n;
+        if (status) status[i] = st;
+    }
+    __device__ __forceinline__ void finish(long long i, double D, double s2, double E, double p)
+    {
+        const double Ep = E + p;
+        const ifp::Divisor dE = ifp::divisor(Ep);
+        const double v1 = ifp::div(cons[count + i], dE), v2 = ifp::div(cons[2 * count + i], dE);
+        const double v3 = ifp::div(cons[3 * count + i], dE);
+        prim[i] = ifp::mul(D, ifp::root(1.0 - ifp::div(s2, ifp::mul(Ep, Ep))));
+        prim[count + i] = v1;
+        prim[2 * count + i] = v2;
+        prim[3 * count + i] = v3;
+        prim[4 * count + i] = p;
+    }
+};
+
+__global__ void __launch_bounds__(kC2pThreads, 5) k_con2prim(RowsIO io, double gamma)
+{
+    __shared__ C2pWarp Q[kC2pThreads / 32];
+    const long long warp = ((long long)blockIdx.x * kC2pThreads + threadIdx.x) >> 5;
+    c2p_warp(io, Q[threadIdx.x >> 5], gamma, io.count, warp, (long long)gridDim.x * (kC2pThreads / 32));
 }
 
 __global__ void k_set(double *p, double v) { *p = v; }
@@ -373,9 +459,8 @@ cudaError_t launch_primitives(const dg_mesh *m, const double *U, double *P, int 
     a.gamma = m->d.gamma;
     a.d_atm = m->d.d_atm;
     a.tau_atm = m->d.tau_atm;
-    const unsigned grid = grid_for(a.total, kThreads);
-    if (m->d.system == 0) k_primitives<0><<<grid, kThreads, 0, s>>>(a);
-    else k_primitives<1><<<grid, kThreads, 0, s>>>(a);
+    if (m->d.system == 0) k_primitives_ne<<<grid_for(a.total, kThreads), kThreads, 0, s>>>(a);
+    else k_primitives_sr<<<c2p_grid(a.total), kC2pThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -468,7 +553,8 @@ cudaError_t launch_prim2con(const dg_mesh *m, const double *prim, double *U, cud
 cudaError_t launch_con2prim(long long count, double gamma, const double *cons, double *prim,
                             const double *guess, int *iters, int *status, cudaStream_t s)
 {
-    k_con2prim<<<grid_for(count, kThreads), kThreads, 0, s>>>(count, gamma, cons, prim, guess, iters, status);
+    const RowsIO io{count, cons, prim, guess, iters, status};
+    k_con2prim<<<c2p_grid(count), kC2pThreads, 0, s>>>(io, gamma);
     return cudaGetLastError();
 }
 

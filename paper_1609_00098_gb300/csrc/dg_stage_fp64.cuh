@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const 
                 const ifp::Factor fl = ifp::factor(f[l]);
 #pragma unroll
                 for (int i = 0; i < NP; ++i) {
-                    const double p = ifp::mul(fl, a.DF[i * NP + l]);
+                    const double p = ifp::mul_unsigned_zero(fl, a.DF[i * NP + l]);
                     s[i] = l == 0 ? p : s[i] + p;
                 }
             }
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const 
             for (int l = 0; l < NP; ++l)
 #pragma unroll
                 for (int i = 0; i < NP; ++i) {
-                    const double p = a.T.D[i * NP + l] * f[l];
+                    const double p = ifp::native_mul(a.T.D[i * NP + l], f[l]);
                     s[i] = l == 0 ? p : s[i] + p;
                 }
         }
@@ -161,7 +161,9 @@ __global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const 
 // w x for a quadrature weight w (prepared factor f of the double fd) and a state value x.
 __device__ __forceinline__ double weighted(const ifp::Factor &f, double fd, double x)
 {
-    return ifp::factor_ok(x) ? ifp::mul(ifp::factor(x), f) : fd * x;
+    double r = ifp::mul_unsigned_zero(ifp::factor(x), f);
+    if (!ifp::factor_ok(x)) r = ifp::native_mul(fd, x);
+    return r;
 }
 
 // Limiter summaries S[e][v][10] of a.G consecutive elements per CTA: [0] the cell mean
