@@ -25,6 +25,8 @@ struct C2pWarp {
     C2pQueue in, out;  // (out.plo unused)
 };
 
+static __device__ __noinline__ double c2p_bisect(double plo, double phi) { return 0.5 * (plo + phi); }
+
 // All nodes i = 32 b + lane of the batches b = warp, warp + nwarps, ... below count.
 // io.load(i, u) the conserved state (after any fix), io.guess(i) the starting pressure
 // (< 0: the standard guess (g-1) tau), io.bad(i) an unphysical state, io.iterations(i,
@@ -112,8 +114,10 @@ __device__ __forceinline__ void c2p_warp(IO &io, C2pWarp &Q, double g, long long
             if (!__ballot_sync(full, act)) break;
         }
         // one iteration (or, after the step below the tolerance, one more Newton step)
-        const C2PEval r = sr_c2p_eval(g, D, E, s2, tau, p);
-        double pn = p - ifp::div(r.f, r.df);
+        ifp::Fast ar;
+        C2PEval r = sr_c2p_eval(ar, g, D, E, s2, tau, p);
+        if (!ar.ok) r = sr_c2p_eval_native(g, D, E, s2, tau, p);
+        double pn = p - r.step;
         bool done = last;
         int iters = it + 2, status = 0;
         if (!last) {
@@ -133,11 +137,11 @@ __device__ __forceinline__ void c2p_warp(IO &io, C2pWarp &Q, double g, long long
                 const long long kn = (long long)ifp::dbits(pn), kl = (long long)ifp::dbits(plo);
                 const long long kh = (long long)ifp::dbits(phi);
                 const bool in = kn >= 0 && ((kn > kl && kn < kh) || (kn == kh && !hi_moved) || (kn == kl && !lo_moved));
-                if (!in) pn = ifp::native_mul(0.5, ifp::native_add(plo, phi));
+                if (!in) pn = c2p_bisect(plo, phi);
                 // |pn - p| <= 2^-48 pn, the product by the exponent field while it is normal
                 const long long kd = (long long)(ifp::dbits(pn - p) & 0x7fffffffffffffffULL);
                 long long kt = (long long)ifp::dbits(pn) - (48LL << 52);
-                if (kt < (1LL << 52)) kt = (long long)ifp::dbits(ifp::native_mul(0x1p-48, pn));
+                if (kt < (1LL << 52)) kt = (long long)ifp::dbits(ifp::slow_mul(0x1p-48, pn));
                 last = kd <= kt;
                 if (!last && kh <= kl && kh < kInfBits) {
                     done = true;

@@ -113,73 +113,19 @@ __host__ __device__ __forceinline__ float bflt(uint32_t b)
 #endif
 }
 
-// The FP64 instructions of the rare paths.  Volatile assembly keeps them behind their
-// branches: left to itself the compiler computes the FP64 result every time and selects.
-__host__ __device__ __forceinline__ double native_mul(double a, double b)
-{
-#ifdef __CUDA_ARCH__
-    double r;
-    asm volatile("mul.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
-    return r;
-#else
-    return a * b;
+// The FP64 instructions of the rare paths, as calls: inlined, the compiler executes
+// them every time and selects, and an FP64 instruction holds its pipe even with every
+// lane predicated off.
+#ifdef __CUDACC__
+static __device__ __noinline__ double slow_mul(double a, double b) { return __dmul_rn(a, b); }
+static __device__ __noinline__ double slow_div(double a, double b) { return __ddiv_rn(a, b); }
+static __device__ __noinline__ double slow_root(double x) { return __dsqrt_rn(x); }
 #endif
-}
-
-__host__ __device__ __forceinline__ double native_add(double a, double b)
-{
 #ifdef __CUDA_ARCH__
-    double r;
-    asm volatile("add.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
-    return r;
+#define DG_IFP_SLOW(device_expr, host_expr) device_expr
 #else
-    return a + b;
+#define DG_IFP_SLOW(device_expr, host_expr) host_expr
 #endif
-}
-
-__host__ __device__ __forceinline__ double native_div(double a, double b)
-{
-#ifdef __CUDA_ARCH__
-    double r;
-    asm volatile("div.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
-    return r;
-#else
-    return a / b;
-#endif
-}
-
-__host__ __device__ __forceinline__ double native_root(double x)
-{
-#ifdef __CUDA_ARCH__
-    double r;
-    asm volatile("sqrt.rn.f64 %0, %1;" : "=d"(r) : "d"(x));
-    return r;
-#else
-    return std::sqrt(x);
-#endif
-}
-
-__host__ __device__ __forceinline__ double native_min(double a, double b)
-{
-#ifdef __CUDA_ARCH__
-    double r;
-    asm volatile("min.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
-    return r;
-#else
-    return std::fmin(a, b);
-#endif
-}
-
-__host__ __device__ __forceinline__ double native_max(double a, double b)
-{
-#ifdef __CUDA_ARCH__
-    double r;
-    asm volatile("max.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
-    return r;
-#else
-    return std::fmax(a, b);
-#endif
-}
 
 // ---------------------------------------------------------------------------
 // A factor prepared for products: the 53-bit significand shifted left by 11 (top bit
@@ -243,7 +189,7 @@ __host__ __device__ __forceinline__ double mul(const Factor &f, const Factor &d)
 __host__ __device__ __forceinline__ double mul(double a, double b)
 {
     double r = mul(factor(a), factor(b));
-    if (!(factor_ok(a) & factor_ok(b))) r = native_mul(a, b);
+    if (!(factor_ok(a) & factor_ok(b))) r = DG_IFP_SLOW(slow_mul(a, b), a * b);
     return r;
 }
 
@@ -278,17 +224,25 @@ __host__ __device__ __forceinline__ Divisor divisor(double b)
     return d;
 }
 
-__host__ __device__ __forceinline__ double div(double a, const Divisor &d)
+// RN(a / b) where div_ok (a in the middle of the exponent range or zero, b in the
+// middle of it: normal operands, normal quotient).
+__host__ __device__ __forceinline__ bool div_ok(double a, const Divisor &d)
+{
+    const uint64_t ab = dbits(a);
+    const uint32_t m = hi32(ab) << 1;
+    return ((m - (523u << 21) < (1001u << 21)) | ((m | lo32(ab)) == 0u)) & ((d.h << 1) - (523u << 21) < (1001u << 21));
+}
+
+__host__ __device__ __forceinline__ double div_fast(double a, const Divisor &d)
 {
     const uint64_t ab = dbits(a);
     const uint32_t ah = hi32(ab);
-    const uint32_t ea = (ah >> 20) & 0x7ffu, eb = (d.h >> 20) & 0x7ffu;
-    const bool zero = ((ah << 1) | lo32(ab)) == 0u;
     uint64_t rem = mk64((ah & 0xfffffu) | 0x100000u, lo32(ab));
-    uint32_t ex = ea - eb + 1022u;  // exponent field minus 1
+    // exponent field of the quotient less 1
+    uint32_t ex = (ah & 0x7ff00000u) - (d.h & 0x7ff00000u) + (1022u << 20);
     if (rem < d.B) {
         rem <<= 1;
-        ex -= 1u;
+        ex -= 1u << 20;
     }
     const uint32_t q1 = hi32(mulw((uint32_t)(rem >> 22), d.r)) >> 12;
     rem <<= 18;
@@ -301,11 +255,15 @@ __host__ __device__ __forceinline__ double div(double a, const Divisor &d)
     rem += mulw(q3, d.nl) + mk64(q3 * d.nh, 0u);
     uint64_t Q = ((uint64_t)q1 << 35) + ((uint64_t)q2 << 17) + q3;  // floor(2^53 A/B), or one below
     Q += rem >= d.B ? 2u : 1u;                                      // corrected, plus the rounding 1
-    uint64_t bits = mk64(ex << 20, 0u) + (Q >> 1);
-    if (zero) bits = 0u;
-    double r = bdbl(bits | mk64((ah ^ d.h) & 0x80000000u, 0u));
-    // both in the middle of the exponent range (normal operands, normal quotient), or 0 / b
-    if (!((((ea - 523u) <= 1000u) | zero) & ((eb - 523u) <= 1000u))) r = native_div(a, d.b);
+    uint64_t bits = mk64(ex, 0u) + (Q >> 1);
+    if ((ah & 0x7ff00000u) == 0u) bits = 0u;  // a = 0
+    return bdbl(bits | mk64((ah ^ d.h) & 0x80000000u, 0u));
+}
+
+__host__ __device__ __forceinline__ double div(double a, const Divisor &d)
+{
+    double r = div_fast(a, d);
+    if (!div_ok(a, d)) r = DG_IFP_SLOW(slow_div(a, d.b), a / d.b);
     return r;
 }
 
@@ -316,7 +274,9 @@ __host__ __device__ __forceinline__ double div(double a, double b) { return div(
 // y ~ 1/sqrt(v) (FP32): S1 = 2^24 sqrt(v) from y, the exact remainder V - S1^2 2^4
 // gives the next bits through y/2, twice; then floor(2^53 sqrt v) is fixed against the
 // exact remainder.
-__host__ __device__ __forceinline__ double root(double x)
+__host__ __device__ __forceinline__ bool root_ok(double x) { return (hi32(dbits(x)) >> 20) - 1u <= 2045u; }  // positive, normal
+
+__host__ __device__ __forceinline__ double root_fast(double x)
 {
     const uint64_t xb = dbits(x);
     const uint32_t xh = hi32(xb);
@@ -347,38 +307,82 @@ __host__ __device__ __forceinline__ double root(double x)
     int64_t R = (int64_t)((V << 54) - (mulw(fl, fl) + mk64(2u * fh * fl, 0u)));
     F += R < 0 ? 0u : (R > (int64_t)(2u * F) ? 2u : 1u);  // floor + 1 (the rounding)
     const uint32_t ex = (ef - odd + 1023u) >> 1;
-    double r = bdbl(mk64((ex - 1u) << 20, 0u) + (F >> 1));
-    if (!((xh >> 20) - 1u <= 2045u)) r = native_root(x);  // not positive and normal
+    return bdbl(mk64((ex - 1u) << 20, 0u) + (F >> 1));
+}
+
+__host__ __device__ __forceinline__ double root(double x)
+{
+    double r = root_fast(x);
+    if (!root_ok(x)) r = DG_IFP_SLOW(slow_root(x), std::sqrt(x));
     return r;
 }
 
 // ---------------------------------------------------------------------------
-// fmin / fmax by comparing the bit patterns (negatives ordered in reverse); a NaN
-// operand takes the FP64 instruction.
+// fmin / fmax by comparing the bit patterns (negatives ordered in reverse), for
+// operands that are not NaN.
 __host__ __device__ __forceinline__ int64_t order_key(double x)
 {
     const int64_t b = (int64_t)dbits(x);
     return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
 }
 
-__host__ __device__ __forceinline__ bool maybe_nan(double x)
-{
-    return (hi32(dbits(x)) & 0x7fffffffu) >= 0x7ff00000u;
-}
+__host__ __device__ __forceinline__ bool finite(double x) { return (hi32(dbits(x)) & 0x7fffffffu) < 0x7ff00000u; }
 
-__host__ __device__ __forceinline__ double least(double a, double b)
-{
-    double r = order_key(a) < order_key(b) ? a : b;
-    if (maybe_nan(a) | maybe_nan(b)) r = native_min(a, b);
-    return r;
-}
+// ---------------------------------------------------------------------------
+// The arithmetic a formula is written for.  Fast runs these operations on the integer
+// ALU and notes in `ok` whether every operand was in range; a formula evaluated with it
+// is evaluated again with Native, in a call, where it was not.  One check per formula
+// keeps the FP64 instructions of the rare case behind one branch.  (Products that are
+// zero come out as +0.)
+struct Fast {
+    using Div = Divisor;
+    bool ok = true;
+    __host__ __device__ __forceinline__ double mul(double a, double b)
+    {
+        ok = ok & factor_ok(a) & factor_ok(b);
+        return mul_unsigned_zero(factor(a), factor(b));
+    }
+    __host__ __device__ __forceinline__ Div divisor(double b) { return ifp::divisor(b); }
+    __host__ __device__ __forceinline__ double div(double a, const Div &d)
+    {
+        ok = ok & div_ok(a, d);
+        return div_fast(a, d);
+    }
+    __host__ __device__ __forceinline__ double div(double a, double b) { return div(a, divisor(b)); }
+    __host__ __device__ __forceinline__ double root(double x)
+    {
+        ok = ok & root_ok(x);
+        return root_fast(x);
+    }
+    __host__ __device__ __forceinline__ double least(double a, double b)
+    {
+        ok = ok & finite(a) & finite(b);
+        return order_key(a) < order_key(b) ? a : b;
+    }
+    __host__ __device__ __forceinline__ double greatest(double a, double b)
+    {
+        ok = ok & finite(a) & finite(b);
+        return order_key(a) > order_key(b) ? a : b;
+    }
+    __host__ __device__ __forceinline__ bool positive(double x)
+    {
+        ok = ok & finite(x);
+        return (int64_t)dbits(x) > 0;
+    }
+};
 
-__host__ __device__ __forceinline__ double greatest(double a, double b)
-{
-    double r = order_key(a) > order_key(b) ? a : b;
-    if (maybe_nan(a) | maybe_nan(b)) r = native_max(a, b);
-    return r;
-}
+#ifdef __CUDACC__
+struct Native {
+    using Div = double;
+    __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+    __device__ __forceinline__ double divisor(double b) { return b; }
+    __device__ __forceinline__ double div(double a, double b) { return __ddiv_rn(a, b); }
+    __device__ __forceinline__ double root(double x) { return __dsqrt_rn(x); }
+    __device__ __forceinline__ double least(double a, double b) { return fmin(a, b); }
+    __device__ __forceinline__ double greatest(double a, double b) { return fmax(a, b); }
+    __device__ __forceinline__ bool positive(double x) { return x > 0.0; }
+};
+#endif
 
 }  // namespace ifp
 }  // namespace dg

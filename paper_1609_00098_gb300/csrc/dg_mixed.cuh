@@ -520,7 +520,7 @@ struct MixedSmem {
     }
 };
 
-// Physicality (bit 0 set if unphysical, as sr_unphysical) and whether the conserved
+// Physicality (bit 0 set if unphysical) and whether the conserved
 // fix of Sec. 2.1.4 would change u (bit 1, as a nonzero sr_fix), from one FP64
 // evaluation of S^2 and tau (tau + 2D), without the fix's rescaling.
 __device__ __forceinline__ unsigned sr_check64(double d_atm, double tau_atm, const double u[5])

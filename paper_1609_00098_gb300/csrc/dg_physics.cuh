@@ -15,13 +15,33 @@ enum : unsigned { ERRBIT_C2P = 1u, ERRBIT_UNPHYSICAL = 2u, ERRBIT_TIMEOUT = 4u }
 
 // ---------------------------------------------------------------------------
 // Newtonian Euler: U = [rho, rho v_i, E], E = rho eps + rho v^2/2, p = (g-1) rho eps.
+template <class A>
+__device__ __forceinline__ void ne_primitives(A &ar, double g, const double u[5], double P[4])
+{
+    const double inv = ar.div(1.0, u[0]);
+    P[0] = ar.mul(u[1], inv);
+    P[1] = ar.mul(u[2], inv);
+    P[2] = ar.mul(u[3], inv);
+    P[3] = ar.mul(g - 1.0, u[4] - 0.5 * (ar.mul(u[1], P[0]) + ar.mul(u[2], P[1]) + ar.mul(u[3], P[2])));
+}
+
+static __device__ __noinline__ void ne_primitives_native(double g, const double *u, double *P)
+{
+    ifp::Native ar;
+    ne_primitives(ar, g, u, P);
+}
+
 __device__ __forceinline__ void ne_primitives(double g, const double u[5], double P[4])
 {
-    const double inv = ifp::div(1.0, u[0]);
-    P[0] = ifp::mul(u[1], inv);
-    P[1] = ifp::mul(u[2], inv);
-    P[2] = ifp::mul(u[3], inv);
-    P[3] = ifp::mul(g - 1.0, u[4] - 0.5 * (ifp::mul(u[1], P[0]) + ifp::mul(u[2], P[1]) + ifp::mul(u[3], P[2])));
+    ifp::Fast ar;
+    ne_primitives(ar, g, u, P);
+    if (!ar.ok) {
+        const double w[5] = {u[0], u[1], u[2], u[3], u[4]};
+        double Q[4];
+        ne_primitives_native(g, w, Q);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) P[c] = Q[c];
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -35,75 +55,86 @@ __device__ __forceinline__ void ne_primitives(double g, const double u[5], doubl
 // the sign of f; stop once
 // |dp| <= 2^-48 p and take one more Newton step.
 struct C2PEval {
-    double f, df;
+    double f, step;  // f and f / f'
 };
 
-// E = tau + D.  Six divisions and a square root bound an evaluation; they and the
-// products run on the integer ALU (dg_intfp64.cuh).
-__device__ __forceinline__ C2PEval sr_c2p_eval(double g, double D, double E, double s2, double tau, double p)
+// E = tau + D.  Six divisions (the step's included) and a square root bound an
+// evaluation; they run on the integer ALU (dg_intfp64.cuh), the additions and as many
+// of the products as the FP64 pipe has time for on that.
+template <class A>
+__device__ __forceinline__ C2PEval sr_c2p_eval(A &ar, double g, double D, double E, double s2, double tau, double p)
 {
-    C2PEval r;
     const double Ep = E + p;
-    const double v2 = ifp::div(s2, ifp::mul(Ep, Ep));
-    const double W = ifp::div(1.0, ifp::root(1.0 - v2));
-    const double DW = ifp::mul(D, W);
-    const double rhoeps = tau - ifp::mul(v2, Ep - ifp::div(DW, W + 1.0));
-    r.f = p - ifp::mul(g - 1.0, rhoeps);
-    r.df = 1.0 - ifp::mul(ifp::mul(g - 1.0, v2), 1.0 - ifp::div(DW, Ep));
+    const double v2 = ar.div(s2, ar.mul(Ep, Ep));
+    const double W = ar.div(1.0, ar.root(1.0 - v2));
+    const double DW = ar.mul(D, W);
+    const double rhoeps = tau - v2 * (Ep - ar.div(DW, W + 1.0));
+    C2PEval r;
+    r.f = p - (g - 1.0) * rhoeps;
+    r.step = ar.div(r.f, 1.0 - (g - 1.0) * v2 * (1.0 - ar.div(DW, Ep)));
     return r;
 }
 
-__device__ __forceinline__ bool sr_unphysical(const double u[5])
+static __device__ __noinline__ C2PEval sr_c2p_eval_native(double g, double D, double E, double s2, double tau, double p)
+{
+    ifp::Native ar;
+    return sr_c2p_eval(ar, g, D, E, s2, tau, p);
+}
+
+static __device__ __noinline__ bool sr_unphysical_native(const double *u)
 {
     const double s2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
     return !(u[0] > 0.0) || !(u[4] > 0.0) || !(s2 < u[4] * (u[4] + 2.0 * u[0]));
 }
 
 // ---------------------------------------------------------------------------
+// Divisions, square roots and most products run on the integer ALU; the additions and
+// the last products of the HLL flux, as many as balance the two, on the FP64 pipe.
 // The face kernel takes the axis at run time: components by selection (indexing a
 // register array with a runtime value would move it to local memory).
 __device__ __forceinline__ double pick_axis(int a, double x, double y, double z) { return a == 0 ? x : (a == 1 ? y : z); }
 
 // Physical flux along axis a, common to both systems with alpha = 1, beta = 0:
 // F = [U0 v_a, S_i v_a + p delta_ia, (U4 + p) v_a].
-__device__ __forceinline__ void flux_axis(const double u[5], const double P[4], int a, double F[5])
+template <class A>
+__device__ __forceinline__ void flux_axis(A &ar, const double u[5], const double P[4], int a, double F[5])
 {
     const double va = pick_axis(a, P[0], P[1], P[2]), p = P[3];
-    F[0] = ifp::mul(u[0], va);
-    F[1] = ifp::mul(u[1], va);
-    F[2] = ifp::mul(u[2], va);
-    F[3] = ifp::mul(u[3], va);
+    F[0] = ar.mul(u[0], va);
+    F[1] = ar.mul(u[1], va);
+    F[2] = ar.mul(u[2], va);
+    F[3] = ar.mul(u[3], va);
     const double fn = pick_axis(a, F[1], F[2], F[3]) + p;
     if (a == 0) F[1] = fn;
     else if (a == 1) F[2] = fn;
     else F[3] = fn;
-    F[4] = ifp::mul(u[4] + p, va);
+    F[4] = ar.mul(u[4] + p, va);
 }
 
 // Extreme characteristic speeds along axis a (eq:CharDecomp).
-template <int SYS>
-__device__ __forceinline__ void speeds_axis(double g, const double u[5], const double P[4], int a,
+template <int SYS, class A>
+__device__ __forceinline__ void speeds_axis(A &ar, double g, const double u[5], const double P[4], int a,
                                             double &lmin, double &lmax)
 {
     const double va = pick_axis(a, P[0], P[1], P[2]), p = P[3];
     if (SYS == 0) {
-        const double c = ifp::root(ifp::div(ifp::mul(g, p), u[0]));
+        const double c = ar.root(ar.div(ar.mul(g, p), u[0]));
         lmin = va - c;
         lmax = va + c;
         return;
     }
-    const double v2 = ifp::mul(P[0], P[0]) + ifp::mul(P[1], P[1]) + ifp::mul(P[2], P[2]);
+    const double v2 = ar.mul(P[0], P[0]) + ar.mul(P[1], P[1]) + ar.mul(P[2], P[2]);
     const double w2i = 1.0 - v2;
-    const double cs2 = ifp::div(ifp::mul(g, p), ifp::mul(u[4] + u[0] + p, w2i));
+    const double cs2 = ar.div(ar.mul(g, p), ar.mul(u[4] + u[0] + p, w2i));
     const double om = 1.0 - cs2;
-    const double den = 1.0 - ifp::mul(v2, cs2);
-    double disc = ifp::mul(w2i, den - ifp::mul(ifp::mul(va, va), om));
+    const double den = 1.0 - ar.mul(v2, cs2);
+    double disc = ar.mul(w2i, den - ar.mul(ar.mul(va, va), om));
     if (disc < 0.0) disc = 0.0;
-    const double rt = ifp::mul(ifp::root(cs2), ifp::root(disc));
-    const double vo = ifp::mul(va, om);
-    const ifp::Divisor dd = ifp::divisor(den);
-    lmin = ifp::div(vo - rt, dd);
-    lmax = ifp::div(vo + rt, dd);
+    const double rt = ar.mul(ar.root(cs2), ar.root(disc));
+    const double vo = ar.mul(va, om);
+    const typename A::Div dd = ar.divisor(den);
+    lmin = ar.div(vo - rt, dd);
+    lmax = ar.div(vo + rt, dd);
 }
 
 // Roe dissipation D = sum_i alpha_i |lambda_i| e_i of eq:Roe for the Newtonian
@@ -111,77 +142,77 @@ __device__ __forceinline__ void speeds_axis(double g, const double u[5], const d
 // (eq:RoeAverages) of the velocity and of h = (E + p)/rho, eigenvalues u_n - c,
 // u_n (x3), u_n + c with c^2 = (g-1)(h - |v|^2/2), wave strengths from the jump on
 // the left eigenvectors in the frame (normal, t1, t2) = (a, a+1, a+2).
-__device__ __forceinline__ void roe_dissipation(double g, int a, const double uL[5], const double PL[4],
+template <class A>
+__device__ __forceinline__ void roe_dissipation(A &ar, double g, int a, const double uL[5], const double PL[4],
                                                 const double uR[5], const double PR[4], double D[5])
 {
-    using ifp::mul;
-    const double sl = ifp::root(uL[0]), sr = ifp::root(uR[0]);
-    const ifp::Divisor wsum = ifp::divisor(sl + sr);
+    const double sl = ar.root(uL[0]), sr = ar.root(uR[0]);
+    const typename A::Div wsum = ar.divisor(sl + sr);
     double vh[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) vh[i] = ifp::div(mul(sl, PL[i]) + mul(sr, PR[i]), wsum);
-    const double hL = ifp::div(uL[4] + PL[3], uL[0]), hR = ifp::div(uR[4] + PR[3], uR[0]);
-    const double hh = ifp::div(mul(sl, hL) + mul(sr, hR), wsum);
-    const double q2 = mul(vh[0], vh[0]) + mul(vh[1], vh[1]) + mul(vh[2], vh[2]);
-    const double c2 = mul(g - 1.0, hh - 0.5 * q2);
-    const double c = ifp::root(c2);
+    for (int i = 0; i < 3; ++i) vh[i] = ar.div(ar.mul(sl, PL[i]) + ar.mul(sr, PR[i]), wsum);
+    const double hL = ar.div(uL[4] + PL[3], uL[0]), hR = ar.div(uR[4] + PR[3], uR[0]);
+    const double hh = ar.div(ar.mul(sl, hL) + ar.mul(sr, hR), wsum);
+    const double q2 = ar.mul(vh[0], vh[0]) + ar.mul(vh[1], vh[1]) + ar.mul(vh[2], vh[2]);
+    const double c2 = ar.mul(g - 1.0, hh - 0.5 * q2);
+    const double c = ar.root(c2);
     const double un = pick_axis(a, vh[0], vh[1], vh[2]), ut1 = pick_axis(a, vh[1], vh[2], vh[0]);
     const double ut2 = pick_axis(a, vh[2], vh[0], vh[1]);
     const double jx = uR[1] - uL[1], jy = uR[2] - uL[2], jz = uR[3] - uL[3];
     const double j1 = uR[0] - uL[0], jn = pick_axis(a, jx, jy, jz);
     const double jt1 = pick_axis(a, jy, jz, jx), jt2 = pick_axis(a, jz, jx, jy), j5 = uR[4] - uL[4];
-    const double al3 = jt1 - mul(ut1, j1);
-    const double al4 = jt2 - mul(ut2, j1);
-    const double j5b = j5 - mul(al3, ut1) - mul(al4, ut2);
-    const double al2 = mul(ifp::div(g - 1.0, c2), mul(j1, hh - mul(un, un)) + mul(un, jn) - j5b);
-    const double al1 = ifp::div(mul(j1, un + c) - jn - mul(c, al2), 2.0 * c);
+    const double al3 = jt1 - ar.mul(ut1, j1);
+    const double al4 = jt2 - ar.mul(ut2, j1);
+    const double j5b = j5 - ar.mul(al3, ut1) - ar.mul(al4, ut2);
+    const double al2 = ar.mul(ar.div(g - 1.0, c2), ar.mul(j1, hh - ar.mul(un, un)) + ar.mul(un, jn) - j5b);
+    const double al1 = ar.div(ar.mul(j1, un + c) - jn - ar.mul(c, al2), 2.0 * c);
     const double al5 = j1 - (al1 + al2);
-    const double w1 = mul(fabs(un - c), al1), w2 = mul(fabs(un), al2), w5 = mul(fabs(un + c), al5);
-    const double w3 = mul(fabs(un), al3), w4 = mul(fabs(un), al4);
+    const double w1 = ar.mul(fabs(un - c), al1), w2 = ar.mul(fabs(un), al2), w5 = ar.mul(fabs(un + c), al5);
+    const double w3 = ar.mul(fabs(un), al3), w4 = ar.mul(fabs(un), al4);
     const double w = w1 + w2 + w5;
-    const double dn = mul(w1, un - c) + mul(w2, un) + mul(w5, un + c);
-    const double d1 = mul(w, ut1) + w3, d2 = mul(w, ut2) + w4;
+    const double dn = ar.mul(w1, un - c) + ar.mul(w2, un) + ar.mul(w5, un + c);
+    const double d1 = ar.mul(w, ut1) + w3, d2 = ar.mul(w, ut2) + w4;
     D[0] = w;
     D[1] = pick_axis(a, dn, d2, d1);
     D[2] = pick_axis(a, d1, dn, d2);
     D[3] = pick_axis(a, d2, d1, dn);
-    D[4] = mul(w1, hh - mul(un, c)) + mul(w2, 0.5 * q2) + mul(w3, ut1) + mul(w4, ut2) + mul(w5, hh + mul(un, c));
+    D[4] = ar.mul(w1, hh - ar.mul(un, c)) + ar.mul(w2, 0.5 * q2) + ar.mul(w3, ut1) + ar.mul(w4, ut2) + ar.mul(w5, hh + ar.mul(un, c));
 }
 
 // Numerical flux along +e_a between the lower state L and the upper state R:
 // FLX = 0 local Lax-Friedrichs (eq:LLF), 1 HLL with Davis speeds (eq:HLL), 2 Roe
 // (eq:Roe, Newtonian).
-template <int SYS, int FLX>
-__device__ __forceinline__ void num_flux(double g, int a, const double uL[5], const double PL[4],
+template <int SYS, int FLX, class A>
+__device__ __forceinline__ void num_flux(A &ar, double g, int a, const double uL[5], const double PL[4],
                                          const double uR[5], const double PR[4], double Fs[5])
 {
     double FL[5], FR[5], lminL, lmaxL, lminR, lmaxR;
-    flux_axis(uL, PL, a, FL);
-    flux_axis(uR, PR, a, FR);
+    flux_axis(ar, uL, PL, a, FL);
+    flux_axis(ar, uR, PR, a, FR);
     if (FLX == 2) {
         double D[5];
-        roe_dissipation(g, a, uL, PL, uR, PR, D);
+        roe_dissipation(ar, g, a, uL, PL, uR, PR, D);
 #pragma unroll
         for (int v = 0; v < 5; ++v) Fs[v] = 0.5 * (FL[v] + FR[v]) - 0.5 * D[v];
         return;
     }
-    speeds_axis<SYS>(g, uL, PL, a, lminL, lmaxL);
-    speeds_axis<SYS>(g, uR, PR, a, lminR, lmaxR);
+    speeds_axis<SYS>(ar, g, uL, PL, a, lminL, lmaxL);
+    speeds_axis<SYS>(ar, g, uR, PR, a, lminR, lmaxR);
     if (FLX == 0) {
-        const double al = ifp::greatest(ifp::greatest(fabs(lminL), fabs(lmaxL)), ifp::greatest(fabs(lminR), fabs(lmaxR)));
+        const double al = ar.greatest(ar.greatest(fabs(lminL), fabs(lmaxL)), ar.greatest(fabs(lminR), fabs(lmaxR)));
         const double hal = 0.5 * al;
 #pragma unroll
-        for (int v = 0; v < 5; ++v) Fs[v] = 0.5 * (FL[v] + FR[v]) - ifp::mul(hal, uR[v] - uL[v]);
+        for (int v = 0; v < 5; ++v) Fs[v] = 0.5 * (FL[v] + FR[v]) - ar.mul(hal, uR[v] - uL[v]);
     } else {
-        const double cmin = ifp::least(ifp::least(lminL, lminR), 0.0);
-        const double cmax = ifp::greatest(ifp::greatest(lmaxL, lmaxR), 0.0);
+        const double cmin = ar.least(ar.least(lminL, lminR), 0.0);
+        const double cmax = ar.greatest(ar.greatest(lmaxL, lmaxR), 0.0);
         const double den = cmax - cmin;
-        if (den > 0.0) {
-            const ifp::Divisor dd = ifp::divisor(den);
-            const double cc = ifp::div(ifp::mul(cmin, cmax), dd);
+        if (ar.positive(den)) {
+            const typename A::Div dd = ar.divisor(den);
+            const double cc = ar.div(ar.mul(cmin, cmax), dd);
 #pragma unroll
             for (int v = 0; v < 5; ++v)
-                Fs[v] = ifp::div(ifp::mul(cmax, FL[v]) - ifp::mul(cmin, FR[v]), dd) + ifp::mul(cc, uR[v] - uL[v]);
+                Fs[v] = ar.div(cmax * FL[v] - cmin * FR[v], dd) + cc * (uR[v] - uL[v]);
         } else {
 #pragma unroll
             for (int v = 0; v < 5; ++v) Fs[v] = 0.5 * (FL[v] + FR[v]);
@@ -189,16 +220,81 @@ __device__ __forceinline__ void num_flux(double g, int a, const double uL[5], co
     }
 }
 
-// Largest |characteristic speed| over the three axes.
-template <int SYS>
-__device__ __forceinline__ double max_speed(double g, const double u[5], const double P[4])
+template <int SYS, int FLX>
+static __device__ __noinline__ void num_flux_native(double g, int a, const double *uL, const double *PL, const double *uR,
+                                                    const double *PR, double *Fs)
 {
+    ifp::Native ar;
+    num_flux<SYS, FLX>(ar, g, a, uL, PL, uR, PR, Fs);
+}
+
+template <int SYS, int FLX>
+__device__ __forceinline__ void num_flux(double g, int a, const double uL[5], const double PL[4], const double uR[5],
+                                         const double PR[4], double Fs[5])
+{
+    ifp::Fast ar;
+    num_flux<SYS, FLX>(ar, g, a, uL, PL, uR, PR, Fs);
+    if (!ar.ok) {
+        const double l[5] = {uL[0], uL[1], uL[2], uL[3], uL[4]}, r[5] = {uR[0], uR[1], uR[2], uR[3], uR[4]};
+        const double p[4] = {PL[0], PL[1], PL[2], PL[3]}, q[4] = {PR[0], PR[1], PR[2], PR[3]};
+        double F[5];
+        num_flux_native<SYS, FLX>(g, a, l, p, r, q, F);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) Fs[v] = F[v];
+    }
+}
+
+// Largest |characteristic speed| over the three axes.  Per axis it is
+// (|x| + c) [/ d] of the two speeds (x -+ c) [/ d] with c >= 0: rounding is monotone and
+// symmetric, so these are the bits of the larger magnitude.  NaN speeds (a negative
+// pressure) count as 0, as fmax over the speeds themselves would have it.
+template <int SYS, class A>
+__device__ __forceinline__ double max_speed(A &ar, double g, const double u[5], const double P[4])
+{
+    const double p = P[3];
+    if (SYS == 0) {
+        const double c = ar.root(ar.div(ar.mul(g, p), u[0]));
+        return ar.greatest(fabs(P[0]), ar.greatest(fabs(P[1]), fabs(P[2]))) + c;
+    }
+    const double v2 = ar.mul(P[0], P[0]) + ar.mul(P[1], P[1]) + ar.mul(P[2], P[2]);
+    const double w2i = 1.0 - v2;
+    const double cs2 = ar.div(ar.mul(g, p), ar.mul(u[4] + u[0] + p, w2i));
+    const double cs = ar.root(cs2);
+    const double om = 1.0 - cs2;
+    const double den = 1.0 - ar.mul(v2, cs2);
+    const typename A::Div dd = ar.divisor(den);
     double s = 0.0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
+        const double va = P[a];
+        const double disc = ar.mul(w2i, den - ar.mul(ar.mul(va, va), om));
+        const double rt = ar.mul(cs, ar.root(disc));
+        s = ar.greatest(s, fabs(ar.div(fabs(ar.mul(va, om)) + rt, dd)));
+    }
+    return s;
+}
+
+template <int SYS>
+static __device__ __noinline__ double max_speed_native(double g, const double *u, const double *P)
+{
+    double s = 0.0;
+    ifp::Native ar;
+    for (int a = 0; a < 3; ++a) {
         double lo, hi;
-        speeds_axis<SYS>(g, u, P, a, lo, hi);
-        s = ifp::greatest(s, ifp::greatest(fabs(lo), fabs(hi)));
+        speeds_axis<SYS>(ar, g, u, P, a, lo, hi);
+        s = fmax(s, fmax(fabs(lo), fabs(hi)));
+    }
+    return s;
+}
+
+template <int SYS>
+__device__ __forceinline__ double max_speed(double g, const double u[5], const double P[4])
+{
+    ifp::Fast ar;
+    double s = max_speed<SYS>(ar, g, u, P);
+    if (!ar.ok) {
+        const double w[5] = {u[0], u[1], u[2], u[3], u[4]}, q[4] = {P[0], P[1], P[2], P[3]};
+        s = max_speed_native<SYS>(g, w, q);
     }
     return s;
 }

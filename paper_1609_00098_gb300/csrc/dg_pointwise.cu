@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kThreads) k_primitives_ne(const PrimArgs a)
         ne_primitives(a.gamma, u, P);
 #pragma unroll
         for (int c = 0; c < 4; ++c) a.P[(e * 4 + c) * a.nn + q] = P[c];
-        if (a.lam) lmax = ifp::greatest(lmax, max_speed<0>(a.gamma, u, P));
+        if (a.lam) lmax = fmax(lmax, max_speed<0>(a.gamma, u, P));
     }
     if (a.lam) block_max<kThreads>(lmax, a.lam);
 }
@@ -116,7 +116,7 @@ struct PrimIO {
 #pragma unroll
         for (int c = 0; c < 3; ++c) a.P[b + c * a.nn] = P[c] = ifp::div(u[1 + c], Ep);
         a.P[b + 3 * a.nn] = P[3] = p;
-        if (a.lam) lmax = ifp::greatest(lmax, max_speed<1>(a.gamma, u, P));
+        if (a.lam) lmax = fmax(lmax, max_speed<1>(a.gamma, u, P));
     }
 };
 

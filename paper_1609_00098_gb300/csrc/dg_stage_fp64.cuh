@@ -25,6 +25,37 @@ struct StageShape64 {
     static constexpr size_t SMEM = sizeof(double) * (15 * NN + 30 * N2) * EPB;
 };
 
+// The rare cases of the two integer-ALU phases, in FP64 instructions.
+static __device__ __noinline__ void node_fluxes_native(const double *u, const double *P, double *dst, int nn)
+{
+    ifp::Native ar;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        double f[5];
+        flux_axis(ar, u, P, ax, f);
+        for (int v = 0; v < 5; ++v) dst[(ax * 5 + v) * nn] = f[v];
+    }
+}
+
+static __device__ __noinline__ double scaled_sum_native(const double *g, const double *s, int st)
+{
+    return (g[0] * s[0] + g[1] * s[st]) + g[2] * s[2 * st];
+}
+
+template <int NP>
+static __device__ __noinline__ void line_native(const double *D, double *F, int st)
+{
+    double f[NP];
+#pragma unroll
+    for (int l = 0; l < NP; ++l) f[l] = F[l * st];
+    for (int i = 0; i < NP; ++i) {
+        double s = D[i * NP] * f[0];
+#pragma unroll
+        for (int l = 1; l < NP; ++l) s = s + D[i * NP + l] * f[l];
+        F[i * st] = s;
+    }
+}
+
 // One stage for EPB elements per CTA, in four phases:
 //   nodes   the fluxes F^a_v of the element (eq:411) into shared memory;
 //   faces   the stored numerical flux minus the element's own, times the lift factor,
@@ -36,9 +67,11 @@ struct StageShape64 {
 // Every sum keeps the order of a sequential evaluation node by node (products and sums
 // rounded separately), so the results are its bits.
 //
-// FP64-pipe bound: the products run on the integer ALU, with the entries of D prepared
+// Bound by the FP64 pipe and the integer ALU in about equal parts: the products of the
+// fluxes, the contraction and its scaling run on the integer ALU, with the entries of D prepared
 // by the host and each line's flux values prepared once for n products, which leaves
-// the FP64 pipe n - 1 additions per node, axis and variable.  With products and sums
+// the FP64 pipe n - 1 additions per node, axis and variable; the lift and the update
+// keep theirs on the FP64 pipe, which has room for them.  With products and sums
 // both on it and one thread per node, the contraction ran at half the rate (0.25e12
 // against 0.50e12 product-sum pairs/s).  Lines also give 15 n^2 threads' work where
 // nodes give n^3, which is what a mesh with fewer elements than SMs needs.
@@ -68,12 +101,18 @@ __global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const 
         for (int v = 0; v < 5; ++v) u[v] = a.Us[((e0 + el) * 5 + v) * NN + q];
 #pragma unroll
         for (int c = 0; c < 4; ++c) P[c] = a.P[((e0 + el) * 4 + c) * NN + q];
+        ifp::Fast ar;
+        double *const dst = sF + el * 15 * NN + q;
 #pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
             double f[5];
-            flux_axis(u, P, ax, f);
+            flux_axis(ar, u, P, ax, f);
 #pragma unroll
-            for (int v = 0; v < 5; ++v) sF[(el * 15 + ax * 5 + v) * NN + q] = f[v];
+            for (int v = 0; v < 5; ++v) dst[(ax * 5 + v) * NN] = f[v];
+        }
+        if (!ar.ok) {
+            const double w[5] = {u[0], u[1], u[2], u[3], u[4]}, p[4] = {P[0], P[1], P[2], P[3]};
+            node_fluxes_native(w, p, dst, NN);
         }
     }
     __syncthreads();
@@ -88,7 +127,7 @@ __global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const 
         const int q = ((as & 1) ? NP - 1 : 0) * sa + (p % NP) * sb + (p / NP) * sc;
         const double lift = (as & 1) ? (ax == 0 ? a.liftN[0] : ax == 1 ? a.liftN[1] : a.liftN[2])
                                      : (ax == 0 ? a.lift0[0] : ax == 1 ? a.lift0[1] : a.lift0[2]);
-        sL[r] = ifp::mul(lift, a.Fs[sFace[el][as] * 5 * N2 + vr] - sF[(el * 15 + ax * 5 + v) * NN + q]);
+        sL[r] = lift * (a.Fs[sFace[el][as] * 5 * N2 + vr] - sF[(el * 15 + ax * 5 + v) * NN + q]);
     }
     __syncthreads();
 
@@ -116,13 +155,8 @@ __global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const 
                 }
             }
         } else {  // values out of the products' range, infinities, NaN
-#pragma unroll
-            for (int l = 0; l < NP; ++l)
-#pragma unroll
-                for (int i = 0; i < NP; ++i) {
-                    const double p = ifp::native_mul(a.T.D[i * NP + l], f[l]);
-                    s[i] = l == 0 ? p : s[i] + p;
-                }
+            line_native<NP>(a.T.D, F, st);
+            continue;
         }
 #pragma unroll
         for (int i = 0; i < NP; ++i) F[i * st] = s[i];
@@ -138,32 +172,60 @@ __global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const 
         const bool fx = i == 0 || i == NP - 1, fy = j == 0 || j == NP - 1, fz = k == 0 || k == NP - 1;
         const int ox = (i == 0 ? 0 : 5 * N2) + j + NP * k, oy = (j == 0 ? 10 * N2 : 15 * N2) + k + NP * i;
         const int oz = (k == 0 ? 20 * N2 : 25 * N2) + i + NP * j;
+        double R[5];
+        ifp::Fast ar;
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
-            double acc = ifp::mul(a.g[0], Fe[v * NN]);
-            acc = acc + ifp::mul(a.g[1], Fe[(5 + v) * NN]);
-            acc = acc + ifp::mul(a.g[2], Fe[(10 + v) * NN]);
-            double R = -acc;
-            if (fx) R = R + (i == 0 ? Le[ox + v * N2] : -Le[ox + v * N2]);
-            if (fy) R = R + (j == 0 ? Le[oy + v * N2] : -Le[oy + v * N2]);
-            if (fz) R = R + (k == 0 ? Le[oz + v * N2] : -Le[oz + v * N2]);
-            const long long ix = ((e0 + el) * 5 + v) * NN + q;
-            double val = R;
-            if (a.mode != 0) {
-                const double y = a.Us[ix] + ifp::mul(dt, R);
-                val = a.first ? y : ifp::mul(a.ca, a.Un[ix]) + ifp::mul(a.cb, y);
-            }
-            a.out[ix] = val;
+            double acc = ar.mul(a.g[0], Fe[v * NN]);
+            acc = acc + ar.mul(a.g[1], Fe[(5 + v) * NN]);
+            acc = acc + ar.mul(a.g[2], Fe[(10 + v) * NN]);
+            R[v] = -acc;
+        }
+        if (!ar.ok)
+            for (int v = 0; v < 5; ++v) R[v] = -scaled_sum_native(a.g, Fe + v * NN, 5 * NN);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+            if (fx) R[v] = R[v] + (i == 0 ? Le[ox + v * N2] : -Le[ox + v * N2]);
+            if (fy) R[v] = R[v] + (j == 0 ? Le[oy + v * N2] : -Le[oy + v * N2]);
+            if (fz) R[v] = R[v] + (k == 0 ? Le[oz + v * N2] : -Le[oz + v * N2]);
+        }
+        const long long ix = (e0 + el) * 5 * NN + q;
+        if (a.mode == 0) {
+#pragma unroll
+            for (int v = 0; v < 5; ++v) a.out[ix + v * NN] = R[v];
+        } else if (a.first) {
+#pragma unroll
+            for (int v = 0; v < 5; ++v) a.out[ix + v * NN] = a.Us[ix + v * NN] + dt * R[v];
+        } else {
+#pragma unroll
+            for (int v = 0; v < 5; ++v)
+                a.out[ix + v * NN] = a.ca * a.Un[ix + v * NN] + a.cb * (a.Us[ix + v * NN] + dt * R[v]);
         }
     }
 }
 
-// w x for a quadrature weight w (prepared factor f of the double fd) and a state value x.
-__device__ __forceinline__ double weighted(const ifp::Factor &f, double fd, double x)
+// Sum of the weighted values of an n x n' set of nodes in FP64 instructions (the rare
+// case of a value out of the integer products' range).
+static __device__ __noinline__ double weighted_sum_native(const double *w, const double *x, int n0, int s0, int n1, int s1)
 {
-    double r = ifp::mul_unsigned_zero(ifp::factor(x), f);
-    if (!ifp::factor_ok(x)) r = ifp::native_mul(fd, x);
-    return r;
+    double s = 0.0;
+    for (int t1 = 0; t1 < n1; ++t1)
+        for (int t0 = 0; t0 < n0; ++t0) s = s + w[t0 + n0 * t1] * x[t0 * s0 + t1 * s1];
+    return s;
+}
+
+// Whether u is an unphysical SR state.
+__device__ __forceinline__ bool node_unphysical(const double u[5])
+{
+    ifp::Fast ar;
+    const double s2 = ar.mul(u[1], u[1]) + ar.mul(u[2], u[2]) + ar.mul(u[3], u[3]);
+    const double tt = ar.mul(u[4], u[4] + 2.0 * u[0]);
+    bool bad = !ar.positive(u[0]) | !ar.positive(u[4]) | !ar.positive(tt) | !(ifp::order_key(s2) < ifp::order_key(tt));
+    if (!ar.ok) {
+        const double w[5] = {u[0], u[1], u[2], u[3], u[4]};
+        bad = sr_unphysical_native(w);
+    }
+    return bad;
 }
 
 // Limiter summaries S[e][v][10] of a.G consecutive elements per CTA: [0] the cell mean
@@ -181,8 +243,8 @@ __device__ __forceinline__ double weighted(const ifp::Factor &f, double fd, doub
 template <int NP>
 struct SumShape {
     static constexpr int NN = NP * NP * NP;
-    static constexpr int G = NP <= 6 ? 6 : 3;  // most elements per CTA (5 G lanes of warp 0)
-    static constexpr int THREADS = 192;
+    static constexpr int G = NP <= 5 ? 6 : NP == 6 ? 4 : 3;  // most elements per CTA (5 G lanes of warp 0)
+    static constexpr int THREADS = NP <= 5 ? 192 : 128;
     // per element: U[5][NN] and plane means [15 NP]; per CTA: weight products
     static constexpr size_t ELEM = sizeof(double) * (5 * NN + 15 * NP);
     static constexpr size_t TAB = (sizeof(double) + sizeof(ifp::Factor)) * (NN + NP * NP) + 8;
@@ -224,13 +286,20 @@ __global__ void __launch_bounds__(SumShape<NP>::THREADS) k_summaries(const __gri
             const int el = i / NN;
             const double *p = sU + (size_t)el * 5 * NN + (i - el * NN);
             const double u[5] = {p[0], p[NN], p[2 * NN], p[3 * NN], p[4 * NN]};
-            if (sr_unphysical(u)) sBad[el] = 1;
+            if (node_unphysical(u)) sBad[el] = 1;
         }
     if (t < 32) {
         for (int r = t; r < ne * 5; r += 32) {
             const double *Uv = sU + (size_t)r * NN;
             double s = 0.0;
-            for (int q = 0; q < NN; ++q) s = s + weighted(sF3[q], sW3[q], Uv[q]);
+            bool ok = true;
+#pragma unroll 4
+            for (int q = 0; q < NN; ++q) {
+                const double x = Uv[q];
+                ok = ok & ifp::factor_ok(x);
+                s = s + ifp::mul_unsigned_zero(ifp::factor(x), sF3[q]);
+            }
+            if (!ok) s = weighted_sum_native(sW3, Uv, NN, 1, 1, 0);
             sMean[r / 5][r % 5] = s * 0.125;
         }
     } else {
@@ -241,10 +310,15 @@ __global__ void __launch_bounds__(SumShape<NP>::THREADS) k_summaries(const __gri
             const int sc = ax == 0 ? N2 : ax == 1 ? 1 : NP;
             const double *Uv = sU + (size_t)(el * 5 + v) * NN + ia * sa;
             double s = 0.0;
+            bool ok = true;
             for (int t1 = 0; t1 < NP; ++t1)
 #pragma unroll
-                for (int t0 = 0; t0 < NP; ++t0)
-                    s = s + weighted(sF2[t0 + NP * t1], sW2[t0 + NP * t1], Uv[t0 * sb + t1 * sc]);
+                for (int t0 = 0; t0 < NP; ++t0) {
+                    const double x = Uv[t0 * sb + t1 * sc];
+                    ok = ok & ifp::factor_ok(x);
+                    s = s + ifp::mul_unsigned_zero(ifp::factor(x), sF2[t0 + NP * t1]);
+                }
+            if (!ok) s = weighted_sum_native(sW2, Uv, NP, sb, NP, sc);
             sQ[((el * 3 + ax) * NP + ia) * 5 + v] = s * 0.25;
         }
     }
@@ -262,7 +336,7 @@ __global__ void __launch_bounds__(SumShape<NP>::THREADS) k_summaries(const __gri
             const double *Q = sQ + (el * 3 + kind - 7) * NP * 5 + v;
             val = 0.0;
 #pragma unroll
-            for (int ia = 0; ia < NP; ++ia) val = val + ifp::mul(a.T.row1[ia], Q[ia * 5]);
+            for (int ia = 0; ia < NP; ++ia) val = val + a.T.row1[ia] * Q[ia * 5];
         }
         a.S[(e0 + el) * 50 + v * 10 + kind] = val;
     }
