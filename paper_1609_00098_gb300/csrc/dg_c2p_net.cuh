@@ -20,13 +20,11 @@ namespace dg {
 
 constexpr int NET_PARAMS = 4481;
 constexpr int OFF_W1 = 0, OFF_B1 = 192, OFF_W2 = 256, OFF_B2 = 4352, OFF_W3 = 4416, OFF_B3 = 4480;
-constexpr int NET_TILE = 128;  // samples per CTA of the standalone kernels, 32 per warp
 constexpr int NET_PARTIAL = NET_PARAMS + 1;  // gradient + loss per CTA
 
 struct NetTileArgs {
     const float *P;              // FP32 parameters
     const __nv_bfloat16 *W2b;    // W2 [j][i] in BF16
-    const __nv_bfloat16 *W2tb;   // W2 transposed [i][j] in BF16
     const double *cons;          // 5 rows of `count`
     const double *p;             // true pressures (training) or nullptr
     double *guess;               // output guesses (inference) or nullptr
@@ -41,12 +39,6 @@ struct NetTileArgs {
 
 __device__ __forceinline__ float silu(float z) { return z * __fdividef(1.0f, 1.0f + __expf(-z)); }
 
-__device__ __forceinline__ float dsilu(float z)
-{
-    const float s = __fdividef(1.0f, 1.0f + __expf(-z));
-    return s * (1.0f + z * (1.0f - s));
-}
-
 __device__ __forceinline__ void mma_bf16(float c[4], const uint32_t a[4], const uint32_t b[2])
 {
     asm volatile(
@@ -54,24 +46,6 @@ __device__ __forceinline__ void mma_bf16(float c[4], const uint32_t a[4], const 
         "{%0,%1,%2,%3};\n"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-// A fragment (16 x 16) of a row-major BF16 matrix M (leading dimension ld) at (r0, c0).
-__device__ __forceinline__ void load_a(uint32_t a[4], const __nv_bfloat16 *M, int ld, int r0, int c0, int lane)
-{
-    const int g = lane >> 2, tq = lane & 3;
-    a[0] = *reinterpret_cast<const uint32_t *>(M + (r0 + g) * ld + c0 + 2 * tq);
-    a[1] = *reinterpret_cast<const uint32_t *>(M + (r0 + g + 8) * ld + c0 + 2 * tq);
-    a[2] = *reinterpret_cast<const uint32_t *>(M + (r0 + g) * ld + c0 + 2 * tq + 8);
-    a[3] = *reinterpret_cast<const uint32_t *>(M + (r0 + g + 8) * ld + c0 + 2 * tq + 8);
-}
-
-// B fragment (16 x 8, k x n) from the row-major transpose Bt[n][k] at (k0, n0).
-__device__ __forceinline__ void load_b(uint32_t b[2], const __nv_bfloat16 *Bt, int ld, int k0, int n0, int lane)
-{
-    const int g = lane >> 2, tq = lane & 3;
-    b[0] = *reinterpret_cast<const uint32_t *>(Bt + (n0 + g) * ld + k0 + 2 * tq);
-    b[1] = *reinterpret_cast<const uint32_t *>(Bt + (n0 + g) * ld + k0 + 2 * tq + 8);
 }
 
 // In-kernel inference evaluates SiLU on halved pre-activations z' = z/2 (the image
