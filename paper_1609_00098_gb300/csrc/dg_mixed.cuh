@@ -288,8 +288,10 @@ __device__ __forceinline__ int sr_con2prim32(float g, const float u[5], float gu
 // step rules of sr_con2prim32 in FP64, stopping when the step is below 2^-40 p or
 // the residual is at the FP64 rounding level of its terms.  That level is
 // reached in a few steps even where tau/(rho eps) is huge, so the cost stays
-// bounded on cold states at the conserved-fix bound.
-__device__ __forceinline__ int sr_polish64(double g, const double u[5], double p0, double Pd[4])
+// bounded on cold states at the conserved-fix bound.  A call of its own: few warps
+// need it, but a warp that does holds its CTA's barrier, so its divisions and roots run
+// on the integer ALU (dg_intfp64.cuh), half the latency of the FP64 sequences.
+static __device__ __noinline__ int sr_polish64(double g, const double *u, double p0, double *Pd)
 {
     const double D = u[0], tau = u[4];
     const double s2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
@@ -298,31 +300,31 @@ __device__ __forceinline__ int sr_polish64(double g, const double u[5], double p
         return 1;
     }
     const double E = tau + D;
-    double plo = fmax(sqrt(s2) - E, 0.0), phi = (g - 1.0) * tau;
+    double plo = fmax(ifp::root(s2) - E, 0.0), phi = (g - 1.0) * tau;
     double p = (p0 >= 0.0) ? fmin(fmax(p0, plo), phi) : phi;
     int status = 2;
     bool lo_moved = false, hi_moved = false;
     for (int it = 0; it < 60; ++it) {
         const double Ep = E + p;
-        const double v2 = s2 / (Ep * Ep);
-        const double W = 1.0 / sqrt(1.0 - v2);
+        const double v2 = ifp::div(s2, Ep * Ep);
+        const double W = ifp::div(1.0, ifp::root(1.0 - v2));
         const double DW = D * W;
-        const double rhoeps = tau - v2 * (Ep - DW / (W + 1.0));
+        const double rhoeps = tau - v2 * (Ep - ifp::div(DW, W + 1.0));
         const double f = p - (g - 1.0) * rhoeps;
-        const double df = 1.0 - (g - 1.0) * v2 * (1.0 - DW / Ep);
+        const double df = 1.0 - (g - 1.0) * v2 * (1.0 - ifp::div(DW, Ep));
         if (fabs(f) <= 0x1p-50 * (p + (g - 1.0) * (tau + v2 * Ep))) { status = 0; break; }
         if (f > 0.0) { phi = p; hi_moved = true; } else { plo = p; lo_moved = true; }
-        double pn = p - f / df;
+        double pn = p - ifp::div(f, df);
         if (!((pn > plo && pn < phi) || (pn == phi && !hi_moved) || (pn == plo && !lo_moved)))
-            pn = phi > 4.0 * plo ? sqrt(fmax(plo, 0x1p-40 * phi) * phi) : 0.5 * (plo + phi);
+            pn = phi > 4.0 * plo ? ifp::root(fmax(plo, 0x1p-40 * phi) * phi) : 0.5 * (plo + phi);
         const double dp = fabs(pn - p);
         p = pn;
         if (dp <= 0x1p-40 * p || !(phi > plo)) { status = 0; break; }
     }
-    const double Ep = E + p;
-    Pd[0] = u[1] / Ep;
-    Pd[1] = u[2] / Ep;
-    Pd[2] = u[3] / Ep;
+    const ifp::Divisor Ep = ifp::divisor(E + p);
+    Pd[0] = ifp::div(u[1], Ep);
+    Pd[1] = ifp::div(u[2], Ep);
+    Pd[2] = ifp::div(u[3], Ep);
     Pd[3] = p;
     return status;
 }
