@@ -543,7 +543,8 @@ __device__ __forceinline__ bool sr_screen32(const float u[5], float d_atm, float
            !(s2 < 0.999f * u[4] * (u[4] + 2.0f * u[0]));
 }
 template <int NP, int SYS, int FLX, int GUESS>
-__global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS) k_stage_mixed(const MixedArgs a)
+__global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS)
+    k_stage_mixed(const __grid_constant__ MixedArgs a)
 {
     constexpr int NN = NP * NP * NP;
     constexpr int TPE = StageShape<NP>::TPE;
@@ -569,13 +570,15 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
 
     const long long ge = (long long)blockIdx.x * a.epb + sub;
     const bool live = sub < a.epb && ge < a.nelem;  // uniform within the element's warps
-    if (t == 0) {
-        sFlag[0] = sFlag[1] = 0;
-        if (live) {
-            const int m = a.slots ? find_slot(a.elem0, a.nslots, ge) : 0;
-            sl = a.slots ? a.slots[m] : a.one;
-            sNb[6] = a.slots ? ge - a.elem0[m] : ge;
-        }
+    if (t == 0) sFlag[0] = sFlag[1] = 0;
+    if (live) {
+        // the slot word by word across the element's threads
+        constexpr int W = (int)(sizeof(MeshSlot) / sizeof(unsigned long long));
+        static_assert(sizeof(MeshSlot) % sizeof(unsigned long long) == 0, "slot words");
+        const int m = a.slots ? find_slot(a.elem0, a.nslots, ge) : 0;
+        const unsigned long long *src = reinterpret_cast<const unsigned long long *>(a.slots ? &a.slots[m] : &a.one);
+        for (int w = t; w < W; w += TPE) reinterpret_cast<unsigned long long *>(&sl)[w] = src[w];
+        if (t == 0) sNb[6] = a.slots ? ge - a.elem0[m] : ge;
     }
     if (GUESS && threadIdx.x == 0) net_bar_init(&sNetBar);
     for (int i = threadIdx.x; i < NP * NP; i += blockDim.x) sD[i] = a.D32[i];
@@ -642,14 +645,13 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
         __syncthreads();  // the guesses are in sFG; the network's regions are dead from here on
     }
 
+    float u[5], P[NPRIM];
     if (own) {
-        float u[5];
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
             u[v] = f64_to_f32(sl.Us[(e * 5 + v) * NN + t]);
             sU[v * NN + t] = u[v];
         }
-        float P[NPRIM];
         const float guess = GUESS ? sFG[t] : (sl.pin ? sl.pin[e * NN + t] : -1.0f);
         if (SYS == 0) {
             ne_primitives32(a.gamma, u, P);
@@ -663,26 +665,27 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
         if (SYS == 1 && sl.pout) sl.pout[e * NN + t] = P[3];
 #pragma unroll
         for (int c = 0; c < NPRIM; ++c) sP[c * NN + t] = P[c];
-#pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
-            float f[5];
-            flux_axis32(u, P, ax, f);
-#pragma unroll
-            for (int v = 0; v < 5; ++v) sF[(ax * 5 + v) * NN + t] = f[v];
-        }
     }
     __syncthreads();
-    // Subtract node 0's flux per axis and variable: D annihilates constants, so
+    // The fluxes less node 0's per axis and variable: D annihilates constants, so
     // the contraction is unchanged in exact arithmetic, and in FP32 its rounding
-    // scales with the flux variation inside the element instead of its size.
-    {
-        float ref[15];
+    // scales with the flux variation inside the element instead of its size.  (Every
+    // thread forms node 0's fluxes itself: read back from shared memory they cost another
+    // barrier and two more passes over the flux arrays.)
+    if (own) {
+        float u0[5], P0[NPRIM];
 #pragma unroll
-        for (int c = 0; c < 15; ++c) ref[c] = sF[c * NN];
-        __syncthreads();
-        if (own)
+        for (int v = 0; v < 5; ++v) u0[v] = sU[v * NN];
 #pragma unroll
-            for (int c = 0; c < 15; ++c) sF[c * NN + t] -= ref[c];
+        for (int c = 0; c < NPRIM; ++c) P0[c] = sP[c * NN];
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            float f[5], r[5];
+            flux_axis32(u, P, ax, f);
+            flux_axis32(u0, P0, ax, r);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) sF[(ax * 5 + v) * NN + t] = f[v] - r[v];
+        }
     }
     __syncthreads();
 
