@@ -735,6 +735,7 @@ dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out)
     st = st ? st : cudaMalloc(&m->err, sizeof(unsigned int));
     if (st == cudaSuccess) st = cudaMemset(m->err, 0, sizeof(unsigned int));
     if (st == cudaSuccess) st = cudaMemset(m->unphys, 0, (size_t)E);
+    if (st == cudaSuccess) st = cudaMemset(m->lam, 0, sizeof(unsigned long long));
     if (st != cudaSuccess) {
         free_scratch(m);
         delete m;
@@ -839,9 +840,8 @@ dg_status dg_compute_dt(dg_mesh *m, const double *U, double cfl, double *dt, voi
     if (!U || !dt) return fail(DG_ERR_ARG, "U and dt must not be NULL");
     if (!(cfl > 0.0)) return fail(DG_ERR_ARG, "cfl must be > 0");
     cudaStream_t s = (cudaStream_t)stream;
-    DG_CUDA(cudaMemsetAsync(m->lam, 0, sizeof(unsigned long long), s));
     DG_CUDA(launch_primitives(m, U, m->P, 0, nullptr, m->lam, s));
-    DG_CUDA(launch_dt(m, cfl, dt, s));
+    DG_CUDA(launch_dt(m, cfl, dt, nullptr, s));
     return DG_OK;
 }
 
@@ -856,14 +856,13 @@ static dg_status rk3_step_ne(dg_mesh *m, double *U, double dt, double cfl, doubl
     const bool lim = m->d.limiter != 0;
     const bool cflmode = cfl > 0.0;
     const double *dtp = cflmode ? m->dt : nullptr;
-    if (cflmode) DG_CUDA(cudaMemsetAsync(m->lam, 0, sizeof(unsigned long long), s));
     const double ct[3] = {0.0, 1.0, 0.5};  // stage times t + ct dt (analytic boundaries)
     for (int st = 0; st < 3; ++st) {
         if (m->gh.mask) DG_LAUNCH(m, s, PROF_OTHER, launch_exterior(m, ct[st], dtp, dt, s));
         NeArgs a = ne_stage_args(m, U, st, lim, cflmode);
         a.one.dt = dt;
         DG_LAUNCH(m, s, PROF_STAGE, launch_ne_stage(m->d.n, m->d.flux, st + 1, a, s));
-        if (st == 0 && cflmode) DG_LAUNCH(m, s, PROF_DT, launch_dt(m, cfl, m->dt, s));
+        if (st == 0 && cflmode) DG_LAUNCH(m, s, PROF_DT, launch_dt(m, cfl, m->dt, dt_used, s));
         NeDecideArgs d = ne_decide_args(m);
         d.one = ne_decide_stage_slot(m, U, st, cflmode, st == 2 ? troubled : nullptr);
         d.one.dt = dt;
@@ -875,10 +874,7 @@ static dg_status rk3_step_ne(dg_mesh *m, double *U, double dt, double cfl, doubl
         }
     }
     if (m->gh.mask) DG_LAUNCH(m, s, PROF_OTHER, launch_time_add(m->t, dtp, dt, s));
-    if (dt_used) {
-        if (cflmode) DG_CUDA(cudaMemcpyAsync(dt_used, m->dt, sizeof(double), cudaMemcpyDeviceToDevice, s));
-        else DG_CUDA(launch_set(dt_used, dt, s));
-    }
+    if (dt_used && !cflmode) DG_CUDA(launch_set(dt_used, dt, s));
     return DG_OK;
 }
 
@@ -906,7 +902,6 @@ static dg_status rk3_step_mixed(dg_mesh *m, double *U, double dt, double cfl, do
     a.mode = 1;
     float *latest = (carry && m->p_valid) ? m->pbuf[m->pi] : nullptr;
     if (cflmode) {
-        DG_CUDA(cudaMemsetAsync(m->lam, 0, sizeof(unsigned long long), s));
         DG_LAUNCH(m, s, PROF_PRIM,
                   launch_cfl_mixed(m, U, latest, carry ? m->pbuf[1 - m->pi] : nullptr, pgiven ? m->pfull : nullptr,
                                    m->kappa_sw, s));
@@ -914,7 +909,7 @@ static dg_status rk3_step_mixed(dg_mesh *m, double *U, double dt, double cfl, do
             m->pi = 1 - m->pi;
             latest = m->pbuf[m->pi];
         }
-        DG_LAUNCH(m, s, PROF_DT, launch_dt(m, cfl, m->dt, s));
+        DG_LAUNCH(m, s, PROF_DT, launch_dt(m, cfl, m->dt, dt_used, s));
     }
     double *ins[3] = {U, m->W1, m->W2};
     double *outs[3] = {m->W1, m->W2, U};
@@ -950,10 +945,7 @@ static dg_status rk3_step_mixed(dg_mesh *m, double *U, double dt, double cfl, do
     }
     m->p_valid = carry ? 1 : 0;
     if (m->gh.mask) DG_LAUNCH(m, s, PROF_OTHER, launch_time_add(m->t, a.one.dt_ptr, dt, s));
-    if (dt_used) {
-        if (cflmode) DG_CUDA(cudaMemcpyAsync(dt_used, m->dt, sizeof(double), cudaMemcpyDeviceToDevice, s));
-        else DG_CUDA(launch_set(dt_used, dt, s));
-    }
+    if (dt_used && !cflmode) DG_CUDA(launch_set(dt_used, dt, s));
     return DG_OK;
 }
 
@@ -977,7 +969,6 @@ dg_status dg_rk3_step(dg_mesh *m, double *U, double dt, double cfl, double *dt_u
     a.mode = 1;
     a.dt = dt;
     a.dt_ptr = cflmode ? m->dt : nullptr;
-    if (cflmode) DG_CUDA(cudaMemsetAsync(m->lam, 0, sizeof(unsigned long long), s));
 
     double *ins[3] = {U, m->W1, m->W2};
     double *outs[3] = {m->W1, m->W2, U};
@@ -988,7 +979,7 @@ dg_status dg_rk3_step(dg_mesh *m, double *U, double dt, double cfl, double *dt_u
         // the SR fix of the previous stage's result is fused into its primitive pass
         DG_LAUNCH(m, s, PROF_PRIM,
                   launch_primitives(m, ins[st], m->P, sr && st > 0, ins[st], (cflmode && st == 0) ? m->lam : nullptr, s));
-        if (cflmode && st == 0) DG_LAUNCH(m, s, PROF_DT, launch_dt(m, cfl, m->dt, s));
+        if (cflmode && st == 0) DG_LAUNCH(m, s, PROF_DT, launch_dt(m, cfl, m->dt, dt_used, s));
         if (m->gh.mask) DG_LAUNCH(m, s, PROF_OTHER, launch_exterior(m, ct[st], a.dt_ptr, dt, s));
         a.Us = ins[st];
         a.Un = U;
@@ -1008,10 +999,7 @@ dg_status dg_rk3_step(dg_mesh *m, double *U, double dt, double cfl, double *dt_u
     }
     if (sr) DG_LAUNCH(m, s, PROF_FIX, launch_fix(m, U, s));
     if (m->gh.mask) DG_LAUNCH(m, s, PROF_OTHER, launch_time_add(m->t, a.dt_ptr, dt, s));
-    if (dt_used) {
-        if (cflmode) DG_CUDA(cudaMemcpyAsync(dt_used, m->dt, sizeof(double), cudaMemcpyDeviceToDevice, s));
-        else DG_CUDA(launch_set(dt_used, dt, s));
-    }
+    if (dt_used && !cflmode) DG_CUDA(launch_set(dt_used, dt, s));
     return DG_OK;
 }
 

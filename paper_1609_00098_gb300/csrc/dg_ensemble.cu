@@ -35,19 +35,15 @@ struct DtSlot {
     double dxmin;
 };
 
-__global__ void k_lam_zero(const DtSlot *slots, int count)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) *slots[i].lam = 0ull;
-}
-
 // dt = C dx_min / lambda_max per mesh (Sec. 3.4), the same operations as k_dt.
 __global__ void k_dt_batch(const DtSlot *slots, int count, double cfl)
 {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
     const double l = __longlong_as_double((long long)*slots[i].lam);
     *slots[i].dt = cfl * slots[i].dxmin / l;
+    *slots[i].lam = 0ull;  // ready for the next maximum, as k_dt leaves it
 }
 
 __global__ void k_dt_gather(const DtSlot *slots, int count, double *out)
@@ -319,8 +315,7 @@ cudaError_t group_stage(EnsGroup &g, bool first, int st, cudaStream_t s)
     return e;
 }
 
-// One step of the ensemble: the per-mesh lambda reset, every group's pre-dt
-// phase, the batched dt, every group's stages, all on s, stage by stage across
+// One step of the ensemble: every group's pre-dt phase, the batched dt, every group's stages, all on s, stage by stage across
 // the groups.  concurrent: each group's phase runs on its own stream instead,
 // forked from and joined back to s by events (in a captured graph: parallel
 // branches), so that the groups' launches overlap.  Both orders give the same
@@ -332,8 +327,7 @@ cudaError_t launch_step(dg_ensemble *en, double cfl, bool first, bool concurrent
     const int count = (int)en->meshes.size();
     const unsigned blocks = (unsigned)((count + 127) / 128);
     const int G = (int)en->groups.size();
-    k_lam_zero<<<blocks, 128, 0, s>>>(en->d_dt, count);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaSuccess;
     auto fan_out = [&](auto &&body) -> cudaError_t {
         cudaError_t r = cudaEventRecord(en->fork, s);
         for (int i = 0; i < G && r == cudaSuccess; ++i) {
@@ -352,8 +346,7 @@ cudaError_t launch_step(dg_ensemble *en, double cfl, bool first, bool concurrent
         }
     }
     if (e != cudaSuccess) return e;
-    k_dt_batch<<<blocks, 128, 0, s>>>(en->d_dt, count, cfl);
-    e = cudaGetLastError();
+    e = launch_pdl(k_dt_batch, blocks, 128, 0, s, en->d_dt, count, cfl);
     if (e != cudaSuccess) return e;
     if (concurrent)
         return fan_out([&](EnsGroup &g, cudaStream_t b) {

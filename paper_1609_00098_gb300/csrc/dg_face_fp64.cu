@@ -23,6 +23,7 @@ constexpr int kFaceThreads = 128;
 template <int SYS, int FLX>
 __global__ void __launch_bounds__(kFaceThreads) k_face_fp64(const __grid_constant__ FaceArgs a)
 {
+    pdl_wait();
     const int n = a.n, n2 = n * n, nn = n2 * n;
     const long long total = (3 * a.E + a.nghost) * n2;
     for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < total;
@@ -99,12 +100,13 @@ cudaError_t launch_face_fp64(int system, int flux, const FaceArgs &a, cudaStream
     const long long total = (3 * a.E + a.nghost) * a.n * a.n;
     const long long blocks = (total + kFaceThreads - 1) / kFaceThreads;
     const unsigned grid = (unsigned)(blocks < 0x7fffffffLL ? blocks : 0x7fffffffLL);
-    if (system == 0 && flux == 2) k_face_fp64<0, 2><<<grid, kFaceThreads, 0, s>>>(a);
-    else if (system == 0 && flux == 0) k_face_fp64<0, 0><<<grid, kFaceThreads, 0, s>>>(a);
-    else if (system == 0) k_face_fp64<0, 1><<<grid, kFaceThreads, 0, s>>>(a);
-    else if (flux == 0) k_face_fp64<1, 0><<<grid, kFaceThreads, 0, s>>>(a);
-    else k_face_fp64<1, 1><<<grid, kFaceThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    void (*kern)(const FaceArgs);
+    if (system == 0 && flux == 2) kern = k_face_fp64<0, 2>;
+    else if (system == 0 && flux == 0) kern = k_face_fp64<0, 0>;
+    else if (system == 0) kern = k_face_fp64<0, 1>;
+    else if (flux == 0) kern = k_face_fp64<1, 0>;
+    else kern = k_face_fp64<1, 1>;
+    return launch_pdl(kern, grid, kFaceThreads, 0, s, a);
 }
 
 }  // namespace dg

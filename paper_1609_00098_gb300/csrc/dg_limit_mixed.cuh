@@ -47,6 +47,7 @@ constexpr int kLimitWarps = 4;
 template <int NP, int SYS>
 __global__ void __launch_bounds__(32 * kLimitWarps) k_limit_mixed(const LimitMixedArgs a)
 {
+    pdl_wait();
     constexpr int NN = NP * NP * NP;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -168,9 +169,7 @@ cudaError_t launch_limit_mixed_np(int system, const LimitMixedArgs &a, cudaStrea
 {
     if (a.E <= 0) return cudaSuccess;
     const unsigned grid = (unsigned)((a.E + kLimitWarps - 1) / kLimitWarps);  // one warp per element
-    if (system == 0) k_limit_mixed<NP, 0><<<grid, 32 * kLimitWarps, 0, s>>>(a);
-    else k_limit_mixed<NP, 1><<<grid, 32 * kLimitWarps, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(system == 0 ? k_limit_mixed<NP, 0> : k_limit_mixed<NP, 1>, grid, 32 * kLimitWarps, 0, s, a);
 }
 
 }  // namespace dg

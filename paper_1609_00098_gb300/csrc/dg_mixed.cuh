@@ -546,6 +546,7 @@ template <int NP, int SYS, int FLX, int GUESS>
 __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS)
     k_stage_mixed(const __grid_constant__ MixedArgs a)
 {
+    pdl_wait();
     constexpr int NN = NP * NP * NP;
     constexpr int TPE = StageShape<NP>::TPE;
     using SM = MixedSmem<NP>;
@@ -980,8 +981,7 @@ cudaError_t launch_stage_mixed_np(int system, int flux, const MixedArgs &a, cuda
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (err != cudaSuccess) return err;
     }
-    kern<<<grid, block, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(kern, grid, block, smem, s, a);
 }
 
 // Largest elements-per-CTA of the stage kernel for n nodes per axis.

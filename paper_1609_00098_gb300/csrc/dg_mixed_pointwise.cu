@@ -26,6 +26,7 @@ struct CflNetSmem {
 template <int SYS, int GUESS>
 __global__ void __launch_bounds__(kThreads, 4) k_cfl_mixed(const CflArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char cfl_smem[];
     CflNetSmem &N = *reinterpret_cast<CflNetSmem *>(cfl_smem);
     __shared__ uint64_t bar;  // completion of the network weights' bulk copy
@@ -122,18 +123,17 @@ cudaError_t launch_cfl_batch(int system, const CflArgs &a, long long nchunks, cu
     if (nchunks <= 0) return cudaSuccess;
     const unsigned grid = (unsigned)nchunks;
     if (system == 0) {
-        k_cfl_mixed<0, 0><<<grid, kThreads, 0, s>>>(a);
+        return launch_pdl(k_cfl_mixed<0, 0>, grid, kThreads, 0, s, a);
     } else if (a.netImg == nullptr) {
-        k_cfl_mixed<1, 0><<<grid, kThreads, 0, s>>>(a);
+        return launch_pdl(k_cfl_mixed<1, 0>, grid, kThreads, 0, s, a);
     } else {
         const size_t smem = sizeof(CflNetSmem);
         if (smem > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(k_cfl_mixed<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        k_cfl_mixed<1, 1><<<grid, kThreads, smem, s>>>(a);
+        return launch_pdl(k_cfl_mixed<1, 1>, grid, kThreads, smem, s, a);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_cfl_mixed(const dg_mesh *m, const double *Un, const float *pin, float *pout, float *Pout,

@@ -479,6 +479,7 @@ __device__ __forceinline__ float ne_final_sum(const NeArgs &a, int kind, Q q)
 template <int NP, int FLX, int ST>
 __global__ void __launch_bounds__(NeShape<NP>::THREADS, NeShape<NP>::MINB) k_ne_stage(const __grid_constant__ NeArgs a)
 {
+    pdl_wait();
     using SH = NeShape<NP>;
     constexpr int L = SH::L, NN = SH::NN, EPB = SH::EPB, N1 = NP - 1;
     extern __shared__ __align__(16) float ne_smem[];
@@ -1148,6 +1149,7 @@ __global__ void __launch_bounds__(NeShape<NP>::THREADS, NeShape<NP>::MINB) k_ne_
 template <int NP, int FINAL>
 __global__ void __launch_bounds__(128) k_ne_decide(const __grid_constant__ NeDecideArgs a)
 {
+    pdl_wait();
     constexpr int NN = NP * NP * NP;
     __shared__ float sx[MAXN];  // LGL nodes, for the final pass's per-lane coordinates
     if (FINAL) {
@@ -1287,8 +1289,7 @@ cudaError_t launch_ne_stage_np(int flux, int stage, const NeArgs &a, cudaStream_
     // static + dynamic shared memory exceed 48 KB for every n: opt in
     const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM);
     if (err != cudaSuccess) return err;
-    kern<<<grid, SH::THREADS, SH::SMEM, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(kern, grid, SH::THREADS, SH::SMEM, s, a);
 }
 
 template <int NP>
@@ -1296,9 +1297,7 @@ cudaError_t launch_ne_decide_np(int final_pass, const NeDecideArgs &a, cudaStrea
 {
     if (a.nelem <= 0) return cudaSuccess;
     const unsigned grid = (unsigned)((a.nelem + 7) / 8);  // 8 elements per 128-thread CTA
-    if (final_pass) k_ne_decide<NP, 1><<<grid, 128, 0, s>>>(a);
-    else k_ne_decide<NP, 0><<<grid, 128, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(final_pass ? k_ne_decide<NP, 1> : k_ne_decide<NP, 0>, grid, 128, 0, s, a);
 }
 
 }  // namespace dg

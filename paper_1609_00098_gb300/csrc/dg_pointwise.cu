@@ -49,6 +49,7 @@ __device__ __forceinline__ void block_max(double lmax, unsigned long long *lam)
 // the largest wave speed into *lam.
 __global__ void __launch_bounds__(kThreads) k_primitives_ne(const PrimArgs a)
 {
+    pdl_wait();
     double lmax = 0.0;
     for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < a.total;
          g += (long long)gridDim.x * blockDim.x) {
@@ -122,6 +123,7 @@ struct PrimIO {
 
 __global__ void __launch_bounds__(kC2pThreads, 5) k_primitives_sr(const PrimArgs a)
 {
+    pdl_wait();
     __shared__ C2pWarp Q[kC2pThreads / 32];
     PrimIO io{a, 0.0, 0u};
     const long long warp = ((long long)blockIdx.x * kC2pThreads + threadIdx.x) >> 5;
@@ -132,6 +134,7 @@ __global__ void __launch_bounds__(kC2pThreads, 5) k_primitives_sr(const PrimArgs
 
 __global__ void __launch_bounds__(kThreads) k_fix(double *U, long long total, int nn, double d_atm, double tau_atm)
 {
+    pdl_wait();
     for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < total;
          g += (long long)gridDim.x * blockDim.x) {
         const long long e = g / nn;
@@ -155,6 +158,7 @@ template <int NP>
 __global__ void __launch_bounds__(256) k_mrs_prepare(const double *U, const double *S, double *T, long long E,
                                                      double g)
 {
+    pdl_wait();
     constexpr int NN = NP * NP * NP;
     const long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -207,6 +211,7 @@ template <int NP>
 __global__ void __launch_bounds__(256) k_mrs_limit(double *U, const double *T, unsigned char *troubled, long long E,
                                                    int K0, int K1, int K2, double wid)
 {
+    pdl_wait();
     constexpr int NN = NP * NP * NP;
     const long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -252,6 +257,7 @@ __global__ void __launch_bounds__(kThreads) k_exterior(double *gU, double *gP, G
                                                      double b5, const double *t, double ct, const double *dt_ptr,
                                                      double dt_val)
 {
+    pdl_wait();
     const double pi = 3.14159265358979323846;
     const int nf = n * n, nn = n * n * n;
     const int K[3] = {K0, K1, K2};
@@ -313,6 +319,7 @@ __global__ void __launch_bounds__(kThreads) k_exterior(double *gU, double *gP, G
 
 __global__ void k_time_add(double *t, const double *dt_ptr, double dt)
 {
+    pdl_wait();
     if (threadIdx.x == 0 && blockIdx.x == 0) *t = *t + (dt_ptr ? *dt_ptr : dt);
 }
 
@@ -321,15 +328,20 @@ __global__ void k_time_add(double *t, const double *dt_ptr, double dt)
 __global__ void __launch_bounds__(kThreads) k_ab3(double *U, const double *L0, const double *L1, const double *L2,
                                                   double dt, double c0, double c1, double c2, long long count)
 {
+    pdl_wait();
     for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < count;
          g += (long long)gridDim.x * blockDim.x)
         U[g] = U[g] + dt * ((c0 * L0[g] - c1 * L1[g]) + c2 * L2[g]);
 }
 
-__global__ void k_dt(const unsigned long long *lam, double cfl, double dxmin, double *dt)
+__global__ void k_dt(unsigned long long *lam, double cfl, double dxmin, double *dt, double *dt_used)
 {
+    pdl_wait();
     const double l = __longlong_as_double((long long)*lam);
-    *dt = cfl * dxmin / l;
+    const double h = cfl * dxmin / l;
+    *dt = h;
+    if (dt_used) *dt_used = h;
+    *lam = 0ull;  // ready for the next maximum
 }
 
 __global__ void __launch_bounds__(kThreads) k_coords(double *xyz, long long total, int n, int K0, int K1,
@@ -435,14 +447,17 @@ __global__ void __launch_bounds__(kC2pThreads, 5) k_con2prim(RowsIO io, double g
     c2p_warp(io, Q[threadIdx.x >> 5], gamma, io.count, warp, (long long)gridDim.x * (kC2pThreads / 32));
 }
 
-__global__ void k_set(double *p, double v) { *p = v; }
+__global__ void k_set(double *p, double v)
+{
+    pdl_wait();
+    *p = v;
+}
 
 }  // namespace
 
 cudaError_t launch_set(double *p, double v, cudaStream_t s)
 {
-    k_set<<<1, 1, 0, s>>>(p, v);
-    return cudaGetLastError();
+    return launch_pdl(k_set, 1, 1, 0, s, p, v);
 }
 
 cudaError_t launch_primitives(const dg_mesh *m, const double *U, double *P, int fix, double *Ufix,
@@ -459,28 +474,26 @@ cudaError_t launch_primitives(const dg_mesh *m, const double *U, double *P, int 
     a.gamma = m->d.gamma;
     a.d_atm = m->d.d_atm;
     a.tau_atm = m->d.tau_atm;
-    if (m->d.system == 0) k_primitives_ne<<<grid_for(a.total, kThreads), kThreads, 0, s>>>(a);
-    else k_primitives_sr<<<c2p_grid(a.total), kC2pThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    return m->d.system == 0 ? launch_pdl(k_primitives_ne, grid_for(a.total, kThreads), kThreads, 0, s, a)
+                            : launch_pdl(k_primitives_sr, c2p_grid(a.total), kC2pThreads, 0, s, a);
 }
 
 cudaError_t launch_fix(const dg_mesh *m, double *U, cudaStream_t s)
 {
     const long long total = m->E * m->nn;
-    k_fix<<<grid_for(total, kThreads), kThreads, 0, s>>>(U, total, m->nn, m->d.d_atm, m->d.tau_atm);
-    return cudaGetLastError();
+    return launch_pdl(k_fix, grid_for(total, kThreads), kThreads, 0, s, U, total, m->nn, m->d.d_atm, m->d.tau_atm);
 }
 
 template <int NP>
 cudaError_t launch_mrs_np(const dg_mesh *m, double *U, unsigned char *troubled, cudaStream_t s)
 {
     const unsigned grid = (unsigned)((m->E * 32 + 255) / 256);
-    k_mrs_prepare<NP><<<grid, 256, 0, s>>>(U, m->S, m->mrsT, m->E, m->d.gamma);
+    const cudaError_t e = launch_pdl(k_mrs_prepare<NP>, grid, 256, 0, s, U, m->S, m->mrsT, m->E, m->d.gamma);
+    if (e != cudaSuccess) return e;
     double h = 0.0;
     for (int a = 0; a < 3; ++a) h = fmax(h, m->dx[a]);
     const double wid = m->d.mrs_alpha * h * sqrt(h);
-    k_mrs_limit<NP><<<grid, 256, 0, s>>>(U, m->mrsT, troubled, m->E, m->d.K[0], m->d.K[1], m->d.K[2], wid);
-    return cudaGetLastError();
+    return launch_pdl(k_mrs_limit<NP>, grid, 256, 0, s, U, m->mrsT, troubled, m->E, m->d.K[0], m->d.K[1], m->d.K[2], wid);
 }
 
 // MRS pass over a state whose summaries S are current (the stage kernel's, or
@@ -504,31 +517,28 @@ cudaError_t launch_exterior(const dg_mesh *m, double ct, const double *dt_ptr, d
     if (!m->gh.mask) return cudaSuccess;
     const long long total = m->nghost * m->d.n * m->d.n;
     const double *b = m->d.exact_par;
-    k_exterior<<<grid_for(total, kThreads), kThreads, 0, s>>>(
+    return launch_pdl(
+        k_exterior, grid_for(total, kThreads), kThreads, 0, s,
         const_cast<double *>(m->gh.U), const_cast<double *>(m->gh.P), m->gh, total, m->d.n, m->d.K[0], m->d.K[1],
         m->d.K[2], m->d.lo[0], m->d.lo[1], m->d.lo[2], m->dx[0], m->dx[1], m->dx[2], m->T, m->d.gamma, b[0], b[1],
         b[2], b[3], b[4], b[5], m->t, ct, dt_ptr, dt);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_time_add(double *t, const double *dt_ptr, double dt, cudaStream_t s)
 {
-    k_time_add<<<1, 32, 0, s>>>(t, dt_ptr, dt);
-    return cudaGetLastError();
+    return launch_pdl(k_time_add, 1, 32, 0, s, t, dt_ptr, dt);
 }
 
 cudaError_t launch_ab3_combine(double *U, const double *L0, const double *L1, const double *L2, double dt,
                                long long count, cudaStream_t s)
 {
-    k_ab3<<<grid_for(count, kThreads), kThreads, 0, s>>>(U, L0, L1, L2, dt, 23.0 / 12.0, 16.0 / 12.0, 5.0 / 12.0,
-                                                         count);
-    return cudaGetLastError();
+    return launch_pdl(k_ab3, grid_for(count, kThreads), kThreads, 0, s, U, L0, L1, L2, dt, 23.0 / 12.0, 16.0 / 12.0,
+                      5.0 / 12.0, count);
 }
 
-cudaError_t launch_dt(const dg_mesh *m, double cfl, double *dt, cudaStream_t s)
+cudaError_t launch_dt(const dg_mesh *m, double cfl, double *dt, double *dt_used, cudaStream_t s)
 {
-    k_dt<<<1, 1, 0, s>>>(m->lam, cfl, m->dxmin, dt);
-    return cudaGetLastError();
+    return launch_pdl(k_dt, 1, 1, 0, s, m->lam, cfl, m->dxmin, dt, dt_used);
 }
 
 cudaError_t launch_coords(const dg_mesh *m, double *xyz, cudaStream_t s)

@@ -78,6 +78,7 @@ static __device__ __noinline__ void line_native(const double *D, double *F, int 
 template <int NP>
 __global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const __grid_constant__ StageArgs a)
 {
+    pdl_wait();
     using SH = StageShape64<NP>;
     constexpr int NN = SH::NN, N2 = SH::N2, EPB = SH::EPB;
     extern __shared__ double smem_stage[];
@@ -254,6 +255,7 @@ struct SumShape {
 template <int NP>
 __global__ void __launch_bounds__(SumShape<NP>::THREADS) k_summaries(const __grid_constant__ SummaryArgs a)
 {
+    pdl_wait();
     constexpr int NN = NP * NP * NP, N2 = NP * NP;
     extern __shared__ double smem_sum[];
     const int G = a.G, t = threadIdx.x;
@@ -354,6 +356,7 @@ __global__ void __launch_bounds__(SumShape<NP>::THREADS) k_summaries(const __gri
 template <int NP>
 __global__ void __launch_bounds__(128) k_limit(const __grid_constant__ LimitArgs a)
 {
+    pdl_wait();
     constexpr int NN = NP * NP * NP, N2 = NP * NP;
     __shared__ double sSl[4][32], sM0[4][32];  // per warp: slopes and means by lane
     __shared__ double sP[4][15 * NP];          // [v][ax][i] slope terms
@@ -423,8 +426,7 @@ cudaError_t launch_stage_np(const StageArgs &args, cudaStream_t s)
             cudaFuncSetAttribute(k_stage_fp64<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM);
         if (err != cudaSuccess) return err;
     }
-    k_stage_fp64<NP><<<(unsigned)((a.E + SH::EPB - 1) / SH::EPB), SH::THREADS, SH::SMEM, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k_stage_fp64<NP>, (unsigned)((a.E + SH::EPB - 1) / SH::EPB), SH::THREADS, SH::SMEM, s, a);
 }
 
 template <int NP>
@@ -440,15 +442,13 @@ cudaError_t launch_summaries_np(const SummaryArgs &args, cudaStream_t s)
             cudaFuncSetAttribute(k_summaries<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (err != cudaSuccess) return err;
     }
-    k_summaries<NP><<<(unsigned)((a.E + a.G - 1) / a.G), SumShape<NP>::THREADS, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k_summaries<NP>, (unsigned)((a.E + a.G - 1) / a.G), SumShape<NP>::THREADS, smem, s, a);
 }
 
 template <int NP>
 cudaError_t launch_limit_np(const LimitArgs &a, cudaStream_t s)
 {
-    k_limit<NP><<<(unsigned)((a.E + 7) / 8), 128, 0, s>>>(a);  // 8 elements per CTA
-    return cudaGetLastError();
+    return launch_pdl(k_limit<NP>, (unsigned)((a.E + 7) / 8), 128, 0, s, a);  // 8 elements per CTA
 }
 
 }  // namespace dg
