@@ -597,6 +597,12 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
     const bool own = live && t < NN;  // this thread holds node t of a live element
     unsigned errs = 0;
 
+    // the node's own state, on its way while the face nodes load
+    double uw[5];
+    if (own)
+#pragma unroll
+        for (int v = 0; v < 5; ++v) uw[v] = sl.Us[(e * 5 + v) * NN + t];
+
     // Neighbour face nodes of all three axes (point f = 2 NP^2 ax + NP^2 side + rem):
     // their FP32 states and guesses, staged first so that the loads overlap the
     // network's phase and the element's own loads.
@@ -631,7 +637,7 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
             float u[5] = {1.0f, 0.0f, 0.0f, 0.0f, 1.0f};
             if (own)
 #pragma unroll
-                for (int v = 0; v < 5; ++v) u[v] = f64_to_f32(sl.Us[(e * 5 + v) * NN + t]);
+                for (int v = 0; v < 5; ++v) u[v] = f64_to_f32(uw[v]);
             net_features(u, a.net_sc, reinterpret_cast<float(*)[6]>(smem_mixed + SM::feat(a.epb, sub))[t]);
         }
         if (!net_copy_wait(&sNetBar, NET_COPY_POLLS)) {
@@ -650,7 +656,7 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
     if (own) {
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
-            u[v] = f64_to_f32(sl.Us[(e * 5 + v) * NN + t]);
+            u[v] = f64_to_f32(uw[v]);
             sU[v * NN + t] = u[v];
         }
         const float guess = GUESS ? sFG[t] : (sl.pin ? sl.pin[e * NN + t] : -1.0f);
@@ -842,6 +848,15 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
         acc[(1 + c) * NN] = o[3];
         acc[4 * NN] = o[4];
     }
+    // the update's FP64 states, on their way while the CTA meets
+    double us[5], un[5];
+    if (own && a.mode != 0) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) us[v] = sl.Us[(e * 5 + v) * NN + t];
+        if (!a.first)
+#pragma unroll
+            for (int v = 0; v < 5; ++v) un[v] = sl.Un[(e * 5 + v) * NN + t];
+    }
     __syncthreads();
     if (own) {
         const int i = t % NP, j = (t / NP) % NP, k = t / (NP * NP);
@@ -870,15 +885,14 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
                 sl.out[ix] = f32_to_f64(R);
                 continue;
             }
-            const double us = sl.Us[ix];
             float inc;
             if (a.first) {
                 inc = dt * R;
             } else {
-                const float dn = f64_to_f32(sl.Un[ix] - us);
+                const float dn = f64_to_f32(un[v] - us[v]);
                 inc = a.ca * dn + a.cb * (dt * R);
             }
-            val[v] = us + f32_to_f64(inc);
+            val[v] = us[v] + f32_to_f64(inc);
         }
     }
     if (a.mode == 0) return;
