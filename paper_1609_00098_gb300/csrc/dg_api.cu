@@ -503,7 +503,7 @@ LimitSlot limit_slot(const dg_mesh *m, double *U, unsigned char *troubled)
         l.tvb[ax] = m->d.tvb_M * m->dx[ax] * m->dx[ax];
         l.inv_dx[ax] = 1.0 / m->dx[ax];
         l.beta_dx[ax] = m->d.beta / m->dx[ax];
-        l.hdx[ax] = 0.5 * m->dx[ax];
+        for (int i = 0; i < m->d.n; ++i) l.hx[ax][i] = 0.5 * m->dx[ax] * m->T.x[i];
     }
     return l;
 }
@@ -518,7 +518,6 @@ LimitMixedArgs limit_mixed_args(const dg_mesh *m, double *U, unsigned char *trou
     l.limiter = m->d.limiter;
     l.d_atm = m->d.d_atm;
     l.tau_atm = m->d.tau_atm;
-    for (int i = 0; i < MAXN; ++i) l.x[i] = m->T.x[i];
     return l;
 }
 

@@ -25,7 +25,7 @@ struct LimitSlot {
     double tvb[3];          // M dx_a^2
     double inv_dx[3];       // 1 / dx_a
     double beta_dx[3];      // beta / dx_a
-    double hdx[3];          // dx_a / 2
+    double hx[3][MAXN];     // (dx_a / 2) x_i, x_i the LGL nodes
 };
 
 struct LimitMixedArgs {
@@ -36,7 +36,6 @@ struct LimitMixedArgs {
     long long E;            // elements in the launch
     int limiter;
     double d_atm, tau_atm;
-    double x[MAXN];         // LGL nodes
 };
 
 // Warps (elements) per CTA of the limiter: small CTAs spread a one-wave launch
@@ -45,7 +44,7 @@ struct LimitMixedArgs {
 constexpr int kLimitWarps = 4;
 
 template <int NP, int SYS>
-__global__ void __launch_bounds__(32 * kLimitWarps) k_limit_mixed(const LimitMixedArgs a)
+__global__ void __launch_bounds__(32 * kLimitWarps) k_limit_mixed(const __grid_constant__ LimitMixedArgs a)
 {
     pdl_wait();
     constexpr int NN = NP * NP * NP;
@@ -106,11 +105,11 @@ __global__ void __launch_bounds__(32 * kLimitWarps) k_limit_mixed(const LimitMix
             s1[v] = __shfl_sync(0xffffffffu, slope, 3 * v + 1);
         }
         for (int ij = lane; ij < NP * NP; ij += 32) {
-            const double h0 = sl.hdx[0] * a.x[ij % NP], h1 = sl.hdx[1] * a.x[ij / NP];
+            const double h0 = sl.hx[0][ij % NP], h1 = sl.hx[1][ij / NP];
 #pragma unroll
             for (int v = 0; v < 5; ++v) sAB[wl][v][ij] = fma(s1[v], h1, fma(s0[v], h0, m0[v]));
         }
-        if (lane < NP) sH2[wl][lane] = sl.hdx[2] * a.x[lane];
+        if (lane < NP) sH2[wl][lane] = sl.hx[2][lane];
         __syncwarp();
     }
     // Node values: the replacement of the limited variables, else the stage state.
@@ -156,7 +155,7 @@ __global__ void __launch_bounds__(32 * kLimitWarps) k_limit_mixed(const LimitMix
             const int q = sFix[wl][r];
             double u[5];
             node(q, u);
-            const unsigned nm = mask | sr_fix(a.d_atm, a.tau_atm, u);
+            const unsigned nm = mask | sr_fix_call(a.d_atm, a.tau_atm, u);
 #pragma unroll
             for (int v = 0; v < 5; ++v)
                 if (nm & (1u << v)) sl.U[(e * 5 + v) * NN + q] = u[v];

@@ -453,7 +453,7 @@ __device__ __forceinline__ unsigned sr_prims_mixed(float g, double gd, float kap
     if (st64 != 0) {
         // unphysical in FP32 or in FP64: recover from the fixed FP64 state,
         // starting from the previous pass's pressure
-        sr_fix(d_atm, tau_atm, u64);
+        sr_fix_native(d_atm, tau_atm, u64);  // (as a call; the integer-ALU form takes longer for so few lanes)
         st64 = sr_polish64(gd, u64, guess >= 0.0f ? f32_to_f64(guess) : -1.0, Pd);
     }
 #pragma unroll
@@ -907,7 +907,10 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
                 bad = c & 1u;
                 needfix = c & 2u;
             } else {
-                sr_fix(a.d_atm, a.tau_atm, val);
+                double w[5] = {val[0], val[1], val[2], val[3], val[4]};
+                sr_fix_call(a.d_atm, a.tau_atm, w);
+#pragma unroll
+                for (int v = 0; v < 5; ++v) val[v] = w[v];
             }
         }
     }
@@ -945,32 +948,31 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
     }
     __syncthreads();
     for (int id = t; live && id < 15 * NP; id += TPE) {
+        // one path for the three axes (an FP64 instruction costs the same for a part of a
+        // warp): x and z sum over t1; y over k the z sums of row ia in plane k
         const int ax = id / (5 * NP), ia = (id / 5) % NP, v = id % 5;
+        const int base = ax == 0 ? ia * NP : ax == 1 ? 2 * NP * NP + ia : (2 * NP + ia) * NP, st = ax == 1 ? NP : 1;
         double q = 0.0;
-        if (ax == 1)
-            for (int k = 0; k < NP; ++k) q = fma(sW64[k], sPart[((2 * NP + k) * NP + ia) * 5 + v], q);
-        else
-            for (int t1 = 0; t1 < NP; ++t1) q = fma(sW64[t1], sPart[((ax * NP + ia) * NP + t1) * 5 + v], q);
-        sQ[(ax * NP + ia) * 5 + v] = q;
+#pragma unroll
+        for (int t1 = 0; t1 < NP; ++t1) q = fma(sW64[t1], sPart[(base + t1 * st) * 5 + v], q);
+        sQ[id] = q;
     }
     __syncthreads();
-    for (int id = t; live && id < 50; id += TPE) {
-        const int v = id / 10, kind = id % 10;
+    for (int id = t; live && id < 50; id += TPE) {  // neighbouring lanes on one kind
+        const int kind = id / 5, v = id % 5;
         double r;
-        if (kind == 0) {
-            double s = 0.0;
-            for (int i = 0; i < NP; ++i) s = fma(sW64[i], sQ[i * 5 + v], s);
-            r = s * 0.125;
-        } else if (kind <= 6) {
+        if (kind >= 1 && kind <= 6) {
             const int ax = (kind - 1) / 2, ia = ((kind - 1) % 2) ? NP - 1 : 0;
             r = sQ[(ax * NP + ia) * 5 + v] * 0.25;
         } else {
-            const int ax = kind - 7;
+            const int ax = kind == 0 ? 0 : kind - 7;
+            const double *wt = kind == 0 ? sW64 : sRow164;
             double s = 0.0;
-            for (int i = 0; i < NP; ++i) s = fma(sRow164[i], sQ[(ax * NP + i) * 5 + v], s);
-            r = s * 0.25;
+#pragma unroll
+            for (int i = 0; i < NP; ++i) s = fma(wt[i], sQ[(ax * NP + i) * 5 + v], s);
+            r = s * (kind == 0 ? 0.125 : 0.25);
         }
-        sl.S[e * 50 + id] = r;
+        sl.S[e * 50 + v * 10 + kind] = r;
     }
     if (SYS == 1 && live && t == 0 && sl.flags) sl.flags[e] = (sFlag[0] ? 1 : 0) | (sFlag[1] ? 2 : 0);
 }

@@ -24,7 +24,7 @@ struct CflNetSmem {
 // the learned network's guess, evaluated per chunk on the tensor cores.  Four CTAs
 // per SM cap the registers at 64 (the SR variants used 74-80, three CTAs).
 template <int SYS, int GUESS>
-__global__ void __launch_bounds__(kThreads, 4) k_cfl_mixed(const CflArgs a)
+__global__ void __launch_bounds__(kThreads, 4) k_cfl_mixed(const __grid_constant__ CflArgs a)
 {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char cfl_smem[];

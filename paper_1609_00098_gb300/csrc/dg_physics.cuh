@@ -302,21 +302,54 @@ __device__ __forceinline__ double max_speed(double g, const double u[5], const d
 // SR conserved-variable fix (Sec. 2.1.4): D >= d_atm, tau >= tau_atm D and
 // S^2 <= (1 - 1e-12) tau (tau + 2D).  Returns the variables it set, as a bit
 // mask (bit v for u[v]; the three momenta together), 0 if u is unchanged.
-__device__ __forceinline__ unsigned sr_fix(double d_atm, double tau_atm, double u[5])
+template <class A>
+__device__ __forceinline__ unsigned sr_fix(A &ar, double d_atm, double tau_atm, double u[5])
 {
     unsigned ch = 0;
     if (!(u[0] >= d_atm)) { u[0] = d_atm; ch |= 1u; }
-    const double tmin = tau_atm * u[0];
+    const double tmin = ar.mul(tau_atm, u[0]);
     if (!(u[4] >= tmin)) { u[4] = tmin; ch |= 16u; }
-    const double s2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
-    const double s2max = (1.0 - 1e-12) * (u[4] * (u[4] + 2.0 * u[0]));
+    const double s2 = ar.mul(u[1], u[1]) + ar.mul(u[2], u[2]) + ar.mul(u[3], u[3]);
+    const double s2max = ar.mul(1.0 - 1e-12, ar.mul(u[4], u[4] + 2.0 * u[0]));
     if (s2 > s2max) {
-        const double f = sqrt(s2max / s2);
-        u[1] *= f;
-        u[2] *= f;
-        u[3] *= f;
+        const double f = ar.root(ar.div(s2max, s2));
+        u[1] = ar.mul(u[1], f);
+        u[2] = ar.mul(u[2], f);
+        u[3] = ar.mul(u[3], f);
         ch |= 14u;
     }
+    return ch;
+}
+
+static __device__ __noinline__ unsigned sr_fix_native(double d_atm, double tau_atm, double *u)
+{
+    ifp::Native ar;
+    return sr_fix(ar, d_atm, tau_atm, u);
+}
+
+__device__ __forceinline__ unsigned sr_fix(double d_atm, double tau_atm, double u[5])
+{
+    ifp::Fast ar;
+    double w[5] = {u[0], u[1], u[2], u[3], u[4]};
+    unsigned ch = sr_fix(ar, d_atm, tau_atm, w);
+    if (!ar.ok) {
+        double q[5] = {u[0], u[1], u[2], u[3], u[4]};
+        ch = sr_fix_native(d_atm, tau_atm, q);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) w[v] = q[v];
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) u[v] = w[v];
+    return ch;
+}
+
+// The same as a call, for kernels where few nodes need it.
+static __device__ __noinline__ unsigned sr_fix_call(double d_atm, double tau_atm, double *u)
+{
+    double w[5] = {u[0], u[1], u[2], u[3], u[4]};
+    const unsigned ch = sr_fix(d_atm, tau_atm, w);
+#pragma unroll
+    for (int v = 0; v < 5; ++v) u[v] = w[v];
     return ch;
 }
 
