@@ -975,14 +975,19 @@ dg_status dg_rk3_step(dg_mesh *m, double *U, double dt, double cfl, double *dt_u
     const double cb[3] = {1.0, 0.25, 2.0 / 3.0};
     const double ct[3] = {0.0, 1.0, 0.5};  // stage times t + ct dt (analytic boundaries)
     for (int st = 0; st < 3; ++st) {
-        // the SR fix of the previous stage's result is fused into its primitive pass
-        DG_LAUNCH(m, s, PROF_PRIM,
-                  launch_primitives(m, ins[st], m->P, sr && st > 0, ins[st], (cflmode && st == 0) ? m->lam : nullptr, s));
+        // the SR fix of the previous stage's result is fused into its primitive pass; where
+        // nothing changes a stage's result (Newtonian, no limiter) the stage kernel writes
+        // the primitives itself
+        if (st == 0 || sr || lim)
+            DG_LAUNCH(m, s, PROF_PRIM,
+                      launch_primitives(m, ins[st], m->P, sr && st > 0, ins[st], (cflmode && st == 0) ? m->lam : nullptr, s));
         if (cflmode && st == 0) DG_LAUNCH(m, s, PROF_DT, launch_dt(m, cfl, m->dt, dt_used, s));
         if (m->gh.mask) DG_LAUNCH(m, s, PROF_OTHER, launch_exterior(m, ct[st], a.dt_ptr, dt, s));
         a.Us = ins[st];
         a.Un = U;
         a.out = outs[st];
+        a.Pout = (!sr && !lim && st < 2) ? m->P : nullptr;
+        a.gamma = m->d.gamma;
         a.first = st == 0;
         a.ca = ca[st];
         a.cb = cb[st];

@@ -111,6 +111,8 @@ struct StageArgs {
     const double *Fs;      // numerical fluxes of Us at the face points (FaceArgs)
     long long E;
     double *out;           // U_{s+1} (mode 1) or dU/dt (mode 0)
+    double *Pout;          // Newtonian primitives of U_{s+1} for the next stage (may be P), or nullptr
+    double gamma;          // (with Pout)
     const double *dt_ptr;  // device dt (CFL mode) or nullptr
     double dt;             // host dt when dt_ptr == nullptr
     double ca, cb;         // out = ca Un + cb (Us + dt R); first stage: out = Us + dt R

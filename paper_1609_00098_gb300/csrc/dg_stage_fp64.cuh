@@ -191,16 +191,27 @@ __global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const 
             if (fz) R[v] = R[v] + (k == 0 ? Le[oz + v * N2] : -Le[oz + v * N2]);
         }
         const long long ix = (e0 + el) * 5 * NN + q;
-        if (a.mode == 0) {
+        if (a.mode != 0) {
+            if (a.first) {
 #pragma unroll
-            for (int v = 0; v < 5; ++v) a.out[ix + v * NN] = R[v];
-        } else if (a.first) {
+                for (int v = 0; v < 5; ++v) R[v] = a.Us[ix + v * NN] + dt * R[v];
+            } else {
 #pragma unroll
-            for (int v = 0; v < 5; ++v) a.out[ix + v * NN] = a.Us[ix + v * NN] + dt * R[v];
-        } else {
+                for (int v = 0; v < 5; ++v)
+                    R[v] = a.ca * a.Un[ix + v * NN] + a.cb * (a.Us[ix + v * NN] + dt * R[v]);
+            }
+        }
 #pragma unroll
-            for (int v = 0; v < 5; ++v)
-                a.out[ix + v * NN] = a.ca * a.Un[ix + v * NN] + a.cb * (a.Us[ix + v * NN] + dt * R[v]);
+        for (int v = 0; v < 5; ++v) a.out[ix + v * NN] = R[v];
+        // Newtonian runs without a limiter: the next stage's primitives, from the state in
+        // registers (one launch less per stage: 48.0 -> 42.6 us per step at 4^3, n = 4;
+        // 4180 -> 4152 us at 24^3, n = 6).  An element's primitives are read in this launch
+        // by its own CTA only, before the barriers above.
+        if (a.Pout) {
+            double P[4];
+            ne_primitives(a.gamma, R, P);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) a.Pout[((e0 + el) * 4 + c) * NN + q] = P[c];
         }
     }
 }
