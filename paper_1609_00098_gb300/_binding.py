@@ -124,12 +124,17 @@ def _check(status: int):
 
 
 def _stream(stream=None):
+    """Raw cudaStream_t of a torch stream (None: the current one)."""
     if stream is None:
         import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        # the current stream's handle without building a torch.cuda.Stream (a third of a
+        # short call's host time); before torch has brought CUDA up, the public way
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def _ptr(t, numel: int | None = None, dtype=None, name: str = "tensor"):
@@ -137,8 +142,7 @@ def _ptr(t, numel: int | None = None, dtype=None, name: str = "tensor"):
     if t is None:
         return None
     if isinstance(t, int):
-        return ctypes.c_void_p(t)
-    import torch
+        return t
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
     if not t.is_contiguous():
@@ -147,7 +151,7 @@ def _ptr(t, numel: int | None = None, dtype=None, name: str = "tensor"):
         raise ValueError(f"{name} must have dtype {dtype}, got {t.dtype}")
     if numel is not None and t.numel() < numel:
         raise ValueError(f"{name} needs at least {numel} elements, has {t.numel()}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def make_desc(system=0, K=(4, 4, 4), n=4, flux=0, limiter=0, precision=0, gamma=1.4,
