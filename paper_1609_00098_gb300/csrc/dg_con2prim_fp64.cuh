@@ -25,7 +25,9 @@ struct C2pWarp {
     C2pQueue in, out;  // (out.plo unused)
 };
 
-static __device__ __noinline__ double c2p_bisect(double plo, double phi) { return 0.5 * (plo + phi); }
+// The iteration's two rare cases in FP64 instructions.
+static __device__ __noinline__ double c2p_bisect_native(double plo, double phi) { return 0.5 * (plo + phi); }
+static __device__ __noinline__ bool c2p_close_native(double pn, double p) { return fabs(pn - p) <= 0x1p-48 * pn; }
 
 // All nodes i = 32 b + lane of the batches b = warp, warp + nwarps, ... below count.
 // io.load(i, u) the conserved state (after any fix), io.guess(i) the starting pressure
@@ -137,12 +139,17 @@ __device__ __forceinline__ void c2p_warp(IO &io, C2pWarp &Q, double g, long long
                 const long long kn = (long long)ifp::dbits(pn), kl = (long long)ifp::dbits(plo);
                 const long long kh = (long long)ifp::dbits(phi);
                 const bool in = kn >= 0 && ((kn > kl && kn < kh) || (kn == kh && !hi_moved) || (kn == kl && !lo_moved));
-                if (!in) pn = c2p_bisect(plo, phi);
-                // |pn - p| <= 2^-48 pn, the product by the exponent field while it is normal
-                const long long kd = (long long)(ifp::dbits(pn - p) & 0x7fffffffffffffffULL);
-                long long kt = (long long)ifp::dbits(pn) - (48LL << 52);
-                if (kt < (1LL << 52)) kt = (long long)ifp::dbits(ifp::slow_mul(0x1p-48, pn));
-                last = kd <= kt;
+                // Some lane of almost every warp bisects, and some lane is close to its end: on
+                // the FP64 pipe these two would cost three of an iteration's 16 instructions.
+                // (On the integer ALU they leave that pipe room for all of the evaluation's
+                // products: 1760 us for 2^22 random states against 1815; one without the
+                // other gains nothing.)
+                if (!in) {
+                    if (ifp::half_sum_ok(plo, phi)) pn = ifp::half_sum_fast(plo, phi);
+                    else pn = c2p_bisect_native(plo, phi);
+                }
+                last = ifp::close_fast(pn, p);
+                if (!ifp::close_ok(pn, p)) last = c2p_close_native(pn, p);
                 if (!last && kh <= kl && kh < kInfBits) {
                     done = true;
                     iters = it + 1;
@@ -175,14 +182,16 @@ __device__ __forceinline__ void c2p_warp(IO &io, C2pWarp &Q, double g, long long
     while (ocnt > 0) finish_batch(ocnt < 32 ? ocnt : 32);
 }
 
-// CTAs for `count` nodes: every warp resident at once (five CTAs per SM by registers),
-// so that each takes an equal share of the batches; one batch per warp when there are
-// fewer.
-inline unsigned c2p_grid(long long count)
+// CTAs for `count` nodes: every warp resident at once (`ctas` per SM), so that each takes
+// an equal share of the batches; one batch per warp when there are fewer.  k_con2prim
+// runs six per SM (80 registers; 1709 us for 2^22 random states against 1740 with five and
+// 1798 with seven), k_primitives_sr, which needs 96 registers, five (16^3, n = 5: 1402 us
+// per step against 1455 with six).
+inline unsigned c2p_grid(long long count, int ctas)
 {
     const long long batches = (count + 31) / 32, warps = kC2pThreads / 32;
     const long long blocks = (batches + warps - 1) / warps;
-    return (unsigned)(blocks < 1 ? 1 : blocks < kNumSMs * 5 ? blocks : kNumSMs * 5);
+    return (unsigned)(blocks < 1 ? 1 : blocks < kNumSMs * ctas ? blocks : kNumSMs * ctas);
 }
 
 }  // namespace dg

@@ -20,8 +20,10 @@ namespace {
 
 constexpr int kFaceThreads = 128;
 
+// Five CTAs per SM where their registers allow it (Newtonian LF and HLL: 96 registers,
+// 106 without the bound; 24^3, n = 6: 128 us per pass against 138).
 template <int SYS, int FLX>
-__global__ void __launch_bounds__(kFaceThreads) k_face_fp64(const __grid_constant__ FaceArgs a)
+__global__ void __launch_bounds__(kFaceThreads, SYS == 0 && FLX != 2 ? 5 : 0) k_face_fp64(const __grid_constant__ FaceArgs a)
 {
     pdl_wait();
     const int n = a.n, n2 = n * n, nn = n2 * n;

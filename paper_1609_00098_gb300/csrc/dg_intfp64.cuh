@@ -17,7 +17,7 @@
 // infinities, NaN, results outside the normal range) takes the FP64 instruction.
 //
 // Methods, from the definitions: the multiply forms the exact 128-bit product of the
-// two significands.  The division is long division in three digits with a reciprocal
+// two significands.  The division is long division in two digits with a reciprocal
 // estimate from below, an exact remainder after every digit, and one final correction;
 // a quotient of two 53-bit significands is never half-way between two 53-bit values,
 // so floor(2^53 q) decides the rounding.  The square root refines an estimate from
@@ -195,10 +195,10 @@ __host__ __device__ __forceinline__ double mul(double a, double b)
 
 // ---------------------------------------------------------------------------
 // RN(a / b): significands A, B in [2^52, 2^53); A doubled if below B, so that the
-// quotient is in [1, 2).  r = 2^84 / B from below, within 2^-20 relative.  Digits of 18,
-// 18 and 17 bits: q = floor-ish(rem 2^k / B), never above the true digit and below it
-// by less than 2, rem exact (modulo 2^64, always below 2^54).  Several quotients by one
-// divisor share its part.
+// quotient is in [1, 2).  r = 2^84 / B from below, within 2^-30 relative.  Digits of 28
+// and 25 bits: q = floor-ish(rem 2^k / B), never above the true digit and below it by
+// less than 2 (rem's truncation costs 1/4, r 1/2, the floor 1), rem exact (modulo 2^64,
+// always below 2^54).  Several quotients by one divisor share its part.
 struct Divisor {
     double b;
     uint64_t B;
@@ -216,9 +216,14 @@ __host__ __device__ __forceinline__ Divisor divisor(double b)
     const uint32_t Bh = (d.h & 0xfffffu) | 0x100000u, Bl = lo32(bb);
     d.B = mk64(Bh, Bl);
     // reciprocal of B's significand rounded up to FP32, y in [0.5, 1), as 2^32 y less
-    // 2^10 (more than the estimate's error): r <= 2^84 / B
-    const float y = rcp_est(bflt(0x3f800001u + ((Bh & 0xfffffu) << 3) + (Bl >> 29)));
-    d.r = (fbits(y) << 8) + 0x7ffffc00u;
+    // 2^10 (more than the estimate's error): r0 <= 2^84 / B
+    const uint32_t c = (Bh << 11) | (Bl >> 21);  // B 2^-21, in [2^31, 2^32)
+    const float y = rcp_est(bflt((c >> 8) + 0x3f000001u));
+    const uint32_t r0 = (fbits(y) << 8) + 0x7ffffc00u;
+    // one Newton step: r0 (1 + e) with e = 1 - (c + 1) r0 2^-63 in (0, 2^-19), no more
+    // than the true error
+    const uint64_t e = 0x8000000000000000ULL - (mulw(c, r0) + r0);
+    d.r = r0 + (hi32(mulw((uint32_t)(e >> 12), r0)) >> 19);
     d.nl = 0u - Bl;
     d.nh = ~Bh + (Bl == 0u ? 1u : 0u);
     return d;
@@ -244,16 +249,13 @@ __host__ __device__ __forceinline__ double div_fast(double a, const Divisor &d)
         rem <<= 1;
         ex -= 1u << 20;
     }
-    const uint32_t q1 = hi32(mulw((uint32_t)(rem >> 22), d.r)) >> 12;
-    rem <<= 18;
+    const uint32_t q1 = hi32(mulw((uint32_t)(rem >> 22), d.r)) >> 2;
+    rem <<= 28;
     rem += mulw(q1, d.nl) + mk64(q1 * d.nh, 0u);
-    const uint32_t q2 = hi32(mulw((uint32_t)(rem >> 22), d.r)) >> 12;
-    rem <<= 18;
+    const uint32_t q2 = hi32(mulw((uint32_t)(rem >> 22), d.r)) >> 5;
+    rem <<= 25;
     rem += mulw(q2, d.nl) + mk64(q2 * d.nh, 0u);
-    const uint32_t q3 = hi32(mulw((uint32_t)(rem >> 22), d.r)) >> 13;
-    rem <<= 17;
-    rem += mulw(q3, d.nl) + mk64(q3 * d.nh, 0u);
-    uint64_t Q = ((uint64_t)q1 << 35) + ((uint64_t)q2 << 17) + q3;  // floor(2^53 A/B), or one below
+    uint64_t Q = ((uint64_t)q1 << 25) + q2;  // floor(2^53 A/B), or one below
     Q += rem >= d.B ? 2u : 1u;                                      // corrected, plus the rounding 1
     uint64_t bits = mk64(ex, 0u) + (Q >> 1);
     if ((ah & 0x7ff00000u) == 0u) bits = 0u;  // a = 0
@@ -315,6 +317,48 @@ __host__ __device__ __forceinline__ double root(double x)
     double r = root_fast(x);
     if (!root_ok(x)) r = DG_IFP_SLOW(slow_root(x), std::sqrt(x));
     return r;
+}
+
+// ---------------------------------------------------------------------------
+// RN(a + b) / 2 of two operands without sign, where half_sum_ok: the larger one normal
+// and neither it nor the sum near the ends of the range, the smaller one normal or zero.
+__host__ __device__ __forceinline__ bool half_sum_ok(double a, double b)
+{
+    const uint64_t x = dbits(a), y = dbits(b), big = x > y ? x : y, small = x > y ? y : x;
+    return ((hi32(big) >> 20) - 2u <= 2042u) & (((hi32(small) >> 20) - 1u <= 2043u) | (small == 0u));
+}
+
+__host__ __device__ __forceinline__ double half_sum_fast(double a, double b)
+{
+    const uint64_t x = dbits(a), y = dbits(b), big = x > y ? x : y, small = x > y ? y : x;
+    const uint32_t ex = hi32(big) >> 20, d = ex - (hi32(small) >> 20), sh = d < 63u ? d : 63u;
+    // significands with their top bits at bit 62, the smaller one aligned, the bits it
+    // loses folded into the lowest one
+    const uint64_t A = ((big & 0xfffffffffffffULL) | 0x10000000000000ULL) << 10;
+    const uint64_t B = small == 0u ? 0u : ((small & 0xfffffffffffffULL) | 0x10000000000000ULL) << 10;
+    uint64_t T = A + (B >> sh);
+    T |= ((B >> sh) << sh) != B ? 1u : 0u;
+    const uint32_t n = (uint32_t)(T >> 63);
+    T += (0x1ffu + (n << 9)) + ((uint32_t)(T >> (10 + n)) & 1u);  // to nearest even at bit 10 + n
+    return bdbl((T >> (10 + n)) + mk64((ex + n - 2u) << 20, 0u));
+}
+
+// Whether |a - b| <= 2^-48 a (difference and bound rounded), where close_ok: b without
+// sign and finite, a positive, normal and so is the bound, and the two in one binade
+// (bit patterns then count their distance in ulps; the bound is 16 to 31 ulps) or more
+// than 64 patterns apart (more than the bound, also where a binade's end halves the ulp).
+__host__ __device__ __forceinline__ bool close_ok(double a, double b)
+{
+    const uint64_t x = dbits(a), y = dbits(b);
+    const bool in = ((hi32(x) >> 20) - 49u <= 1997u) & ((hi32(y) >> 20) <= 2046u);
+    return in & (((hi32(x) ^ hi32(y)) >> 20 == 0u) | (x - y + 64u > 128u));
+}
+
+__host__ __device__ __forceinline__ bool close_fast(double a, double b)
+{
+    const uint64_t x = dbits(a), y = dbits(b);
+    const uint32_t t = 16u + ((hi32(x) >> 16) & 15u);
+    return x - y + t <= 2u * t;
 }
 
 // ---------------------------------------------------------------------------

@@ -59,15 +59,15 @@ struct C2PEval {
 };
 
 // E = tau + D.  Six divisions (the step's included) and a square root bound an
-// evaluation; they run on the integer ALU (dg_intfp64.cuh), the additions and as many
-// of the products as the FP64 pipe has time for on that.
+// evaluation; they run on the integer ALU (dg_intfp64.cuh), the additions and the
+// products on the FP64 pipe.
 template <class A>
 __device__ __forceinline__ C2PEval sr_c2p_eval(A &ar, double g, double D, double E, double s2, double tau, double p)
 {
     const double Ep = E + p;
-    const double v2 = ar.div(s2, ar.mul(Ep, Ep));
+    const double v2 = ar.div(s2, Ep * Ep);
     const double W = ar.div(1.0, ar.root(1.0 - v2));
-    const double DW = ar.mul(D, W);
+    const double DW = D * W;
     const double rhoeps = tau - v2 * (Ep - ar.div(DW, W + 1.0));
     C2PEval r;
     r.f = p - (g - 1.0) * rhoeps;

@@ -440,7 +440,7 @@ struct RowsIO {
     }
 };
 
-__global__ void __launch_bounds__(kC2pThreads, 5) k_con2prim(RowsIO io, double gamma)
+__global__ void __launch_bounds__(kC2pThreads, 6) k_con2prim(RowsIO io, double gamma)
 {
     __shared__ C2pWarp Q[kC2pThreads / 32];
     const long long warp = ((long long)blockIdx.x * kC2pThreads + threadIdx.x) >> 5;
@@ -475,7 +475,7 @@ cudaError_t launch_primitives(const dg_mesh *m, const double *U, double *P, int 
     a.d_atm = m->d.d_atm;
     a.tau_atm = m->d.tau_atm;
     return m->d.system == 0 ? launch_pdl(k_primitives_ne, grid_for(a.total, kThreads), kThreads, 0, s, a)
-                            : launch_pdl(k_primitives_sr, c2p_grid(a.total), kC2pThreads, 0, s, a);
+                            : launch_pdl(k_primitives_sr, c2p_grid(a.total, 5), kC2pThreads, 0, s, a);
 }
 
 cudaError_t launch_fix(const dg_mesh *m, double *U, cudaStream_t s)
@@ -564,7 +564,7 @@ cudaError_t launch_con2prim(long long count, double gamma, const double *cons, d
                             const double *guess, int *iters, int *status, cudaStream_t s)
 {
     const RowsIO io{count, cons, prim, guess, iters, status};
-    k_con2prim<<<c2p_grid(count), kC2pThreads, 0, s>>>(io, gamma);
+    k_con2prim<<<c2p_grid(count, 6), kC2pThreads, 0, s>>>(io, gamma);
     return cudaGetLastError();
 }
 

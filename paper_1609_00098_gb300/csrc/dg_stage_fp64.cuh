@@ -23,6 +23,9 @@ struct StageShape64 {
     static constexpr int EPB = NP == 2 ? 4 : NP == 3 ? 2 : 1;
     static constexpr int THREADS = NP == 2 || NP == 4 ? 256 : NP == 3 || NP == 6 ? 288 : NP == 8 ? 512 : 384;
     static constexpr size_t SMEM = sizeof(double) * (15 * NN + 30 * N2) * EPB;
+    // n = 6: four CTAs fit by their 56 registers either way, but told so the compiler
+    // spills less (24^3: 4106 us per step against 4225)
+    static constexpr int MIN_CTAS = NP == 6 ? 4 : 0;
 };
 
 // The rare cases of the two integer-ALU phases, in FP64 instructions.
@@ -75,8 +78,9 @@ static __device__ __noinline__ void line_native(const double *D, double *F, int 
 // both on it and one thread per node, the contraction ran at half the rate (0.25e12
 // against 0.50e12 product-sum pairs/s).  Lines also give 15 n^2 threads' work where
 // nodes give n^3, which is what a mesh with fewer elements than SMs needs.
-template <int NP>
-__global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const __grid_constant__ StageArgs a)
+template <int NP, bool PRIMS>
+__global__ void __launch_bounds__(StageShape64<NP>::THREADS, StageShape64<NP>::MIN_CTAS)
+    k_stage_fp64(const __grid_constant__ StageArgs a)
 {
     pdl_wait();
     using SH = StageShape64<NP>;
@@ -204,10 +208,11 @@ __global__ void __launch_bounds__(StageShape64<NP>::THREADS) k_stage_fp64(const 
 #pragma unroll
         for (int v = 0; v < 5; ++v) a.out[ix + v * NN] = R[v];
         // Newtonian runs without a limiter: the next stage's primitives, from the state in
-        // registers (one launch less per stage: 48.0 -> 42.6 us per step at 4^3, n = 4;
-        // 4180 -> 4152 us at 24^3, n = 6).  An element's primitives are read in this launch
-        // by its own CTA only, before the barriers above.
-        if (a.Pout) {
+        // registers (one launch less in stages 2 and 3: 48.0 -> 42.6 us per step at 4^3,
+        // n = 4).  An element's primitives are read in this launch by its own CTA only,
+        // before the barriers above.  (A variant of its own: as a run-time choice it took
+        // 2 % from the other runs at n = 6, by its registers.)
+        if (PRIMS) {
             double P[4];
             ne_primitives(a.gamma, R, P);
 #pragma unroll
@@ -432,12 +437,13 @@ cudaError_t launch_stage_np(const StageArgs &args, cudaStream_t s)
     using SH = StageShape64<NP>;
     StageArgs a = args;
     for (int i = 0; i < NP * NP; ++i) a.DF[i] = ifp::factor(a.T.D[i]);
+    void (*const kern)(const StageArgs) = a.Pout ? k_stage_fp64<NP, true> : k_stage_fp64<NP, false>;
     if (SH::SMEM > 48 * 1024) {
         const cudaError_t err =
-            cudaFuncSetAttribute(k_stage_fp64<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM);
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM);
         if (err != cudaSuccess) return err;
     }
-    return launch_pdl(k_stage_fp64<NP>, (unsigned)((a.E + SH::EPB - 1) / SH::EPB), SH::THREADS, SH::SMEM, s, a);
+    return launch_pdl(kern, (unsigned)((a.E + SH::EPB - 1) / SH::EPB), SH::THREADS, SH::SMEM, s, a);
 }
 
 template <int NP>

@@ -19,6 +19,15 @@ extern "C" void run(long n, const double *a, const double *b, double *m, double 
         r[i] = root(a[i]);
     }
 }
+extern "C" void run2(long n, const double *a, const double *b, double *h, int *hok, int *c, int *cok)
+{
+    for (long i = 0; i < n; ++i) {
+        h[i] = half_sum_fast(a[i], b[i]);
+        hok[i] = half_sum_ok(a[i], b[i]);
+        c[i] = close_fast(a[i], b[i]);
+        cok[i] = close_ok(a[i], b[i]);
+    }
+}
 """
 
 
@@ -63,3 +72,30 @@ def test_same_bits(lib, ka, kb):
             nan = np.isnan(ref)
             assert np.array_equal(np.isnan(got), nan)
             assert np.array_equal(got[~nan].view(np.uint64), ref[~nan].view(np.uint64))
+
+
+@pytest.mark.parametrize("ka", ["near", "sparse", "any", "special"])
+@pytest.mark.parametrize("kb", ["near", "sparse", "any", "special", "patterns"])
+def test_half_sum_and_closeness(lib, ka, kb):
+    a = np.abs(_operands(ka))
+    r = np.random.RandomState(5)
+    if kb == "patterns":  # a few patterns from a, and from the lower end of its binade across it
+        u = a.view(np.uint64)
+        u = np.where(r.rand(len(a)) < 0.3, u >> np.uint64(52) << np.uint64(52), u)
+        a = u.view(np.float64)
+        b = (u.view(np.int64) + r.randint(-70, 71, len(a))).view(np.float64)
+    else:
+        b = np.abs(np.roll(_operands(kb), 7))
+    a, b = np.ascontiguousarray(a), np.ascontiguousarray(b)
+    h = np.empty_like(a)
+    hok, c, cok = (np.empty(len(a), np.int32) for _ in range(3))
+    lib.run2(ctypes.c_long(len(a)), *[x.ctypes.data_as(ctypes.c_void_p) for x in (a, b, h, hok, c, cok)])
+    with np.errstate(all="ignore"):
+        ref, close = 0.5 * (a + b), np.abs(a - b) <= 2.0 ** -48 * a
+    hok, cok = hok != 0, cok != 0
+    assert np.array_equal(h[hok].view(np.uint64), ref[hok].view(np.uint64))
+    assert np.array_equal(c[cok] != 0, close[cok])
+    if ka == kb == "near":
+        assert hok.all() and cok.mean() > 0.9
+    if ka == "near" and kb == "patterns":
+        assert cok.mean() > 0.5 and close[cok].any() and not close[cok].all()
