@@ -402,12 +402,12 @@ def _con2prim_bench(pkg, torch, reps=3):
 # their state at capture.
 # The same capture's pipe utilisation (ncu, % of peak sustained while active, mean
 # of the three launches) is reported beside the flop fractions.
-SR_STAGE_FLOPS = {"fp64": 18911529, "fp32": 348447061}
-SR_STAGE_PIPES = {"fp64_pipe_pct": 35.2, "fma_pipe_pct": 13.9, "alu_pipe_pct": 22.1, "tensor_pipe_pct": 4.6,
-                  "issue_active_pct": 40.8}
+SR_STAGE_FLOPS = {"fp64": 18756852, "fp32": 358826423}
+SR_STAGE_PIPES = {"fp64_pipe_pct": 36.4, "fma_pipe_pct": 17.7, "alu_pipe_pct": 25.0, "tensor_pipe_pct": 5.1,
+                  "issue_active_pct": 47.4}
 SR_STAGE_SOURCES = ("paper_1609_00098_gb300/csrc/dg_mixed.cuh", "paper_1609_00098_gb300/csrc/dg_physics.cuh",
                     "paper_1609_00098_gb300/csrc/dg_c2p_net.cuh", "paper_1609_00098_gb300/csrc/dg_internal.h")
-SR_STAGE_SOURCES_SHA256 = "8d675640bc064200bd0ad8de38aa766def3ba352f8d371be08a4ad4bbbc41120"
+SR_STAGE_SOURCES_SHA256 = "c5993908742b5eb2bcebd9cf64861b2c0ac5b89f42c5ec86385b2fd5305b0fd2"
 # FMA throughput of this GPU (independent dependent-FMA chains, every SM busy;
 # flops count an FMA as two): FP64 1.20 TFLOP/s, FP32 75.0 TFLOP/s.
 FP64_PEAK_TFLOPS = 1.20
@@ -644,10 +644,10 @@ def _ensemble(pkg, torch, args):
 # stages of a step), from a one-kernel ncu capture of the same kernel on the
 # 32^3-element case of the same problem scaled by the node count (64^3 / 32^3 = 8).
 # Reported only while the kernel's sources still hash to their state at capture.
-# (409.7 MB per launch at 32^3, 57.9 B per node.)
-TRAFFIC_BYTES_PER_LAUNCH = 3277945515
+# (407.3 MB per launch at 32^3, 57.5 B per node.)
+TRAFFIC_BYTES_PER_LAUNCH = 3258189141
 TRAFFIC_SOURCES = ("paper_1609_00098_gb300/csrc/dg_ne_mixed.cuh", "paper_1609_00098_gb300/csrc/dg_internal.h")
-TRAFFIC_SOURCES_SHA256 = "55ff2325c3b9ad59fcdbeb0a4866b7772eff667623c900db9cdc2798eb3aa4ac"
+TRAFFIC_SOURCES_SHA256 = "77d37f00bff3e15d1ffa105eebd78939cbfecab043eeb6487dfb48382102d425"
 
 
 def _traffic():

@@ -223,8 +223,8 @@ dg_status dg_c2p_net_train(dg_c2p_net *net, long long count, const double *cons,
  * and result as dg_rhs on a mesh made from `desc` (FP64 only), but the node
  * primitives and the face fluxes live in static device arrays for
  * DG_RHS_STATIC_MAX_NODES nodes (4 and up to 7.5 doubles each, 11.5 MiB, held by
- * every GPU that loads the library until exit) and nothing is allocated.  U and dUdt are caller-owned device arrays in state
- * layout.  DG_ERR_ARG if the mesh has more than DG_RHS_STATIC_MAX_NODES nodes or
+ * every GPU that loads the library until exit) and nothing is allocated.  U and
+ * dUdt are caller-owned device arrays in state layout.  DG_ERR_ARG if the mesh has more than DG_RHS_STATIC_MAX_NODES nodes or
  * the descriptor is invalid.  The first call on a device looks up the arrays'
  * device addresses; make that first call before any stream capture.  The arrays are
  * shared by all calls and keep the last call's contents; calls that overlap on

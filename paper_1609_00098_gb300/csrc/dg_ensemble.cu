@@ -315,8 +315,8 @@ cudaError_t group_stage(EnsGroup &g, bool first, int st, cudaStream_t s)
     return e;
 }
 
-// One step of the ensemble: every group's pre-dt phase, the batched dt, every group's stages, all on s, stage by stage across
-// the groups.  concurrent: each group's phase runs on its own stream instead,
+// One step of the ensemble: every group's pre-dt phase, the batched dt, every group's
+// stages, all on s, stage by stage across the groups.  concurrent: each group's phase runs on its own stream instead,
 // forked from and joined back to s by events (in a captured graph: parallel
 // branches), so that the groups' launches overlap.  Both orders give the same
 // bits: no data crosses groups.  (On the 256-mesh recipe the two orders run within

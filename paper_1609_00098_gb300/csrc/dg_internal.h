@@ -15,8 +15,8 @@ constexpr int kNumSMs = 152;
 // (programmatic stream serialization): every kernel launched with launch_pdl begins with
 // pdl_wait(), which waits until the kernels before it have completed and their writes are
 // visible; nothing in memory is read or written before that.  A step of a small mesh is a
-// dozen launches of a few microseconds (smooth wave 4^3 x 4^3 FP64: 70 us a step without
-// this, 48 with).  No kernel lets its successor's CTAs onto the chip before it ends
+// dozen launches of a few microseconds (smooth wave 4^3 x 4^3 FP64, then ten launches: 70
+// us a step without this, 48 with).  No kernel lets its successor's CTAs onto the chip before it ends
 // (griddepcontrol.launch_dependents): they take room from its last wave, measured 53
 // us for that wave, shear layer 24^3 x 6^3 FP64 4.18 -> 4.36 ms, 64-mesh ensemble 10.75 ->
 // 11.29 ms.

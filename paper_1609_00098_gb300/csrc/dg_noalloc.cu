@@ -10,9 +10,9 @@
 // face fluxes) in file-scope static device arrays of fixed size, takes the mesh
 // descriptor directly, and allocates nothing.  The caller still owns U and dUdt.
 //
-// The array is global to the process on each device that loads the library and
-// keeps the last call's contents.  Calls that overlap on the GPU (two streams,
-// or two host threads) race on it and must be serialised by the caller.
+// The arrays are global to the process on each device that loads the library and
+// keep the last call's contents.  Calls that overlap on the GPU (two streams,
+// or two host threads) race on them and must be serialised by the caller.
 #include <cstring>
 #include <mutex>
 
