@@ -501,7 +501,7 @@ LimitSlot limit_slot(const dg_mesh *m, double *U, unsigned char *troubled)
     for (int ax = 0; ax < 3; ++ax) {
         l.K[ax] = m->d.K[ax];
         l.tvb[ax] = m->d.tvb_M * m->dx[ax] * m->dx[ax];
-        l.inv_dx[ax] = 1.0 / m->dx[ax];
+        l.inv_dx2[ax] = 2.0 * (1.0 / m->dx[ax]);
         l.beta_dx[ax] = m->d.beta / m->dx[ax];
         for (int i = 0; i < m->d.n; ++i) l.hx[ax][i] = 0.5 * m->dx[ax] * m->T.x[i];
     }

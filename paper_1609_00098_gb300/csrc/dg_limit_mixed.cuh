@@ -16,6 +16,11 @@ namespace dg {
 // FP64 fix runs in as few warp passes as possible).  Elements that are neither
 // troubled nor flagged by the stage kernel as needing the fix are left alone.
 // Like the stage kernel, a launch covers one mesh or a ragged batch of meshes.
+//
+// Bound by the FP64 pipe (a warp instruction costs it the same with 15 lanes active as
+// with 32) and, at one wave, by latency.  The slopes' products run on the integer ALU
+// and the replacement's partial sums are dealt to all lanes: relativistic blast 16^3, n =
+// 5, 26.5 -> 21.7 us per launch.
 struct LimitSlot {
     double *U;
     const double *S;
@@ -23,7 +28,7 @@ struct LimitSlot {
     unsigned char *troubled;
     int K[3];
     double tvb[3];          // M dx_a^2
-    double inv_dx[3];       // 1 / dx_a
+    double inv_dx2[3];      // 2 / dx_a
     double beta_dx[3];      // beta / dx_a
     double hx[3][MAXN];     // (dx_a / 2) x_i, x_i the LGL nodes
 };
@@ -74,9 +79,10 @@ __global__ void __launch_bounds__(32 * kLimitWarps) k_limit_mixed(const __grid_c
             const double vr = U0 + minmod3_bits(uhi - U0, U0 - U0m, U0p - U0);
             if (abs_gt(vl - ulo, 1e-8) || abs_gt(vr - uhi, 1e-8)) flag = 1;
         }
-        const double s1 = 2.0 * Se[7 + ax] * sl.inv_dx[ax];
+        const double s1 = ifp::mul(Se[7 + ax], sl.inv_dx2[ax]);
         slope = abs_le(s1, sl.tvb[ax]) ? s1
-                                       : minmod3_bits(s1, (U0p - U0) * sl.beta_dx[ax], (U0 - U0m) * sl.beta_dx[ax]);
+                                       : minmod3_bits(s1, ifp::mul(U0p - U0, sl.beta_dx[ax]),
+                                                      ifp::mul(U0 - U0m, sl.beta_dx[ax]));
     }
     const unsigned fb = __ballot_sync(0xffffffffu, flag);
     unsigned mask = 0;
@@ -88,28 +94,29 @@ __global__ void __launch_bounds__(32 * kLimitWarps) k_limit_mixed(const __grid_c
     if (lane == 0 && sl.troubled) sl.troubled[e] = (unsigned char)mask;
     if (!mask && !(fl & 2)) return;
     // The replacement m0 + s0 h0(i) + s1 h1(j) + s2 h2(k) (h_a = (dx_a/2) xbar): the
-    // part m0 + s0 h0(i) + s1 h1(j) is built once per (i, j) plane point and
-    // variable, so a node costs one FP64 FMA per limited variable.
+    // part m0 + s0 h0(i) is built once per variable and i, then s1 h1(j) added once per
+    // (i, j) plane point and variable, so a node costs one FP64 FMA per limited variable.
     __shared__ double sAB[kLimitWarps][5][NP * NP];  // per warp of the CTA
+    __shared__ double sA[kLimitWarps][5 * NP], sM[kLimitWarps][5], sS[kLimitWarps][2][5];
     __shared__ double sH2[kLimitWarps][NP];
     const int wl = threadIdx.x >> 5;
     double s2[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) s2[v] = __shfl_sync(0xffffffffu, slope, 3 * v + 2);
     if (mask) {
-        double m0[5], s0[5], s1[5];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) {
-            m0[v] = __shfl_sync(0xffffffffu, U0, 3 * v);
-            s0[v] = __shfl_sync(0xffffffffu, slope, 3 * v);
-            s1[v] = __shfl_sync(0xffffffffu, slope, 3 * v + 1);
-        }
-        for (int ij = lane; ij < NP * NP; ij += 32) {
-            const double h0 = sl.hx[0][ij % NP], h1 = sl.hx[1][ij / NP];
-#pragma unroll
-            for (int v = 0; v < 5; ++v) sAB[wl][v][ij] = fma(s1[v], h1, fma(s0[v], h0, m0[v]));
-        }
+        if (lane < 15 && lane % 3 == 0) sM[wl][lane / 3] = U0;
+        if (lane < 15 && lane % 3 < 2) sS[wl][lane % 3][lane / 3] = slope;
         if (lane < NP) sH2[wl][lane] = sl.hx[2][lane];
+        __syncwarp();
+        for (int r = lane; r < 5 * NP; r += 32) {
+            const int v = r / NP;
+            sA[wl][r] = fma(sS[wl][0][v], sl.hx[0][r - v * NP], sM[wl][v]);
+        }
+        __syncwarp();
+        for (int r = lane; r < 5 * NP * NP; r += 32) {
+            const int v = r / (NP * NP), ij = r - v * NP * NP, j = ij / NP;
+            sAB[wl][v][ij] = fma(sS[wl][1][v], sl.hx[1][j], sA[wl][v * NP + ij - j * NP]);
+        }
         __syncwarp();
     }
     // Node values: the replacement of the limited variables, else the stage state.
