@@ -10,7 +10,9 @@
 // Bound by the FP64 pipe and the integer ALU together: divisions, square roots and
 // products run on the latter (dg_intfp64.cuh), additions on the former.  Evaluated
 // inside the stage kernel instead, every face was taken twice, by 2 n^2 of the CTA's
-// threads, in three passes.
+// threads, in three passes: the step of the shear layer at 24^3, n = 6 went from 12.0 to
+// 9.1 ms with this kernel, that of the relativistic blast at 16^3, n = 5 from 4.7 to 4.1.
+// Now 128 us per launch on the former (FP64 pipe 77 %, integer ALU 57 %), 52 on the latter.
 #include "dg_internal.h"
 #include "dg_physics.cuh"
 

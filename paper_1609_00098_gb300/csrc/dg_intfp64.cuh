@@ -4,7 +4,7 @@
 // This GPU issues an FP64 instruction from a warp once every 64 cycles per SM
 // sub-partition (0.5e12 lane operations/s over the chip, measured), while its integer
 // ALU retires more than a warp instruction every other cycle.  An FP64 multiply costs
-// about 28 integer instructions here, a division about 65 and a square root about 60
+// about 28 integer instructions here, a division or a square root about 60
 // (the compiler's FP64 division and square root are each a sequence of FP64
 // instructions), so kernels bound by the FP64 pipe run these operations on the integer
 // ALU, beside the additions that stay on the FP64 pipe.  Measured on a line contraction

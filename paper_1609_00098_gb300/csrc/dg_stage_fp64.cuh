@@ -77,7 +77,9 @@ static __device__ __noinline__ void line_native(const double *D, double *F, int 
 // keep theirs on the FP64 pipe, which has room for them.  With products and sums
 // both on it and one thread per node, the contraction ran at half the rate (0.25e12
 // against 0.50e12 product-sum pairs/s).  Lines also give 15 n^2 threads' work where
-// nodes give n^3, which is what a mesh with fewer elements than SMs needs.
+// nodes give n^3, which is what a mesh with fewer elements than SMs needs.  24^3, n =
+// 6: 5430 us per launch with the faces and summaries inside, 900 now (FP64 pipe 81 %,
+// integer ALU 52 %); 16^3, n = 5: 1145 and 152; 4^3, n = 4: 33 and 10.7.
 template <int NP, bool PRIMS>
 __global__ void __launch_bounds__(StageShape64<NP>::THREADS, StageShape64<NP>::MIN_CTAS)
     k_stage_fp64(const __grid_constant__ StageArgs a)
@@ -256,7 +258,8 @@ __device__ __forceinline__ bool node_unphysical(const double u[5])
 // FP64-pipe bound.  The terms' products run on the integer ALU, and the weight products
 // are formed once per CTA.  Several elements share a CTA because a warp-wide FP64
 // instruction costs the same with 5 or 30 lanes active; one element per CTA, every
-// summary summing its own nodes, took two thirds of the FP64 stage's time.
+// summary summing its own nodes, took two thirds of the FP64 stage's time.  24^3, n = 6:
+// 210 us (FP64 pipe 62 %); 16^3, n = 5: 49 us.
 template <int NP>
 struct SumShape {
     static constexpr int NN = NP * NP * NP;
@@ -368,7 +371,8 @@ __global__ void __launch_bounds__(SumShape<NP>::THREADS) k_summaries(const __gri
 // dU-/(dx/beta); M)(x_a - x_a0) (eq:MinModSol) at every node, the terms added one
 // after another.  The terms depend on one node index each and the first two partial
 // sums on two, so they are formed once per (variable, index) and (variable, plane
-// point): one FP64 addition per node is left of nine operations.
+// point): one FP64 addition per node is left of nine operations.  24^3, n = 6: 466 us
+// per launch before, 54 now; 16^3, n = 5: 105 and 14.
 template <int NP>
 __global__ void __launch_bounds__(128) k_limit(const __grid_constant__ LimitArgs a)
 {
