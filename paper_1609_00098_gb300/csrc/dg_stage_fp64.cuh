@@ -23,9 +23,13 @@ struct StageShape64 {
     static constexpr int EPB = NP == 2 ? 4 : NP == 3 ? 2 : 1;
     static constexpr int THREADS = NP == 2 || NP == 4 ? 256 : NP == 3 || NP == 6 ? 288 : NP == 8 ? 512 : 384;
     static constexpr size_t SMEM = sizeof(double) * (15 * NN + 30 * N2) * EPB;
-    // n = 6: four CTAs fit by their 56 registers either way, but told so the compiler
-    // spills less (24^3: 4106 us per step against 4225)
-    static constexpr int MIN_CTAS = NP == 6 ? 4 : 0;
+    // CTAs that must fit on an SM, which caps the registers (36 for n = 2, 3, 40 for n = 5,
+    // 64 for n = 4, 80 for n = 7): more warps to hide the FP64 latency.  Step without a limiter at
+    // about 0.5 M nodes (KH, LLF), us, unbounded and so: n = 2 801, 646; n = 3 1000, 883; n
+    // = 4 1026, 979; n = 5 1080, 1045; n = 7 (one CTA per SM before) 1562, 1217.  n = 6 had
+    // four CTAs anyway, but spills less (24^3, limiter: 4225, 4106).  n = 8 keeps its own
+    // choice (64 registers, two CTAs: 1129; with 320 threads 1130 to 1224).
+    static constexpr int MIN_CTAS = NP == 2 ? 7 : NP == 3 ? 6 : NP == 7 ? 2 : NP <= 6 ? 4 : 0;
 };
 
 // The rare cases of the two integer-ALU phases, in FP64 instructions.
@@ -79,7 +83,7 @@ static __device__ __noinline__ void line_native(const double *D, double *F, int 
 // against 0.50e12 product-sum pairs/s).  Lines also give 15 n^2 threads' work where
 // nodes give n^3, which is what a mesh with fewer elements than SMs needs.  24^3, n =
 // 6: 5430 us per launch with the faces and summaries inside, 900 now (FP64 pipe 81 %,
-// integer ALU 52 %); 16^3, n = 5: 1145 and 152; 4^3, n = 4: 33 and 10.7.
+// integer ALU 52 %); 16^3, n = 5: 1145 and 146; 4^3, n = 4: 33 and 10.7.
 template <int NP, bool PRIMS>
 __global__ void __launch_bounds__(StageShape64<NP>::THREADS, StageShape64<NP>::MIN_CTAS)
     k_stage_fp64(const __grid_constant__ StageArgs a)
@@ -259,12 +263,15 @@ __device__ __forceinline__ bool node_unphysical(const double u[5])
 // are formed once per CTA.  Several elements share a CTA because a warp-wide FP64
 // instruction costs the same with 5 or 30 lanes active; one element per CTA, every
 // summary summing its own nodes, took two thirds of the FP64 stage's time.  24^3, n = 6:
-// 210 us (FP64 pipe 62 %); 16^3, n = 5: 49 us.
+// 209 us (FP64 pipe 62 %); 16^3, n = 5: 44 us.
 template <int NP>
 struct SumShape {
     static constexpr int NN = NP * NP * NP;
     static constexpr int G = NP <= 5 ? 6 : NP == 6 ? 4 : 3;  // most elements per CTA (5 G lanes of warp 0)
-    static constexpr int THREADS = NP <= 5 ? 192 : 128;
+    // (n = 7, 8: three elements fill the shared memory of a CTA, so more threads each: 1609
+    // -> 1573 us per step at n = 7 against 128; n = 5: 1 % against 192; n = 6 with 160: 2 %
+    // more for the kernel at 24^3)
+    static constexpr int THREADS = NP <= 4 ? 192 : NP == 6 ? 128 : 256;
     // per element: U[5][NN] and plane means [15 NP]; per CTA: weight products
     static constexpr size_t ELEM = sizeof(double) * (5 * NN + 15 * NP);
     static constexpr size_t TAB = (sizeof(double) + sizeof(ifp::Factor)) * (NN + NP * NP) + 8;
