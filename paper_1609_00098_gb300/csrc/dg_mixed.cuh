@@ -694,7 +694,9 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
     // the contraction is unchanged in exact arithmetic, and in FP32 its rounding
     // scales with the flux variation inside the element instead of its size.  (Every
     // thread forms node 0's fluxes itself: read back from shared memory they cost another
-    // barrier and two more passes over the flux arrays.)
+    // barrier and two more passes over the flux arrays.)  Flux and difference are rounded
+    // apart: fused with the subtraction, a product would leave its rounding error in the
+    // difference of equal fluxes, and a uniform flow a right-hand side of that size.
     if (own) {
         float u0[5], P0[NPRIM];
 #pragma unroll
@@ -707,7 +709,7 @@ __global__ void __launch_bounds__(StageShape<NP>::MAXT, StageShape<NP>::MIN_CTAS
             flux_axis32(u, P, ax, f);
             flux_axis32(u0, P0, ax, r);
 #pragma unroll
-            for (int v = 0; v < 5; ++v) sF[(ax * 5 + v) * NN + t] = f[v] - r[v];
+            for (int v = 0; v < 5; ++v) sF[(ax * 5 + v) * NN + t] = __fsub_rn(f[v], r[v]);
         }
     }
     __syncthreads();
