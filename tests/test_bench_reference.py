@@ -56,3 +56,18 @@ def test_roofline_arithmetic():
     assert abs(bench.FP64_STATE_BYTES_PER_NODE_STAGE * 3 - 320.0) < 1e-12
     r = bench._ensemble_roofline(1_000_000, 1.0)
     assert abs(r["achieved"] - 320.0) < 1e-9 and abs(r["frac"] - 320.0 / r["peak"]) < 1e-12
+
+
+def test_stage_counters_depend_on_every_source_of_the_kernel():
+    """The files whose hash guards the SR stage kernel's counters are the kernel's own and all
+    that its file's head includes, directly or not (the ABI's header aside, which has no code)."""
+    import re
+    csrc = "paper_1609_00098_gb300/csrc/"
+    todo, seen = [csrc + "dg_mixed.cuh"], set()
+    while todo:
+        f = todo.pop()
+        seen.add(f)
+        with open(os.path.join(ROOT, f)) as fh:
+            head = fh.read().split("namespace dg {")[0]  # (below it: other kernels' files)
+        todo += [csrc + i for i in re.findall(r'#include "(dg_\w+\.\w+)"', head) if csrc + i not in seen]
+    assert seen == set(bench.SR_STAGE_SOURCES)
