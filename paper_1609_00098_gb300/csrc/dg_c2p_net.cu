@@ -228,7 +228,6 @@ struct NetTrainSmem {
     float4 feat[2][NET_ROWS];         // features and target of the tile and of the next one
     double raw[6][NET_ROWS];          // the next tile's conserved values and pressures, loaded ahead
     float recv[NET_CLUSTER][NET_OWN]; // one-launch epochs: every CTA's gradient of the parameters this CTA owns
-    float bc[2];                      // Adam's bias corrections
 };
 
 // Barrier of the two warps of a pair.
@@ -569,8 +568,8 @@ __global__ void __launch_bounds__(256) k_net_reduce(const float *partial, int nb
     if (k >= OFF_W2 && k < OFF_W2 + 4096) W2b[k - OFF_W2] = __float2bfloat16_rn(pk);
 }
 
-// A whole epoch in one launch, by one cluster of CTAs that keep the weights in shared
-// memory: per mini-batch every CTA takes its tiles and writes its gradient into the
+// An epoch (or NET_LAUNCH_BATCHES mini-batches of it) in one launch, by one cluster of CTAs that
+// keep the weights in shared memory: per mini-batch every CTA takes its tiles and writes its gradient into the
 // owners' shared memory (CTA r owns the parameters [r NET_OWN, (r + 1) NET_OWN)), a cluster
 // barrier, every owner sums its parameters' gradients in CTA order, takes the Adam step
 // and writes the new values into every CTA's copy of the weights, a second barrier.
@@ -579,17 +578,20 @@ __global__ void __launch_bounds__(256) k_net_reduce(const float *partial, int nb
 // barriers and the exchange).  Launched per mini-batch, the same work is two launches
 // that use a fraction of the chip for a few microseconds each: 14.8 us per mini-batch
 // of 2048 against 8.2 us here (39 us before both).
+constexpr int NET_LAUNCH_BATCHES = 448;  // mini-batches of a launch, so that its arguments stay below 4 KB
+
 struct NetEpochArgs {
     NetTileArgs a;
     float *P, *m, *v;
     int batch;
-    long long step0;   // Adam steps taken before
+    long long begin, end;  // the samples of this launch (begin a multiple of batch)
     float lr;
-    float *loss;       // the epoch's mean loss, or nullptr
+    float *loss;           // the epoch's mean loss, added to, or nullptr
     float loss_scale;
+    float2 bc[NET_LAUNCH_BATCHES];  // Adam's bias corrections of every mini-batch
 };
 
-__global__ void __launch_bounds__(NET_THREADS, 1) k_net_epoch(const NetEpochArgs e)
+__global__ void __launch_bounds__(NET_THREADS, 1) k_net_epoch(const __grid_constant__ NetEpochArgs e)
 {
     namespace cg = cooperative_groups;
     extern __shared__ __align__(16) unsigned char net_smem_raw[];
@@ -601,19 +603,14 @@ __global__ void __launch_bounds__(NET_THREADS, 1) k_net_epoch(const NetEpochArgs
     // the parameter this thread owns, with its Adam moments (the loss counts as one)
     const int k = threadIdx.x < NET_OWN && rank * NET_OWN + (int)threadIdx.x < NET_PARTIAL ? rank * NET_OWN + threadIdx.x : -1;
     const bool par = k >= 0 && k < NET_PARAMS;
-    float pk = par ? e.P[k] : 0.0f, mk = par ? e.m[k] : 0.0f, vk = par ? e.v[k] : 0.0f, loss = 0.0f;
-    long long step = e.step0;
-    net_first_tile(S, a, 0, 0, a.count < e.batch ? a.count : e.batch, rank);
+    float pk = par ? e.P[k] : 0.0f, mk = par ? e.m[k] : 0.0f, vk = par ? e.v[k] : 0.0f;
+    float loss = k == NET_PARAMS && e.loss ? *e.loss : 0.0f;
+    net_first_tile(S, a, 0, e.begin, e.end - e.begin < e.batch ? e.end - e.begin : e.batch, rank);
     cl.sync();  // (every CTA of the cluster runs before its shared memory is written)
-    int buf = 0;
-    for (long long base = 0; base < a.count; base += e.batch) {
-        const long long ns = a.count - base < e.batch ? a.count - base : e.batch;
-        const long long nb = base + e.batch, left = a.count - nb;
-        step += 1;
-        if (threadIdx.x == NET_THREADS - 1) {
-            S.bc[0] = 1.0f - powf(0.9f, (float)step);
-            S.bc[1] = 1.0f - powf(0.999f, (float)step);
-        }
+    int buf = 0, mb = 0;
+    for (long long base = e.begin; base < e.end; base += e.batch, ++mb) {
+        const long long ns = e.end - base < e.batch ? e.end - base : e.batch;
+        const long long nb = base + e.batch, left = e.end - nb;
         net_cta_grad(
             S, a, buf, base, ns, left > 0 ? nb : 0, left > e.batch ? e.batch : left > 0 ? left : 0, rank, NET_CLUSTER,
             1.0f / (float)ns,
@@ -630,7 +627,7 @@ __global__ void __launch_bounds__(NET_THREADS, 1) k_net_epoch(const NetEpochArgs
             if (k == NET_PARAMS) {
                 loss += s * e.loss_scale;
             } else {
-                pk = net_adam(pk, mk, vk, s, e.lr, S.bc[0], S.bc[1]);
+                pk = net_adam(pk, mk, vk, s, e.lr, e.bc[mb].x, e.bc[mb].y);
                 if (k < OFF_B1) reinterpret_cast<float *>(&S.W.W1b1[k / 3])[k % 3] = pk;
                 else if (k < OFF_W2) S.W.W1b1[k - OFF_B1].w = pk;
                 else if (k < OFF_B2) S.W.W2[(k - OFF_W2) / 64][(k - OFF_W2) % 64] = __float2bfloat16_rn(pk);
@@ -672,7 +669,7 @@ __global__ void __launch_bounds__(NET_THREADS, 1) k_net_epoch(const NetEpochArgs
         e.m[k] = mk;
         e.v[k] = vk;
     } else if (k == NET_PARAMS && e.loss) {
-        *e.loss += loss;
+        *e.loss = loss;
     }
 }
 
@@ -801,8 +798,16 @@ bool net_cluster_fits()
     return n > 0;
 }
 
-cudaError_t launch_net_epoch(const dg_c2p_net *n, const double *cons, const double *p, long long count, int batch,
-                             float lr, float *loss, cudaStream_t s)
+// Adam's bias corrections of step `step`, on the host for both training paths: 1 - powf(0.999f, 1)
+// multiplies a rounding error of powf by a thousand, and the device's powf is another function.
+float2 net_bias(long long step)
+{
+    return make_float2(1.0f - powf(0.9f, (float)step), 1.0f - powf(0.999f, (float)step));
+}
+
+// The samples [begin, end) of an epoch, at most NET_LAUNCH_BATCHES mini-batches.
+cudaError_t launch_net_epoch(const dg_c2p_net *n, const double *cons, const double *p, long long count, long long begin,
+                             long long end, int batch, float lr, float *loss, cudaStream_t s)
 {
     NetEpochArgs e;
     std::memset(&e, 0, sizeof(e));
@@ -811,7 +816,9 @@ cudaError_t launch_net_epoch(const dg_c2p_net *n, const double *cons, const doub
     e.m = n->m;
     e.v = n->v;
     e.batch = batch;
-    e.step0 = n->step;
+    e.begin = begin;
+    e.end = end;
+    for (long long b = 0; begin + b * batch < end; ++b) e.bc[b] = net_bias(n->step + 1 + b);
     e.lr = lr;
     e.loss = loss;
     e.loss_scale = 1.0f / (float)count;
@@ -955,10 +962,14 @@ dg_status dg_c2p_net_train(dg_c2p_net *n, long long count, const double *cons, c
     for (int ep = 0; ep < epochs; ++ep) {
         float *loss = loss_per_epoch ? loss_per_epoch + ep : nullptr;
         if (cluster) {
-            NET_CUDA(launch_net_epoch(n, cons, p, count, batch, lr, loss, s));
-            n->step += nb;
-            k_net_bf16<<<16, 256, 0, s>>>(n->P, n->W2b);
-            NET_CUDA(cudaGetLastError());
+            for (long long b = 0; b < nb; b += NET_LAUNCH_BATCHES) {
+                const long long m = nb - b < NET_LAUNCH_BATCHES ? nb - b : NET_LAUNCH_BATCHES;
+                const long long end = b + m == nb ? count : (b + m) * batch;
+                NET_CUDA(launch_net_epoch(n, cons, p, count, b * batch, end, batch, lr, loss, s));
+                n->step += m;
+                k_net_bf16<<<16, 256, 0, s>>>(n->P, n->W2b);
+                NET_CUDA(cudaGetLastError());
+            }
             continue;
         }
         for (long long b = 0; b < nb; ++b) {
@@ -966,10 +977,9 @@ dg_status dg_c2p_net_train(dg_c2p_net *n, long long count, const double *cons, c
             const long long ns = (first + batch <= count) ? batch : count - first;
             NET_CUDA(launch_net_grad(n, cons, p, count, first, ns, s));
             n->step += 1;
-            const float bc1 = 1.0f - powf(0.9f, (float)n->step);
-            const float bc2 = 1.0f - powf(0.999f, (float)n->step);
+            const float2 bc = net_bias(n->step);
             k_net_reduce<<<(NET_PARTIAL + 31) / 32, 256, 0, s>>>(n->partial, (int)net_grad_blocks(ns), nullptr, n->P, n->m,
-                                                                  n->v, n->W2b, lr, bc1, bc2, 1, loss,
+                                                                  n->v, n->W2b, lr, bc.x, bc.y, 1, loss,
                                                                   1.0f / (float)count);
             NET_CUDA(cudaGetLastError());
         }

@@ -1,6 +1,11 @@
 """Outputs whose rounding is part of what the kernels promise."""
+import ctypes
+
 import numpy as np
 import pytest
+
+import dg_inputs as di
+from oracle import mlp
 
 pytestmark = pytest.mark.gpu
 
@@ -30,3 +35,90 @@ def test_relativistic_volume_term_of_a_uniform_flow_is_zero(pkg, n, flux):
     R = m.rhs(m.from_prim(prim[:, None].expand(5, m.E * n ** 3).contiguous())).cpu().numpy()
     inner = R.reshape(m.E, 5, n, n, n)[:, :, 1:-1, 1:-1, 1:-1]
     assert inner.size and np.abs(inner).max() == 0.0
+
+
+
+# ---- training of the guess network, bit for bit ------------------------------------------
+# The states and weights are built from seeded uniforms by operations that IEEE arithmetic rounds
+# the same everywhere.
+def net_states(count):
+    u = [di.uniform(77, s, np.arange(count)) for s in range(1, 9)]
+    D = np.ldexp(0.5 + u[1], (12.0 * u[0]).astype(int) - 8)
+    tau = D * np.ldexp(0.5 + u[3], (14.0 * u[2]).astype(int) - 7)
+    cons = np.stack([D, tau * (u[4] - 0.5), tau * (u[5] - 0.5), tau * (u[6] - 0.5), tau])
+    return cons, tau * (0.01 + 0.25 * u[7])
+
+
+def net_params():
+    p = mlp.init_params(di.uniform(5, 9, np.arange(mlp.N_PARAMS)))
+    for name in ("b1", "b2"):
+        o = mlp.OFFSETS[name]
+        p[o:o + 64] = 0.4 * (di.uniform(5, 10, np.arange(o, o + 64)) - 0.5)
+    return p.astype(np.float32)
+
+
+def net_grad(pkg, params, cons, p):
+    import torch
+    net = pkg.abi.dg_c2p_net_create(params, mlp.DEFAULT_SCALES)
+    grad = torch.empty(mlp.N_PARAMS, dtype=torch.float32, device="cuda")
+    loss = torch.empty(1, dtype=torch.float32, device="cuda")
+    pkg.abi.dg_c2p_net_grad(net, cons.shape[1], cons.contiguous(), p.contiguous(), grad, loss)
+    pkg.abi.dg_c2p_net_destroy(net)
+    return grad.cpu().numpy(), np.float32(loss.item())
+
+
+class Adam:
+    """The update in FP32, every operation rounded on its own, the bias corrections from the host's powf."""
+
+    def __init__(self, params, lr):
+        self.p, self.lr = params.copy(), np.float32(lr)
+        self.m, self.v, self.step = np.zeros_like(self.p), np.zeros_like(self.p), 0
+        self.powf = ctypes.CDLL("libm.so.6").powf
+        self.powf.restype, self.powf.argtypes = ctypes.c_float, [ctypes.c_float, ctypes.c_float]
+
+    def update(self, g):
+        f = np.float32
+        self.step += 1
+        self.m = f(0.9) * self.m + f(0.1) * g
+        self.v = f(0.999) * self.v + f(0.001) * g * g
+        b1, b2 = (f(1.0) - f(self.powf(b, self.step)) for b in (0.9, 0.999))
+        self.p = self.p - self.lr * (self.m / b1) / (np.sqrt(self.v / b2) + f(1e-8))
+
+
+def test_training_steps_are_adam_on_the_gradients(pkg):
+    """Every parameter after every one of 300 steps, one mini-batch each, is Adam's update of the one
+    before with dg_c2p_net_grad's gradient, to the bit (the device's powf gives other bias corrections
+    for some of the steps)."""
+    import torch
+    cons, p = (torch.from_numpy(x).cuda() for x in net_states(96))
+    adam = Adam(net_params(), 1e-3)
+    net = pkg.abi.dg_c2p_net_create(adam.p, mlp.DEFAULT_SCALES)
+    for step in range(300):
+        adam.update(net_grad(pkg, adam.p, cons, p)[0])
+        pkg.abi.dg_c2p_net_train(net, 96, cons, p, 1, 96, 1e-3)
+        assert np.array_equal(pkg.abi.dg_c2p_net_get_params(net), adam.p), step
+    pkg.abi.dg_c2p_net_destroy(net)
+
+
+def test_epochs_of_many_mini_batches(pkg):
+    """An epoch longer than one launch takes (448 mini-batches): two launches, one running loss."""
+    import torch
+    cons, p = (torch.from_numpy(x).cuda() for x in net_states(449 * 2 + 1))
+    params, out = net_params(), []
+    for whole in (True, False):
+        net = pkg.abi.dg_c2p_net_create(params, mlp.DEFAULT_SCALES)
+        if whole:
+            loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+            pkg.abi.dg_c2p_net_train(net, 449 * 2 + 1, cons, p, 1, 2, 1e-3, loss)
+            total = loss.item()
+        else:  # the same mini-batches, one call for each
+            total, one = 0.0, torch.zeros(1, dtype=torch.float32, device="cuda")
+            for i in range(0, 449 * 2 + 1, 2):
+                c, t = cons[:, i:i + 2].contiguous(), p[i:i + 2].contiguous()
+                pkg.abi.dg_c2p_net_train(net, t.numel(), c, t, 1, 2, 1e-3, one)
+                total += one.item() * t.numel() / (449 * 2 + 1)
+        out.append((pkg.abi.dg_c2p_net_get_params(net), total))
+        pkg.abi.dg_c2p_net_destroy(net)
+    assert np.array_equal(out[0][0], out[1][0])
+    # 450 terms of FP32 rounding each
+    assert abs(out[0][1] - out[1][1]) <= 450 * 2.0 ** -24 * out[1][1]
