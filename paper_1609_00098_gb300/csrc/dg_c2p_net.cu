@@ -93,19 +93,15 @@ __device__ __forceinline__ NetSample net_sample(const double v[5], const float s
 // sigma(z) = 1 / (1 + e^-z)
 __device__ __forceinline__ float sigmoid32(float z) { return __fdividef(1.0f, 1.0f + __expf(-z)); }
 
-// Layer 1 of two hidden units (16 kk + 8 hn + 2 tq, + 1) for rows g and g + 8 (x[0], x[1]
-// their features): h[c] with row c >> 1 and unit c & 1, and silu' in ds.
-template <bool TRAIN>
-__device__ __forceinline__ void net_layer1(const NetW &W, const float x[2][3], int unit, float h[4], float ds[4])
+// Layer 1 of two hidden units (unit, unit + 1) for two rows (x[0], x[1] their features): h[c]
+// with row c >> 1 and unit c & 1.
+__device__ __forceinline__ void net_layer1(const NetW &W, const float x[2][3], int unit, float h[4])
 {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         const float4 w = W.W1b1[unit + (c & 1)];
         const float *xr = x[c >> 1];
-        const float z = fmaf(w.x, xr[0], fmaf(w.y, xr[1], fmaf(w.z, xr[2], w.w)));
-        const float sg = sigmoid32(z);
-        h[c] = z * sg;
-        if (TRAIN) ds[c] = fmaf(h[c], 1.0f - sg, sg);
+        h[c] = silu(fmaf(w.x, xr[0], fmaf(w.y, xr[1], fmaf(w.z, xr[2], w.w))));
     }
 }
 
@@ -129,7 +125,7 @@ __device__ __forceinline__ void net_forward(const NetW &W, const float x[2][3], 
 #pragma unroll
         for (int hn = 0; hn < 2; ++hn) {
             float h[4];
-            net_layer1<false>(W, x, 16 * kk + 8 * hn + 2 * tq, h, nullptr);
+            net_layer1(W, x, 16 * kk + 8 * hn + 2 * tq, h);
             hf[2 * hn] = pack_bf16x2(h[0], h[1]);
             hf[2 * hn + 1] = pack_bf16x2(h[2], h[3]);
         }
@@ -208,13 +204,21 @@ __global__ void __launch_bounds__(NET_GUESS_THREADS, 2) k_net_guess(const NetTil
 }
 
 // ---------------------------------------------------------------------------
-// Training.  A CTA of 16 warps takes tiles of 128 samples: 16 samples per pair of warps,
-// each with half of every layer's columns, which exchange BF16 copies of h1 and dz2
-// through shared memory (two warps per tile shorten the serial chain of a mini-batch,
-// which is what training time is made of).  The layer-2 weight gradient dz2^T h1
-// over the tile is taken by all warps from those copies.
-constexpr int NET_WARPS = 16, NET_THREADS = 32 * NET_WARPS, NET_PAIRS = NET_WARPS / 2, NET_ROWS = 16 * NET_PAIRS;
+// Training.  A CTA of 16 warps takes a tile of 128 samples: four groups of four warps with
+// 32 samples each, a quarter (16) of every layer's columns per warp.  The warps of a group
+// exchange BF16 copies of h1 and dz2 and layer 3's products through shared memory (four
+// warps per 32 samples shorten the serial chain of a mini-batch, which is what training
+// time is made of).  The layer-2 weight gradient dz2^T h1 over the tile is taken by all
+// warps from those copies.
+//
+// The order of every sum is part of the result, and the same in each kind of launch: layer
+// 1 as ((w0 x0 + w1 x1) + w2 x2) + b1; layer 2's bias after its products; layer 3 over the
+// units of a lane (8 i + 2 tq, + 1) in turn, then over the four lanes; gradients and loss over
+// a lane's four samples, the eight lanes by halves (g ^ 1, g ^ 2, g ^ 4), the four groups and
+// the tiles in turn; no product is fused with a sum outside the tensor cores.
+constexpr int NET_WARPS = 16, NET_THREADS = 32 * NET_WARPS, NET_GROUPS = NET_WARPS / 4, NET_ROWS = 32 * NET_GROUPS;
 constexpr int NET_RED = 192 + 64 + 64 + 64 + 2;  // W1, b1, b2, W3, b3, loss
+constexpr int NET_YP_LD = 80;                    // (320 bytes: eight rows' 16-byte pieces in different banks)
 // CTAs of a one-launch epoch and the parameters each owns (a multiple of 8: 16-byte
 // pieces of W2's BF16 rows have one owner)
 constexpr int NET_CLUSTER = 16, NET_OWN = (NET_PARTIAL + 8 * NET_CLUSTER - 1) / (8 * NET_CLUSTER) * 8;
@@ -223,27 +227,26 @@ static_assert(NET_OWN <= NET_THREADS && NET_OWN * NET_CLUSTER >= NET_PARTIAL, "o
 struct NetTrainSmem {
     NetW W;
     __nv_bfloat16 h1[NET_ROWS][NET_W2_LD], dz2[NET_ROWS][NET_W2_LD];
-    float red[NET_PAIRS][NET_RED + 2];
-    float yp[2][NET_ROWS];            // layer 3's partial sums of the two column halves
+    float yp[NET_ROWS][NET_YP_LD];    // layer 3's products, [16 quarter + 4 tq + unit of the lane]
+    float y[NET_ROWS];
+    float red[NET_GROUPS][NET_RED + 2];
     float4 feat[2][NET_ROWS];         // features and target of the tile and of the next one
     double raw[6][NET_ROWS];          // the next tile's conserved values and pressures, loaded ahead
     float recv[NET_CLUSTER][NET_OWN]; // one-launch epochs: every CTA's gradient of the parameters this CTA owns
 };
 
-// Barrier of the two warps of a pair.
-__device__ __forceinline__ void net_pair_sync(int pair)
+// Barrier of the four warps of a group.
+__device__ __forceinline__ void net_group_sync(int group)
 {
-    asm volatile("bar.sync %0, 64;" ::"r"(pair + 1) : "memory");
+    asm volatile("bar.sync %0, 128;" ::"r"(group + 1) : "memory");
 }
 
-// Sums over the eight row groups g of 8 values per lane (column 8 nt + 2 tq + e of the
-// warp's half at index 2 nt + e), halving the values as the lanes pair up; this lane ends
-// with the sum of index lane >> 2 (bits reversed to the halving's order), added to dst
-// at its column.
-__device__ __forceinline__ void net_reduce_cols(float v[8], float *dst, int stride, int lane)
+// Sums over the eight row groups g of 8 values per lane, halving the values as the lanes pair
+// up (g ^ 1, then g ^ 2, g ^ 4); the lane ends with the sum of value `idx`.
+__device__ __forceinline__ float net_reduce8(float v[8], int lane, int &idx)
 {
 #pragma unroll
-    for (int n = 4, o = 16; n >= 1; n >>= 1, o >>= 1) {
+    for (int n = 4, o = 4; n >= 1; n >>= 1, o <<= 1) {
         const bool up = lane & o;
 #pragma unroll
         for (int i = 0; i < n; ++i) {
@@ -251,127 +254,162 @@ __device__ __forceinline__ void net_reduce_cols(float v[8], float *dst, int stri
             v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
     }
-    const int idx = lane >> 2;  // bits 4, 3, 2 of the lane: index bits 2, 1, 0
-    dst[((idx >> 1) * 8 + 2 * (lane & 3) + (idx & 1)) * stride] += v[0];
+    idx = (lane & 4) + ((lane & 8) >> 2) + ((lane & 16) >> 4);
+    return v[0];
 }
 
-// Loss and gradient of one tile, added to S.red (the pair's row, this warp's columns) and
+// Loss and gradient of one tile, written to S.red (the group's row, this warp's columns) and
 // gw2 (this warp's part of dW2: rows 16 (warp & 3) + .., columns 16 (warp >> 2) + ..).
 // feat: the tile's features and targets.  All warps of the CTA together.
 __device__ __forceinline__ void net_tile(NetTrainSmem &S, const float4 *feat, float inv_batch, float gw2[2][4])
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
-    const int pair = warp >> 1, half = warp & 1, c0 = 32 * half;  // the warp's columns c0 .. c0 + 31
-    float *red = S.red[pair];
-    const int row = pair * 16 + g;
-    float x[2][3], t[2];
-    bool ok[2];
+    const int group = warp >> 2, quarter = warp & 3;
+    const int r0 = 32 * group, c0 = 16 * quarter;  // the warp's rows r0 .. r0 + 31, columns c0 .. c0 + 15
+    float *red = S.red[group];
+    // the lane's rows r0 + 8 i + g
+    float x[4][3], t[4];
+    bool ok[4];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
+    for (int i = 0; i < 4; ++i) {
         // samples past the end and such without finite features or target (D or tau not
         // positive, a pressure below the FP32 range) enter neither the loss nor the gradient
-        const float4 f = feat[row + 8 * r];
-        ok[r] = isfinite(f.x) && isfinite(f.y) && isfinite(f.z) && isfinite(f.w);
-        x[r][0] = ok[r] ? f.x : 0.0f;
-        x[r][1] = ok[r] ? f.y : 0.0f;
-        x[r][2] = ok[r] ? f.z : 0.0f;
-        t[r] = f.w;
+        const float4 f = feat[r0 + 8 * i + g];
+        ok[i] = isfinite(f.x) && isfinite(f.y) && isfinite(f.z) && isfinite(f.w);
+        x[i][0] = ok[i] ? f.x : 0.0f;
+        x[i][1] = ok[i] ? f.y : 0.0f;
+        x[i][2] = ok[i] ? f.z : 0.0f;
+        t[i] = f.w;
     }
-    // layer 1, this warp's hidden units
-    float ds1[4][4];
+    // Accumulator layout below: [mt][nt][c], row r0 + 16 mt + 8 (c >> 1) + g (the lane's row 2 mt +
+    // (c >> 1)), column c0 + 8 nt + 2 tq + (c & 1).
+    float ds1[2][2][4];
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        float h[4];
-        net_layer1<true>(S.W, x, c0 + 8 * nt + 2 * tq, h, ds1[nt]);
-        *reinterpret_cast<uint32_t *>(&S.h1[row][c0 + 8 * nt + 2 * tq]) = pack_bf16x2(h[0], h[1]);
-        *reinterpret_cast<uint32_t *>(&S.h1[row + 8][c0 + 8 * nt + 2 * tq]) = pack_bf16x2(h[2], h[3]);
+    for (int nt = 0; nt < 2; ++nt) {
+        const int col = c0 + 8 * nt + 2 * tq;
+        const float4 w[2] = {S.W.W1b1[col], S.W.W1b1[col + 1]};
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+            float h[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float4 q = w[c & 1];
+                const float *xr = x[2 * mt + (c >> 1)];
+                const float z = q.x * xr[0] + q.y * xr[1] + q.z * xr[2] + q.w, sg = sigmoid32(z);
+                h[c] = z * sg;
+                ds1[mt][nt][c] = sg * (1.0f + z * (1.0f - sg));
+            }
+            *reinterpret_cast<uint32_t *>(&S.h1[r0 + 16 * mt + g][col]) = pack_bf16x2(h[0], h[1]);
+            *reinterpret_cast<uint32_t *>(&S.h1[r0 + 16 * mt + 8 + g][col]) = pack_bf16x2(h[2], h[3]);
+        }
     }
-    net_pair_sync(pair);
+    net_group_sync(group);
     // layer 2, this warp's columns
-    const int a_r = pair * 16 + (lane & 15), a_c = 8 * (lane >> 4);  // A fragments from row-major tiles
+    const int a_r = r0 + (lane & 15), a_c = 8 * (lane >> 4);  // A fragments from row-major tiles
     const int lr_n = (lane & 7) + 8 * (lane >> 4), lr_k = 8 * ((lane >> 3) & 1);
-    float z2[4][4], h2[4][4];
+    float z2[2][2][4], h2[2][2][4];
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const float2 b = *reinterpret_cast<const float2 *>(&S.W.b2[c0 + nt * 8 + 2 * tq]);
-        z2[nt][0] = z2[nt][2] = b.x;
-        z2[nt][1] = z2[nt][3] = b.y;
-    }
+    for (int i = 0; i < 16; ++i) z2[i >> 3][(i >> 2) & 1][i & 3] = 0.0f;
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
         uint32_t af[4], bq[4];
-        ldmatrix_x4(af, &S.h1[a_r][16 * kk + a_c]);
+        ldmatrix_x4(bq, &S.W.W2[c0 + lr_n][kk * 16 + lr_k]);
 #pragma unroll
-        for (int n2 = 0; n2 < 2; ++n2) {
-            ldmatrix_x4(bq, &S.W.W2[c0 + 16 * n2 + lr_n][kk * 16 + lr_k]);
-            mma_bf16(z2[2 * n2], af, bq);
-            mma_bf16(z2[2 * n2 + 1], af, bq + 2);
+        for (int mt = 0; mt < 2; ++mt) {
+            ldmatrix_x4(af, &S.h1[a_r + 16 * mt][16 * kk + a_c]);
+            mma_bf16(z2[mt][0], af, bq);
+            mma_bf16(z2[mt][1], af, bq + 2);
         }
     }
-    // layer 3: y = W3 . silu(z2) + b3
-    float y[2] = {0.0f, 0.0f};
+    // layer 3: the products W3 silu(z2 + b2), then y = their sum + b3 for one of the lane's rows
+    float w3[2][2];
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
+    for (int nt = 0; nt < 2; ++nt) {
+        const float2 b = *reinterpret_cast<const float2 *>(&S.W.b2[c0 + nt * 8 + 2 * tq]);
+        const float2 w = *reinterpret_cast<const float2 *>(&S.W.W3[c0 + nt * 8 + 2 * tq]);
+        w3[nt][0] = w.x;
+        w3[nt][1] = w.y;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float z = z2[nt][c], sg = sigmoid32(z);
-            h2[nt][c] = z * sg;
-            z2[nt][c] = fmaf(h2[nt][c], 1.0f - sg, sg);  // silu'(z2)
-            y[c >> 1] = fmaf(S.W.W3[c0 + nt * 8 + 2 * tq + (c & 1)], h2[nt][c], y[c >> 1]);
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float z = z2[mt][nt][c] + ((c & 1) ? b.y : b.x), sg = sigmoid32(z);
+                h2[mt][nt][c] = z * sg;
+                z2[mt][nt][c] = sg * (1.0f + z * (1.0f - sg));  // silu'(z2)
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float(*h)[4] = h2[i >> 1];
+        const int c = 2 * (i & 1);
+        *reinterpret_cast<float4 *>(&S.yp[r0 + 8 * i + g][16 * quarter + 4 * tq]) =
+            make_float4(w3[0][0] * h[0][c], w3[0][1] * h[0][c + 1], w3[1][0] * h[1][c], w3[1][1] * h[1][c + 1]);
+    }
+    net_group_sync(group);
+    {
+        const int row = r0 + 8 * quarter + g;
+        float v = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 p = *reinterpret_cast<const float4 *>(&S.yp[row][16 * q + 4 * tq]);
+            v = v + p.x + p.y + p.z + p.w;
         }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        y[r] += __shfl_xor_sync(0xffffffffu, y[r], 1);
-        y[r] += __shfl_xor_sync(0xffffffffu, y[r], 2);
-        if (tq == 0) S.yp[half][row + 8 * r] = y[r];
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        if (tq == 0) S.y[row] = v + S.W.b3;
     }
-    net_pair_sync(pair);
-    float dy[2], loss = 0.0f, db3 = 0.0f;
+    net_group_sync(group);
+    float dy[4], loss = 0.0f, db3 = 0.0f;
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const float d = ok[r] ? (S.yp[0][row + 8 * r] + S.yp[1][row + 8 * r]) + S.W.b3 - t[r] : 0.0f;
-        dy[r] = 2.0f * d * inv_batch;
-        loss = fmaf(d, d, loss);
-        db3 += dy[r];
+    for (int i = 0; i < 4; ++i) {
+        const float d = ok[i] ? S.y[r0 + 8 * i + g] - t[i] : 0.0f;
+        dy[i] = 2.0f * d * inv_batch;
+        loss += d * d;
+        db3 += dy[i];
     }
-    // dW3 = sum dy h2, db2 = sum dz2, dz2 = dy W3 silu'(z2)
-    float w3p[8], b2p[8];
+    // dW3 = sum dy h2, db2 = sum dz2, dz2 = dy W3 silu'(z2): values 2 nt + e and 4 + 2 nt + e
+    float p3[8];
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        float dz[4];
+    for (int i = 0; i < 8; ++i) p3[i] = 0.0f;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) dz[c] = dy[c >> 1] * S.W.W3[c0 + nt * 8 + 2 * tq + (c & 1)] * z2[nt][c];
+    for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            w3p[2 * nt + e] = fmaf(dy[0], h2[nt][e], dy[1] * h2[nt][2 + e]);
-            b2p[2 * nt + e] = dz[e] + dz[2 + e];
+        for (int nt = 0; nt < 2; ++nt) {
+            float dz[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float d = dy[2 * mt + (c >> 1)];
+                dz[c] = d * w3[nt][c & 1] * z2[mt][nt][c];
+                p3[2 * nt + (c & 1)] += d * h2[mt][nt][c];
+                p3[4 + 2 * nt + (c & 1)] += dz[c];
+            }
+            const int col = c0 + 8 * nt + 2 * tq;
+            *reinterpret_cast<uint32_t *>(&S.dz2[r0 + 16 * mt + g][col]) = pack_bf16x2(dz[0], dz[1]);
+            *reinterpret_cast<uint32_t *>(&S.dz2[r0 + 16 * mt + 8 + g][col]) = pack_bf16x2(dz[2], dz[3]);
         }
-        *reinterpret_cast<uint32_t *>(&S.dz2[row][c0 + 8 * nt + 2 * tq]) = pack_bf16x2(dz[0], dz[1]);
-        *reinterpret_cast<uint32_t *>(&S.dz2[row + 8][c0 + 8 * nt + 2 * tq]) = pack_bf16x2(dz[2], dz[3]);
-    }
     __syncthreads();
     // dh1 = dz2 W2, dz1 = dh1 silu'(z1), this warp's hidden units
-    float hacc[4][4];
+    float hacc[2][2][4];
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) hacc[nt][c] = 0.0f;
+    for (int i = 0; i < 16; ++i) hacc[i >> 3][(i >> 2) & 1][i & 3] = 0.0f;
     const int t_k = (lane & 7) + 8 * ((lane >> 3) & 1), t_n = 8 * (lane >> 4);  // B fragments, transposed loads
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
         uint32_t af[4], bq[4];
-        ldmatrix_x4(af, &S.dz2[a_r][16 * kk + a_c]);
+        ldmatrix_x4_trans(bq, &S.W.W2[kk * 16 + t_k][c0 + t_n]);
 #pragma unroll
-        for (int n2 = 0; n2 < 2; ++n2) {
-            ldmatrix_x4_trans(bq, &S.W.W2[kk * 16 + t_k][c0 + 16 * n2 + t_n]);
-            mma_bf16(hacc[2 * n2], af, bq);
-            mma_bf16(hacc[2 * n2 + 1], af, bq + 2);
+        for (int mt = 0; mt < 2; ++mt) {
+            ldmatrix_x4(af, &S.dz2[a_r + 16 * mt][16 * kk + a_c]);
+            mma_bf16(hacc[mt][0], af, bq);
+            mma_bf16(hacc[mt][1], af, bq + 2);
         }
     }
     // dW2 over the whole tile
     {
         const int j0 = 16 * (warp & 3), i0 = 16 * (warp >> 2);
         const int a_s = (lane & 7) + 8 * (lane >> 4), a_j = 8 * ((lane >> 3) & 1);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) gw2[i >> 2][i & 3] = 0.0f;
 #pragma unroll
         for (int kk = 0; kk < NET_ROWS / 16; ++kk) {
             uint32_t af[4], bq[4];
@@ -381,34 +419,39 @@ __device__ __forceinline__ void net_tile(NetTrainSmem &S, const float4 *feat, fl
             mma_bf16(gw2[1], af, bq + 2);
         }
     }
-    net_reduce_cols(w3p, red + 320 + c0, 1, lane);
-    net_reduce_cols(b2p, red + 256 + c0, 1, lane);
     // db1 = sum dz1, dW1 = sum dz1 x
+    float pa[8], pb[8];
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
+    for (int i = 0; i < 8; ++i) pa[i] = pb[i] = 0.0f;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) hacc[nt][c] *= ds1[nt][c];
+    for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        float p[8];
+        for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-                p[2 * nt + e] = q == 0 ? hacc[nt][e] + hacc[nt][2 + e]
-                                       : fmaf(hacc[nt][e], x[0][q - 1], hacc[nt][2 + e] * x[1][q - 1]);
-        if (q == 0) net_reduce_cols(p, red + 192 + c0, 1, lane);
-        else net_reduce_cols(p, red + 3 * c0 + (q - 1), 3, lane);
-    }
-    if (half == 0) {
+            for (int c = 0; c < 4; ++c) {
+                const int i = 2 * nt + (c & 1);
+                const float dz = hacc[mt][nt][c] * ds1[mt][nt][c], *xr = x[2 * mt + (c >> 1)];
+                pa[i] += dz;
+                pa[4 + i] += dz * xr[0];
+                pb[i] += dz * xr[1];
+                pb[4 + i] += dz * xr[2];
+            }
+    int idx;
+    const float s3 = net_reduce8(p3, lane, idx), sa = net_reduce8(pa, lane, idx), sb = net_reduce8(pb, lane, idx);
+    const int col = c0 + 8 * ((idx >> 1) & 1) + 2 * tq + (idx & 1);
+    red[(idx < 4 ? 320 : 256) + col] = s3;
+    if (idx < 4) red[192 + col] = sa;
+    else red[3 * col] = sa;
+    red[3 * col + (idx < 4 ? 1 : 2)] = sb;
+    if (quarter == 0) {
 #pragma unroll
         for (int o = 4; o < 32; o <<= 1) {
             loss += __shfl_xor_sync(0xffffffffu, loss, o);
             db3 += __shfl_xor_sync(0xffffffffu, db3, o);
         }
         if (lane == 0) {
-            red[384] += db3;
-            red[385] += loss;
+            red[384] = db3;
+            red[385] = loss;
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -464,35 +507,21 @@ __device__ __forceinline__ void net_first_tile(NetTrainSmem &S, const NetTileArg
     __syncthreads();
 }
 
-// The CTA's gradient and loss of tiles first, first + step, ... of `nsamp` samples from
-// sample `base` on, every pair's sums added in order: put2(k, v0, v1) receives the pairs of
-// dW2, put(k, v) the other parameters and the loss sum (k = NET_PARAMS).  S.feat[buf]
-// holds the first tile's features on entry; on return S.feat[buf] those of tile `first`
-// of the next mini-batch (nnsamp samples from nbase on).
+// The gradient and loss of tile tl of `nsamp` samples from sample `base` on, the four groups'
+// sums added in order: put2(k, v0, v1) receives the pairs of dW2, put(k, v) the other
+// parameters and the loss sum (k = NET_PARAMS).  S.feat[buf] holds the tile's features on
+// entry; on return (after the CTA's next barrier) S.feat[buf] those of tile ntl of the
+// nnsamp samples from nbase on.
 template <class Put2, class Put>
-__device__ __forceinline__ void net_cta_grad(NetTrainSmem &S, const NetTileArgs &a, int &buf, long long base,
-                                             long long nsamp, long long nbase, long long nnsamp, int first, int step,
-                                             float inv_batch, Put2 put2, Put put)
+__device__ __forceinline__ void net_cta_grad(NetTrainSmem &S, const NetTileArgs &a, int &buf, long long nbase,
+                                             long long nnsamp, long long ntl, float inv_batch, Put2 put2, Put put)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
     float gw2[2][4];
-#pragma unroll
-    for (int n = 0; n < 2; ++n)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) gw2[n][c] = 0.0f;
-    for (int k = lane; k < NET_RED; k += 32)
-        if (warp < NET_PAIRS) S.red[warp][k] = 0.0f;
-    const long long tiles = (nsamp + NET_ROWS - 1) / NET_ROWS;
-    if (first >= tiles) net_first_tile(S, a, buf, nbase, nnsamp, first);  // no tile here (a short last mini-batch)
-    for (long long tl = first; tl < tiles; tl += step) {
-        const bool more = tl + step < tiles;
-        const long long nx = more ? tl + step : first, nxs = more ? nsamp : nnsamp;
-        net_load_raw(S, a, more ? base : nbase, nxs, nx);
-        net_tile(S, S.feat[buf], inv_batch, gw2);  // (its last barrier also ends the loads)
-        buf ^= 1;
-        net_store_feature(S, S.feat[buf], nxs, nx, a.sc);
-        if (more) __syncthreads();
-    }
+    net_load_raw(S, a, nbase, nnsamp, ntl);
+    net_tile(S, S.feat[buf], inv_batch, gw2);  // (its last barrier also ends the loads)
+    buf ^= 1;
+    net_store_feature(S, S.feat[buf], nnsamp, ntl, a.sc);
     const int j = 16 * (warp & 3) + g, i = 16 * (warp >> 2) + 2 * tq;
 #pragma unroll
     for (int n = 0; n < 2; ++n) {
@@ -501,28 +530,30 @@ __device__ __forceinline__ void net_cta_grad(NetTrainSmem &S, const NetTileArgs 
     }
     if (threadIdx.x < NET_RED) {
         const int k = threadIdx.x;
-        float v = 0.0f;
-#pragma unroll
-        for (int w = 0; w < NET_PAIRS; ++w) v += S.red[w][k];
+        const float v = S.red[0][k] + S.red[1][k] + S.red[2][k] + S.red[3][k];
         put(k < 192 ? OFF_W1 + k : k < 256 ? OFF_B1 + k - 192 : k < 320 ? OFF_B2 + k - 256 : k < 384 ? OFF_W3 + k - 320
             : k == 384 ? OFF_B3 : NET_PARAMS, v);
     }
 }
+static_assert(NET_GROUPS == 4, "the sum over groups");
 static_assert(NET_RED <= NET_THREADS && NET_THREADS == 4 * NET_ROWS, "one thread per sum; four per sample");
 
-// One mini-batch's gradient partials, one per CTA (batches of many tiles).
+// One mini-batch's gradients, tile by tile into its rows of a.partial (batches of many tiles).
 __global__ void __launch_bounds__(NET_THREADS, 1) k_net_grad(const NetTileArgs a)
 {
     extern __shared__ __align__(16) unsigned char net_smem_raw[];
-    NetTrainSmem &S = *reinterpret_cast<NetTrainSmem *>(net_smem_raw);
+    NetTrainSmem &S = *reinterpret_cast<NetTrainSmem *>(net_smem_raw);  // (up to recv)
     net_load_weights(S.W, a.P, a.W2b);
     net_first_tile(S, a, 0, a.first, a.nsamp, blockIdx.x);
-    float *out = a.partial + (long long)blockIdx.x * NET_PARTIAL;
     int buf = 0;
-    net_cta_grad(
-        S, a, buf, a.first, a.nsamp, 0, 0, blockIdx.x, gridDim.x, a.inv_batch,
-        [out](int k, float v0, float v1) { *reinterpret_cast<float2 *>(out + k) = make_float2(v0, v1); },
-        [out](int k, float v) { out[k] = v; });
+    for (long long tl = blockIdx.x; tl * NET_ROWS < a.nsamp; tl += gridDim.x) {
+        float *out = a.partial + tl * NET_PARTIAL;
+        net_cta_grad(
+            S, a, buf, a.first, a.nsamp, tl + gridDim.x, a.inv_batch,
+            [out](int k, float v0, float v1) { *reinterpret_cast<float2 *>(out + k) = make_float2(v0, v1); },
+            [out](int k, float v) { out[k] = v; });
+        __syncthreads();
+    }
 }
 
 // One Adam step (Kingma & Ba) of a parameter; bc1, bc2 the bias corrections.
@@ -533,27 +564,42 @@ __device__ __forceinline__ float net_adam(float p, float &m, float &v, float gra
     return p - lr * (m / bc1) / (sqrtf(v / bc2) + 1e-8f);
 }
 
-// Sum the CTA partials: eight threads per parameter take every eighth partial in
-// order, then their sums are added in order.  Optionally one Adam step, which also
-// refreshes the BF16 copy of W2.
-constexpr int NET_SLICES = 8;
+// Sum the tiles' gradients in order, 64 tiles at a time: eight threads per parameter load
+// them, one adds them up while the next 64 are on their way.  Optionally one Adam step, which
+// also refreshes the BF16 copy of W2.
+constexpr int NET_SLICES = 8, NET_AHEAD = 8;
 
-__global__ void __launch_bounds__(256) k_net_reduce(const float *partial, int nblocks, float *grad, float *P, float *m,
-                                                    float *v, __nv_bfloat16 *W2b, float lr, float bc1, float bc2,
-                                                    int adam, float *loss_acc, float loss_scale)
+__global__ void __launch_bounds__(32 * NET_SLICES) k_net_reduce(const float *partial, long long tiles, float *grad,
+                                                                float *P, float *m, float *v, __nv_bfloat16 *W2b,
+                                                                float lr, float bc1, float bc2, int adam,
+                                                                float *loss_acc, float loss_scale)
 {
-    __shared__ float sum[NET_SLICES][32];
+    constexpr int ROWS = NET_SLICES * NET_AHEAD;
+    __shared__ float sq[2][ROWS][32];
     const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
     const int k = blockIdx.x * 32 + lane;
-    float s = 0.0f;
-    if (k <= NET_PARAMS)
-        for (int b = sl; b < nblocks; b += NET_SLICES) s += partial[(long long)b * NET_PARTIAL + k];
-    sum[sl][lane] = s;
-    __syncthreads();
-    if (sl != 0 || k > NET_PARAMS) return;
-    s = 0.0f;
+    float q[NET_AHEAD], s = 0.0f;
+    auto load = [&](long long b) {
 #pragma unroll
-    for (int q = 0; q < NET_SLICES; ++q) s += sum[q][lane];
+        for (int i = 0; i < NET_AHEAD; ++i) {
+            const long long r = b + sl + NET_SLICES * i;
+            q[i] = k <= NET_PARAMS && r < tiles ? partial[r * NET_PARTIAL + k] : 0.0f;
+        }
+    };
+    load(0);
+    int buf = 0;
+    for (long long b = 0; b < tiles; b += ROWS, buf ^= 1) {
+#pragma unroll
+        for (int i = 0; i < NET_AHEAD; ++i) sq[buf][sl + NET_SLICES * i][lane] = q[i];
+        __syncthreads();  // (also: the sum two rounds back, of the same buffer, is done)
+        load(b + ROWS);
+        if (sl == 0) {
+            const int n = tiles - b < ROWS ? (int)(tiles - b) : ROWS;
+#pragma unroll 16
+            for (int r = 0; r < n; ++r) s += sq[buf][r][lane];
+        }
+    }
+    if (sl != 0 || k > NET_PARAMS) return;
     if (k == NET_PARAMS) {
         if (loss_acc) *loss_acc += s * loss_scale;
         return;
@@ -576,8 +622,8 @@ __global__ void __launch_bounds__(256) k_net_reduce(const float *partial, int nb
 //
 // Bound by the serial chain of a mini-batch (a tile's forward and backward, two
 // barriers and the exchange).  Launched per mini-batch, the same work is two launches
-// that use a fraction of the chip for a few microseconds each: 14.8 us per mini-batch
-// of 2048 against 8.2 us here (39 us before both).
+// that use a fraction of the chip for a few microseconds each: 14.5 us per mini-batch
+// of 4096 against 8.2 us here for 2048 (39 us before both).
 constexpr int NET_LAUNCH_BATCHES = 448;  // mini-batches of a launch, so that its arguments stay below 4 KB
 
 struct NetEpochArgs {
@@ -611,19 +657,24 @@ __global__ void __launch_bounds__(NET_THREADS, 1) k_net_epoch(const __grid_const
     for (long long base = e.begin; base < e.end; base += e.batch, ++mb) {
         const long long ns = e.end - base < e.batch ? e.end - base : e.batch;
         const long long nb = base + e.batch, left = e.end - nb;
-        net_cta_grad(
-            S, a, buf, base, ns, left > 0 ? nb : 0, left > e.batch ? e.batch : left > 0 ? left : 0, rank, NET_CLUSTER,
-            1.0f / (float)ns,
-            [&](int q, float v0, float v1) {
-                float *d = cl.map_shared_rank(&S.recv[rank][q % NET_OWN], q / NET_OWN);
-                *reinterpret_cast<float2 *>(d) = make_float2(v0, v1);
-            },
-            [&](int q, float v) { *cl.map_shared_rank(&S.recv[rank][q % NET_OWN], q / NET_OWN) = v; });
+        const int tiles = (int)((ns + NET_ROWS - 1) / NET_ROWS);  // CTA r takes tile r, if there is one
+        if (rank < tiles)
+            net_cta_grad(
+                S, a, buf, left > 0 ? nb : 0, left > e.batch ? e.batch : left > 0 ? left : 0, rank, 1.0f / (float)ns,
+                [&](int q, float v0, float v1) {
+                    float *d = cl.map_shared_rank(&S.recv[rank][q % NET_OWN], q / NET_OWN);
+                    *reinterpret_cast<float2 *>(d) = make_float2(v0, v1);
+                },
+                [&](int q, float v) { *cl.map_shared_rank(&S.recv[rank][q % NET_OWN], q / NET_OWN) = v; });
         cl.sync();
         if (k >= 0) {
             float s = 0.0f;
+            if (tiles == NET_CLUSTER) {
 #pragma unroll
-            for (int r = 0; r < NET_CLUSTER; ++r) s += S.recv[r][threadIdx.x];
+                for (int r = 0; r < NET_CLUSTER; ++r) s += S.recv[r][threadIdx.x];
+            } else {
+                for (int r = 0; r < tiles; ++r) s += S.recv[r][threadIdx.x];
+            }
             if (k == NET_PARAMS) {
                 loss += s * e.loss_scale;
             } else {
@@ -721,16 +772,9 @@ dg_status set_error(dg_status st, const char *msg);
 
 namespace {
 
-// CTAs of a gradient launch: one per tile up to two rounds of the chip.
-long long net_grad_blocks(long long nsamp)
-{
-    const long long tiles = (nsamp + NET_ROWS - 1) / NET_ROWS;
-    return tiles < 2 * kNumSMs ? tiles : 2 * kNumSMs;
-}
-
-// Largest mini-batch an epoch runs in one cluster: a tile of 128 samples per CTA (8.2 us a
-// mini-batch of 2048 against 14.8 in two launches; at 4096, two tiles per CTA, the two
-// are equal).
+long long net_tiles(long long nsamp) { return (nsamp + NET_ROWS - 1) / NET_// Largest mini-batch an epoch runs in one cluster: a tile of 128 samples per CTA, 8.2 us a
+// mini-batch of 2048.  (A mini-batch of 4096 in two launches takes 14.5 us; in one cluster, two
+// tiles per CTA, it took the same.)
 constexpr int kClusterBatch = NET_CLUSTER * NET_ROWS;
 
 NetTileArgs net_args(const dg_c2p_net *n, const double *cons, const double *p, long long count)
@@ -754,10 +798,11 @@ cudaError_t launch_net_grad(const dg_c2p_net *n, const double *cons, const doubl
     a.first = first;
     a.nsamp = nsamp;
     a.inv_batch = 1.0f / (float)nsamp;
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_net_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NetTrainSmem));
+    constexpr size_t smem = offsetof(NetTrainSmem, recv);
+    const cudaError_t e = cudaFuncSetAttribute(k_net_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_net_grad<<<(unsigned)net_grad_blocks(nsamp), NET_THREADS, sizeof(NetTrainSmem), s>>>(a);
+    const long long tiles = net_tiles(nsamp);
+    k_net_grad<<<(unsigned)(tiles < kNumSMs ? tiles : kNumSMs), NET_THREADS, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -937,13 +982,13 @@ dg_status dg_c2p_net_grad(dg_c2p_net *n, long long count, const double *cons, co
 {
     if (!n || count <= 0 || !cons || !p || !grad || !loss)
         return set_error(DG_ERR_ARG, "net, cons, p, grad, loss must not be NULL and count > 0");
-    const long long blocks = net_grad_blocks(count);
-    if (dg_status st = ensure_partial(n, blocks)) return st;
+    const long long tiles = net_tiles(count);
+    if (dg_status st = ensure_partial(n, tiles)) return st;
     cudaStream_t s = (cudaStream_t)stream;
     NET_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s));
     NET_CUDA(launch_net_grad(n, cons, p, count, 0, count, s));
-    k_net_reduce<<<(NET_PARTIAL + 31) / 32, 256, 0, s>>>(n->partial, (int)blocks, grad, n->P, n->m, n->v, n->W2b, 0.0f,
-                                                          1.0f, 1.0f, 0, loss, 1.0f / (float)count);
+    k_net_reduce<<<(NET_PARTIAL + 31) / 32, 32 * NET_SLICES, 0, s>>>(n->partial, tiles, grad, n->P, n->m, n->v, n->W2b,
+                                                                      0.0f, 1.0f, 1.0f, 0, loss, 1.0f / (float)count);
     NET_CUDA(cudaGetLastError());
     return DG_OK;
 }
@@ -957,7 +1002,7 @@ dg_status dg_c2p_net_train(dg_c2p_net *n, long long count, const double *cons, c
     const long long nb = (count + batch - 1) / batch;
     const bool cluster = batch <= kClusterBatch && net_cluster_fits();
     if (!cluster)
-        if (dg_status st = ensure_partial(n, net_grad_blocks(batch))) return st;
+        if (dg_status st = ensure_partial(n, net_tiles(batch))) return st;
     if (loss_per_epoch) NET_CUDA(cudaMemsetAsync(loss_per_epoch, 0, sizeof(float) * epochs, s));
     for (int ep = 0; ep < epochs; ++ep) {
         float *loss = loss_per_epoch ? loss_per_epoch + ep : nullptr;
@@ -978,9 +1023,9 @@ dg_status dg_c2p_net_train(dg_c2p_net *n, long long count, const double *cons, c
             NET_CUDA(launch_net_grad(n, cons, p, count, first, ns, s));
             n->step += 1;
             const float2 bc = net_bias(n->step);
-            k_net_reduce<<<(NET_PARTIAL + 31) / 32, 256, 0, s>>>(n->partial, (int)net_grad_blocks(ns), nullptr, n->P, n->m,
-                                                                  n->v, n->W2b, lr, bc.x, bc.y, 1, loss,
-                                                                  1.0f / (float)count);
+            k_net_reduce<<<(NET_PARTIAL + 31) / 32, 32 * NET_SLICES, 0, s>>>(n->partial, net_tiles(ns), nullptr, n->P, n->m, n->v,
+                                                                              n->W2b, lr, bc.x, bc.y, 1, loss,
+                                                                              1.0f / (float)count);
             NET_CUDA(cudaGetLastError());
         }
     }

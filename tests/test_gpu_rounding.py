@@ -1,5 +1,6 @@
 """Outputs whose rounding is part of what the kernels promise."""
 import ctypes
+import os
 
 import numpy as np
 import pytest
@@ -40,7 +41,12 @@ def test_relativistic_volume_term_of_a_uniform_flow_is_zero(pkg, n, flux):
 
 # ---- training of the guess network, bit for bit ------------------------------------------
 # The states and weights are built from seeded uniforms by operations that IEEE arithmetic rounds
-# the same everywhere.
+# the same everywhere.  tests/golden/c2p_net_bits.txt holds gradients and trained values of some
+# of the parameters as hexadecimal floats, from kernels that evaluate every layer and sum in the
+# order that the comments of csrc/dg_c2p_net.cu give.
+NET_PICK, NET_GRAD, NET_TRAIN = slice(3, None, 61), (100, 300), ((300, 128), (4500, 2048), (5000, 2200))
+
+
 def net_states(count):
     u = [di.uniform(77, s, np.arange(count)) for s in range(1, 9)]
     D = np.ldexp(0.5 + u[1], (12.0 * u[0]).astype(int) - 8)
@@ -85,19 +91,67 @@ class Adam:
         self.p = self.p - self.lr * (self.m / b1) / (np.sqrt(self.v / b2) + f(1e-8))
 
 
-def test_training_steps_are_adam_on_the_gradients(pkg):
-    """Every parameter after every one of 300 steps, one mini-batch each, is Adam's update of the one
-    before with dg_c2p_net_grad's gradient, to the bit (the device's powf gives other bias corrections
-    for some of the steps)."""
+@pytest.mark.parametrize("count,steps", [(96, 300), (1000, 3), (2048, 3), (2049, 3)])
+def test_training_steps_are_adam_on_the_gradients(pkg, count, steps):
+    """Every parameter after every step, one mini-batch each, is Adam's update of the one before with
+    dg_c2p_net_grad's gradient, to the bit, whichever launch takes the mini-batch (the device's powf
+    gives other bias corrections for some of the first 300 steps)."""
     import torch
-    cons, p = (torch.from_numpy(x).cuda() for x in net_states(96))
+    cons, p = (torch.from_numpy(x).cuda() for x in net_states(count))
     adam = Adam(net_params(), 1e-3)
     net = pkg.abi.dg_c2p_net_create(adam.p, mlp.DEFAULT_SCALES)
-    for step in range(300):
+    for step in range(steps):
         adam.update(net_grad(pkg, adam.p, cons, p)[0])
-        pkg.abi.dg_c2p_net_train(net, 96, cons, p, 1, 96, 1e-3)
+        pkg.abi.dg_c2p_net_train(net, count, cons, p, 1, count, 1e-3)
         assert np.array_equal(pkg.abi.dg_c2p_net_get_params(net), adam.p), step
     pkg.abi.dg_c2p_net_destroy(net)
+
+
+@pytest.mark.parametrize("tiles", [2, 16, 32, 256])
+def test_gradient_is_the_sum_of_its_tiles_in_order(pkg, tiles):
+    """Gradient and loss of 128 t samples are those of every 128, added one after another in FP32 (a
+    power of two in the number of samples scales every term exactly)."""
+    import torch
+    cons, p = (torch.from_numpy(x).cuda() for x in net_states(128 * tiles))
+    g, loss = net_grad(pkg, net_params(), cons, p)
+    sg, sl = np.zeros_like(g), np.float32(0.0)
+    for i in range(0, 128 * tiles, 128):
+        q, one = net_grad(pkg, net_params(), cons[:, i:i + 128], p[i:i + 128])
+        sg, sl = sg + q, sl + one
+    assert np.array_equal(g, sg / np.float32(tiles)) and loss == sl / np.float32(tiles)
+
+
+def net_grad_bits(pkg, count):
+    import torch
+    g, loss = net_grad(pkg, net_params(), *(torch.from_numpy(x).cuda() for x in net_states(count)))
+    return np.concatenate([[loss], g[NET_PICK]])
+
+
+def net_train_bits(pkg, count, batch):
+    import torch
+    cons, p = (torch.from_numpy(x).cuda() for x in net_states(count))
+    net = pkg.abi.dg_c2p_net_create(net_params(), mlp.DEFAULT_SCALES)
+    loss = torch.zeros(2, dtype=torch.float32, device="cuda")
+    pkg.abi.dg_c2p_net_train(net, count, cons, p, 2, batch, 2e-3, loss)
+    out = pkg.abi.dg_c2p_net_get_params(net)
+    pkg.abi.dg_c2p_net_destroy(net)
+    return np.concatenate([loss.cpu().numpy(), out[NET_PICK]])
+
+
+def golden_bits(key):
+    with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "c2p_net_bits.txt")) as f:
+        rows = [ln.split() for ln in f if ln[0] != "#"]
+    return np.array([float.fromhex(x) for row in rows if row[0] == key for x in row[1:]])
+
+
+@pytest.mark.parametrize("count", NET_GRAD)
+def test_gradient_bits(pkg, count):
+    assert np.array_equal(net_grad_bits(pkg, count), golden_bits(f"grad{count}"))
+
+
+@pytest.mark.parametrize("count,batch", NET_TRAIN)
+def test_training_bits(pkg, count, batch):
+    assert np.array_equal(net_train_bits(pkg, count, batch), golden_bits(f"train{count}x{batch}"))
 
 
 def test_epochs_of_many_mini_batches(pkg):
