@@ -772,7 +772,9 @@ dg_status set_error(dg_status st, const char *msg);
 
 namespace {
 
-long long net_tiles(long long nsamp) { return (nsamp + NET_ROWS - 1) / NET_// Largest mini-batch an epoch runs in one cluster: a tile of 128 samples per CTA, 8.2 us a
+long long net_tiles(long long nsamp) { return (nsamp + NET_ROWS - 1) / NET_ROWS; }
+
+// Largest mini-batch an epoch runs in one cluster: a tile of 128 samples per CTA, 8.2 us a
 // mini-batch of 2048.  (A mini-batch of 4096 in two launches takes 14.5 us; in one cluster, two
 // tiles per CTA, it took the same.)
 constexpr int kClusterBatch = NET_CLUSTER * NET_ROWS;
