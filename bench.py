@@ -402,13 +402,13 @@ def _con2prim_bench(pkg, torch, reps=3):
 # their state at capture.
 # The same capture's pipe utilisation (ncu, % of peak sustained while active, mean
 # of the three launches) is reported beside the flop fractions.
-SR_STAGE_FLOPS = {"fp64": 18756654, "fp32": 358825936}
-SR_STAGE_PIPES = {"fp64_pipe_pct": 36.2, "fma_pipe_pct": 17.8, "alu_pipe_pct": 24.9, "tensor_pipe_pct": 5.1,
+SR_STAGE_FLOPS = {"fp64": 18772488, "fp32": 358819649}
+SR_STAGE_PIPES = {"fp64_pipe_pct": 36.8, "fma_pipe_pct": 18.0, "alu_pipe_pct": 25.1, "tensor_pipe_pct": 5.2,
                   "issue_active_pct": 47.5}
 SR_STAGE_SOURCES = ("paper_1609_00098_gb300/csrc/dg_mixed.cuh", "paper_1609_00098_gb300/csrc/dg_physics.cuh",
                     "paper_1609_00098_gb300/csrc/dg_c2p_net.cuh", "paper_1609_00098_gb300/csrc/dg_intfp64.cuh",
-                    "paper_1609_00098_gb300/csrc/dg_internal.h")
-SR_STAGE_SOURCES_SHA256 = "6509d7c1ed598f45fc581b532c37660cd3ac9fff35d62178b9d4acf8163c9b69"
+                    "paper_1609_00098_gb300/csrc/dg_polish64.cuh", "paper_1609_00098_gb300/csrc/dg_internal.h")
+SR_STAGE_SOURCES_SHA256 = "05a3ce46da02505f7e8a107b4add8b67f1ed98cf3f5bc92ac34cacad4d9bccad"
 # FMA throughput of this GPU (independent dependent-FMA chains, every SM busy;
 # flops count an FMA as two): FP64 1.20 TFLOP/s, FP32 75.0 TFLOP/s.
 FP64_PEAK_TFLOPS = 1.20

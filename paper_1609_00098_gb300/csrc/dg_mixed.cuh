@@ -15,6 +15,7 @@
 #include "dg_c2p_net.cuh"
 #include "dg_internal.h"
 #include "dg_physics.cuh"
+#include "dg_polish64.cuh"
 
 namespace dg {
 
@@ -291,7 +292,7 @@ __device__ __forceinline__ int sr_con2prim32(float g, const float u[5], float gu
 // bounded on cold states at the conserved-fix bound.  A call of its own: few warps
 // need it, but a warp that does holds its CTA's barrier, so its divisions and roots run
 // on the integer ALU (dg_intfp64.cuh), half the latency of the FP64 sequences, and an
-// iteration has two divisions and a root.
+// iteration has three divisions and a root (dg_polish64.cuh).
 static __device__ __noinline__ int sr_polish64(double g, const double *u, double p0, double *Pd)
 {
     const double D = u[0], tau = u[4];
@@ -306,20 +307,10 @@ static __device__ __noinline__ int sr_polish64(double g, const double *u, double
     int status = 2;
     bool lo_moved = false, hi_moved = false;
     for (int it = 0; it < 60; ++it) {
-        const double Ep = E + p;
-        const double inv = ifp::div(1.0, Ep);
-        const double v2 = s2 * inv * inv;
-        const double q = ifp::root(1.0 - v2);  // 1 / W
-        // rho eps with D W/(W + 1) = D/(1 + 1/W)
-        const double rhoeps = tau - v2 * (Ep - ifp::div(D, 1.0 + q));
-        const double f = p - (g - 1.0) * rhoeps;
-        if (fabs(f) <= 0x1p-50 * (p + (g - 1.0) * (tau + v2 * Ep))) { status = 0; break; }
-        if (f > 0.0) { phi = p; hi_moved = true; } else { plo = p; lo_moved = true; }
-        // f' in FP32: it only sets the step's length (to 1e-6 relative), the residual
-        // decides
-        const float v2f = f64_to_f32(v2);
-        const float df = 1.0f - (float)(g - 1.0) * v2f * (1.0f - f64_to_f32(D * inv) / f64_to_f32(q));
-        double pn = p - f * f32_to_f64(1.0f / df);
+        const PolishEval r = sr_polish_eval(g, D, E, s2, tau, p);
+        if (fabs(r.f) <= 0x1p-50 * r.scale) { status = 0; break; }
+        if (r.f > 0.0) { phi = p; hi_moved = true; } else { plo = p; lo_moved = true; }
+        double pn = p - ifp::div(r.fq, r.dq);
         if (!((pn > plo && pn < phi) || (pn == phi && !hi_moved) || (pn == plo && !lo_moved)))
             pn = phi > 4.0 * plo ? ifp::root(fmax(plo, 0x1p-40 * phi) * phi) : 0.5 * (plo + phi);
         const double dp = fabs(pn - p);
