@@ -593,6 +593,19 @@ SummaryArgs summary_args(const dg_mesh *m, const double *U, double *S)
     return a;
 }
 
+// A call between the pass that raises *lam and k_dt, which takes the maximum and clears it: a
+// return on an error in between clears it too, or the next step's dt would be that of both
+// states.
+struct LamGuard {
+    const dg_mesh *m;  // nullptr: nothing to clear
+    cudaStream_t s;
+    ~LamGuard()
+    {
+        if (m && cudaMemsetAsync(m->lam, 0, sizeof(*m->lam), s) != cudaSuccess) cudaGetLastError();
+    }
+    void taken() { m = nullptr; }
+};
+
 dg_status check_mesh(const dg_mesh *m)
 {
     if (!m) return fail(DG_ERR_ARG, "mesh is NULL");
@@ -839,8 +852,10 @@ dg_status dg_compute_dt(dg_mesh *m, const double *U, double cfl, double *dt, voi
     if (!U || !dt) return fail(DG_ERR_ARG, "U and dt must not be NULL");
     if (!(cfl > 0.0)) return fail(DG_ERR_ARG, "cfl must be > 0");
     cudaStream_t s = (cudaStream_t)stream;
+    LamGuard lam{m, s};
     DG_CUDA(launch_primitives(m, U, m->P, 0, nullptr, m->lam, s));
     DG_CUDA(launch_dt(m, cfl, dt, nullptr, s));
+    lam.taken();
     return DG_OK;
 }
 
@@ -855,6 +870,7 @@ static dg_status rk3_step_ne(dg_mesh *m, double *U, double dt, double cfl, doubl
     const bool lim = m->d.limiter != 0;
     const bool cflmode = cfl > 0.0;
     const double *dtp = cflmode ? m->dt : nullptr;
+    LamGuard lam{cflmode ? m : nullptr, s};
     const double ct[3] = {0.0, 1.0, 0.5};  // stage times t + ct dt (analytic boundaries)
     for (int st = 0; st < 3; ++st) {
         if (m->gh.mask) DG_LAUNCH(m, s, PROF_OTHER, launch_exterior(m, ct[st], dtp, dt, s));
@@ -862,6 +878,7 @@ static dg_status rk3_step_ne(dg_mesh *m, double *U, double dt, double cfl, doubl
         a.one.dt = dt;
         DG_LAUNCH(m, s, PROF_STAGE, launch_ne_stage(m->d.n, m->d.flux, st + 1, a, s));
         if (st == 0 && cflmode) DG_LAUNCH(m, s, PROF_DT, launch_dt(m, cfl, m->dt, dt_used, s));
+        lam.taken();
         NeDecideArgs d = ne_decide_args(m);
         d.one = ne_decide_stage_slot(m, U, st, cflmode, st == 2 ? troubled : nullptr);
         d.one.dt = dt;
@@ -901,6 +918,7 @@ static dg_status rk3_step_mixed(dg_mesh *m, double *U, double dt, double cfl, do
     a.mode = 1;
     float *latest = (carry && m->p_valid) ? m->pbuf[m->pi] : nullptr;
     if (cflmode) {
+        LamGuard lam{m, s};
         DG_LAUNCH(m, s, PROF_PRIM,
                   launch_cfl_mixed(m, U, latest, carry ? m->pbuf[1 - m->pi] : nullptr, pgiven ? m->pfull : nullptr,
                                    m->kappa_sw, s));
@@ -909,6 +927,7 @@ static dg_status rk3_step_mixed(dg_mesh *m, double *U, double dt, double cfl, do
             latest = m->pbuf[m->pi];
         }
         DG_LAUNCH(m, s, PROF_DT, launch_dt(m, cfl, m->dt, dt_used, s));
+        lam.taken();
     }
     double *ins[3] = {U, m->W1, m->W2};
     double *outs[3] = {m->W1, m->W2, U};
@@ -968,6 +987,7 @@ dg_status dg_rk3_step(dg_mesh *m, double *U, double dt, double cfl, double *dt_u
     a.mode = 1;
     a.dt = dt;
     a.dt_ptr = cflmode ? m->dt : nullptr;
+    LamGuard lam{cflmode ? m : nullptr, s};
 
     double *ins[3] = {U, m->W1, m->W2};
     double *outs[3] = {m->W1, m->W2, U};
@@ -982,6 +1002,7 @@ dg_status dg_rk3_step(dg_mesh *m, double *U, double dt, double cfl, double *dt_u
             DG_LAUNCH(m, s, PROF_PRIM,
                       launch_primitives(m, ins[st], m->P, sr && st > 0, ins[st], (cflmode && st == 0) ? m->lam : nullptr, s));
         if (cflmode && st == 0) DG_LAUNCH(m, s, PROF_DT, launch_dt(m, cfl, m->dt, dt_used, s));
+        lam.taken();
         if (m->gh.mask) DG_LAUNCH(m, s, PROF_OTHER, launch_exterior(m, ct[st], a.dt_ptr, dt, s));
         a.Us = ins[st];
         a.Un = U;

@@ -315,13 +315,26 @@ cudaError_t group_stage(EnsGroup &g, bool first, int st, cudaStream_t s)
     return e;
 }
 
+// An error between the passes that raise the meshes' wave-speed maxima and k_dt_batch, which
+// takes and clears them: they are cleared here, after the groups' launches still in flight, or
+// the next step's dt would be that of both states.
+void clear_maxima(dg_ensemble *en, cudaStream_t s)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+        for (cudaStream_t b : en->branch) cudaStreamSynchronize(b);
+        for (dg_mesh *m : en->meshes) cudaMemsetAsync(m->lam, 0, sizeof(*m->lam), s);
+    }  // (launches that are being captured have not run, and their graph is dropped)
+    cudaGetLastError();
+}
+
 // One step of the ensemble: every group's pre-dt phase, the batched dt, every group's
-// stages, all on s, stage by stage across the groups.  concurrent: each group's phase runs on its own stream instead,
-// forked from and joined back to s by events (in a captured graph: parallel
-// branches), so that the groups' launches overlap.  Both orders give the same
-// bits: no data crosses groups.  (On the 256-mesh recipe the two orders run within
-// about 1 % of each other: the launches' tails that the branches overlap are a
-// small part of a step.)
+// stages, all on s, stage by stage across the groups.  concurrent: each group's phase runs
+// on its own stream instead, forked from and joined back to s by events (in a captured
+// graph: parallel branches), so that the groups' launches overlap.  Both orders give the
+// same bits: no data crosses groups.  (On the 256-mesh recipe the two orders run within
+// about 1 % of each other: the launches' tails that the branches overlap are a small part
+// of a step.)
 cudaError_t launch_step(dg_ensemble *en, double cfl, bool first, bool concurrent, cudaStream_t s)
 {
     const int count = (int)en->meshes.size();
@@ -345,9 +358,11 @@ cudaError_t launch_step(dg_ensemble *en, double cfl, bool first, bool concurrent
             for (int i = 0; i < G && e == cudaSuccess; ++i) e = group_pre_dt(en->groups[i], first, s);
         }
     }
-    if (e != cudaSuccess) return e;
-    e = launch_pdl(k_dt_batch, blocks, 128, 0, s, en->d_dt, count, cfl);
-    if (e != cudaSuccess) return e;
+    if (e == cudaSuccess) e = launch_pdl(k_dt_batch, blocks, 128, 0, s, en->d_dt, count, cfl);
+    if (e != cudaSuccess) {
+        clear_maxima(en, s);
+        return e;
+    }
     if (concurrent)
         return fan_out([&](EnsGroup &g, cudaStream_t b) {
             cudaError_t r = cudaSuccess;
