@@ -606,6 +606,28 @@ struct LamGuard {
     void taken() { m = nullptr; }
 };
 
+// The new mesh's scratch that must be zero at its first use, zeroed before the creation returns:
+// that use may be on any stream, and memsets on the default stream would reach the device when
+// that stream's earlier work is done, perhaps in the middle of a step.
+cudaError_t clear_scratch(const dg_mesh *m)
+{
+    cudaStream_t s;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    auto zero = [&](const void *p, size_t bytes) {
+        if (e == cudaSuccess && bytes) e = cudaMemsetAsync(const_cast<void *>(p), 0, bytes, s);
+    };
+    zero(m->t, sizeof(*m->t));
+    zero(m->err, sizeof(*m->err));
+    zero(m->lam, sizeof(*m->lam));
+    zero(m->unphys, (size_t)m->E);
+    zero(m->gh.U, sizeof(double) * (size_t)m->nghost * 5 * m->nn);
+    zero(m->gh.P, sizeof(double) * (size_t)m->nghost * 4 * m->nn);
+    const cudaError_t w = cudaStreamSynchronize(s);
+    cudaStreamDestroy(s);
+    return e == cudaSuccess ? w : e;
+}
+
 dg_status check_mesh(const dg_mesh *m)
 {
     if (!m) return fail(DG_ERR_ARG, "mesh is NULL");
@@ -722,7 +744,6 @@ dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out)
     st = st ? st : cudaMalloc(&m->S, sizeof(double) * (size_t)E * 50);
     if (d->limiter == DG_LIMITER_MRS) st = st ? st : cudaMalloc(&m->mrsT, sizeof(double) * (size_t)E * 20);
     st = st ? st : cudaMalloc(&m->t, sizeof(double));
-    if (st == cudaSuccess) st = cudaMemset(m->t, 0, sizeof(double));
     for (int a = 0; a < 3; ++a) {
         if (d->bc[a] != DG_BC_ANALYTIC) continue;
         const long long cnt = (long long)d->K[(a + 1) % 3] * d->K[(a + 2) % 3];
@@ -737,17 +758,13 @@ dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out)
         st = st ? st : cudaMalloc(&gP, sizeof(double) * (size_t)m->nghost * 4 * m->nn);
         m->gh.U = gU;
         m->gh.P = gP;
-        if (st == cudaSuccess) st = cudaMemset(gU, 0, sizeof(double) * (size_t)m->nghost * 5 * m->nn);
-        if (st == cudaSuccess) st = cudaMemset(gP, 0, sizeof(double) * (size_t)m->nghost * 4 * m->nn);
     }
     if (!mixed) st = st ? st : cudaMalloc(&m->Fs, sizeof(double) * (size_t)(3 * E + m->nghost) * 5 * d->n * d->n);
     st = st ? st : cudaMalloc(&m->unphys, (size_t)E);
     st = st ? st : cudaMalloc(&m->lam, sizeof(unsigned long long));
     st = st ? st : cudaMalloc(&m->dt, sizeof(double));
     st = st ? st : cudaMalloc(&m->err, sizeof(unsigned int));
-    if (st == cudaSuccess) st = cudaMemset(m->err, 0, sizeof(unsigned int));
-    if (st == cudaSuccess) st = cudaMemset(m->unphys, 0, (size_t)E);
-    if (st == cudaSuccess) st = cudaMemset(m->lam, 0, sizeof(unsigned long long));
+    if (st == cudaSuccess) st = clear_scratch(m);
     if (st != cudaSuccess) {
         free_scratch(m);
         delete m;
