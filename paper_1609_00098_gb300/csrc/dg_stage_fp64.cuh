@@ -464,10 +464,12 @@ cudaError_t launch_summaries_np(const SummaryArgs &args, cudaStream_t s)
     // few elements: fewer per CTA, so that every SM gets some
     const long long per = (a.E + kNumSMs - 1) / kNumSMs;
     a.G = per < 1 ? 1 : per < SumShape<NP>::G ? (int)per : SumShape<NP>::G;
-    const size_t smem = SumShape<NP>::smem(a.G);
-    if (smem > 48 * 1024) {
+    const size_t smem = SumShape<NP>::smem(a.G), most = SumShape<NP>::smem(SumShape<NP>::G);
+    if (most > 48 * 1024) {
+        // the limit is the kernel's, for every thread of the process: always the largest, or a
+        // launch of another mesh would find it lowered
         const cudaError_t err =
-            cudaFuncSetAttribute(k_summaries<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaFuncSetAttribute(k_summaries<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
         if (err != cudaSuccess) return err;
     }
     return launch_pdl(k_summaries<NP>, (unsigned)((a.E + a.G - 1) / a.G), SumShape<NP>::THREADS, smem, s, a);
