@@ -128,9 +128,13 @@ def _stream(stream=None):
     if stream is None:
         import torch
         # the current stream's handle without building a torch.cuda.Stream (a third of a
-        # short call's host time); before torch has brought CUDA up, the public way
+        # short call's host time); before torch has brought CUDA up, or where it lacks these
+        # two private functions, the public way
         if torch.cuda.is_initialized():
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            try:
+                return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            except AttributeError:
+                pass
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
