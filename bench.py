@@ -403,12 +403,12 @@ def _con2prim_bench(pkg, torch, reps=3):
 # The same capture's pipe utilisation (ncu, % of peak sustained while active, mean
 # of the three launches) is reported beside the flop fractions.
 SR_STAGE_FLOPS = {"fp64": 18772488, "fp32": 358819649}
-SR_STAGE_PIPES = {"fp64_pipe_pct": 36.8, "fma_pipe_pct": 18.0, "alu_pipe_pct": 25.1, "tensor_pipe_pct": 5.2,
+SR_STAGE_PIPES = {"fp64_pipe_pct": 36.6, "fma_pipe_pct": 17.8, "alu_pipe_pct": 24.9, "tensor_pipe_pct": 5.1,
                   "issue_active_pct": 47.5}
 SR_STAGE_SOURCES = ("paper_1609_00098_gb300/csrc/dg_mixed.cuh", "paper_1609_00098_gb300/csrc/dg_physics.cuh",
                     "paper_1609_00098_gb300/csrc/dg_c2p_net.cuh", "paper_1609_00098_gb300/csrc/dg_intfp64.cuh",
                     "paper_1609_00098_gb300/csrc/dg_polish64.cuh", "paper_1609_00098_gb300/csrc/dg_internal.h")
-SR_STAGE_SOURCES_SHA256 = "05a3ce46da02505f7e8a107b4add8b67f1ed98cf3f5bc92ac34cacad4d9bccad"
+SR_STAGE_SOURCES_SHA256 = "6c49bcd247d611ba8fa0a400604c7215c377360588c5ceef2aa33b4dca845548"
 # FMA throughput of this GPU (independent dependent-FMA chains, every SM busy;
 # flops count an FMA as two): FP64 1.20 TFLOP/s, FP32 75.0 TFLOP/s.
 FP64_PEAK_TFLOPS = 1.20
@@ -645,10 +645,10 @@ def _ensemble(pkg, torch, args):
 # stages of a step), from a one-kernel ncu capture of the same kernel on the
 # 32^3-element case of the same problem scaled by the node count (64^3 / 32^3 = 8).
 # Reported only while the kernel's sources still hash to their state at capture.
-# (407.3 MB per launch at 32^3, 57.5 B per node.)
-TRAFFIC_BYTES_PER_LAUNCH = 3258189141
+# (407.4 MB per launch at 32^3, 57.6 B per node.)
+TRAFFIC_BYTES_PER_LAUNCH = 3259546283
 TRAFFIC_SOURCES = ("paper_1609_00098_gb300/csrc/dg_ne_mixed.cuh", "paper_1609_00098_gb300/csrc/dg_internal.h")
-TRAFFIC_SOURCES_SHA256 = "77d37f00bff3e15d1ffa105eebd78939cbfecab043eeb6487dfb48382102d425"
+TRAFFIC_SOURCES_SHA256 = "1dd66f71215d72d169eb2e4ac9a1d70fe076e603c3692e53fc7004869ccdc9a3"
 
 
 def _traffic():

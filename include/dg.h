@@ -81,8 +81,11 @@ enum { DG_EXACT_NONE = 0, DG_EXACT_ISENTROPIC_VORTEX = 1 };
 
 typedef struct dg_mesh dg_mesh;
 
-/* Create a mesh on the current device.  Allocates the library's scratch (two
- * state copies, a primitive buffer, limiter summaries, flags) with cudaMalloc.
+/* Create a mesh on the current device.  Allocates the library's scratch with
+ * cudaMalloc: primitives (4 doubles per node), a state copy (5) and the face fluxes
+ * (15/n doubles per node) for FP64; primitives, two state copies and limiter
+ * summaries (50 doubles per element) for mixed precision, with a few floats more per
+ * node or element; flags; ghosts of analytic boundaries.
  * Returns DG_ERR_ARG for an invalid descriptor, DG_ERR_NOMEM if allocation fails. */
 dg_status dg_mesh_create(const dg_mesh_desc *desc, dg_mesh **out);
 /* Free a mesh and its scratch (synchronises the device first).  NULL is ignored. */
@@ -224,12 +227,12 @@ dg_status dg_c2p_net_train(dg_c2p_net *net, long long count, const double *cons,
  * primitives and the face fluxes live in static device arrays for
  * DG_RHS_STATIC_MAX_NODES nodes (4 and up to 7.5 doubles each, 11.5 MiB, held by
  * every GPU that loads the library until exit) and nothing is allocated.  U and
- * dUdt are caller-owned device arrays in state layout.  DG_ERR_ARG if the mesh has more than DG_RHS_STATIC_MAX_NODES nodes or
- * the descriptor is invalid.  The first call on a device looks up the arrays'
- * device addresses; make that first call before any stream capture.  The arrays are
- * shared by all calls and keep the last call's contents; calls that overlap on
- * the GPU race on them.  A node without a physical primitive state gives non-finite
- * values in dUdt. */
+ * dUdt are caller-owned device arrays in state layout.  DG_ERR_ARG if the mesh has
+ * more than DG_RHS_STATIC_MAX_NODES nodes or the descriptor is invalid.  The first
+ * call on a device looks up the arrays' device addresses; make that first call
+ * before any stream capture.  The arrays are shared by all calls and keep the last
+ * call's contents; calls that overlap on the GPU race on them.  A node without a
+ * physical primitive state gives non-finite values in dUdt. */
 #define DG_RHS_STATIC_MAX_NODES 131072
 /* (periodic meshes only: DG_ERR_ARG for analytic boundaries) */
 dg_status dg_rhs_static(const dg_mesh_desc *desc, const double *U, double *dUdt, void *stream);

@@ -661,7 +661,7 @@ void free_scratch(dg_mesh *m)
     for (int i = 0; i < 3; ++i) cudaFree(m->abL[i]);
     cudaFree(m->P);
     cudaFree(m->Fs);
-    cudaFree(m->S);
+    if (m->S != m->Fs) cudaFree(m->S);
     cudaFree(m->mrsT);
     cudaFree(m->t);
     cudaFree(const_cast<double *>(m->gh.U));
@@ -728,7 +728,7 @@ dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out)
     m->epb = 1;
     cudaError_t st = cudaSuccess;
     st = st ? st : cudaMalloc(&m->W1, state);
-    st = st ? st : cudaMalloc(&m->W2, state);
+    if (mixed) st = st ? st : cudaMalloc(&m->W2, state);
     if (mixed && d->system == 0) {
         st = st ? st : cudaMalloc(&m->ne_SD, sizeof(float) * (size_t)E * 50);
         st = st ? st : cudaMalloc(&m->ne_M0, sizeof(double) * (size_t)E * 5);
@@ -741,7 +741,7 @@ dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out)
         st = st ? st : cudaMalloc(&m->pfull, sizeof(float) * 5 * (size_t)E * m->nn);
     }
     st = st ? st : cudaMalloc(&m->P, sizeof(double) * (size_t)E * 4 * m->nn);
-    st = st ? st : cudaMalloc(&m->S, sizeof(double) * (size_t)E * 50);
+    if (mixed) st = st ? st : cudaMalloc(&m->S, sizeof(double) * (size_t)E * 50);
     if (d->limiter == DG_LIMITER_MRS) st = st ? st : cudaMalloc(&m->mrsT, sizeof(double) * (size_t)E * 20);
     st = st ? st : cudaMalloc(&m->t, sizeof(double));
     for (int a = 0; a < 3; ++a) {
@@ -759,7 +759,12 @@ dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out)
         m->gh.U = gU;
         m->gh.P = gP;
     }
-    if (!mixed) st = st ? st : cudaMalloc(&m->Fs, sizeof(double) * (size_t)(3 * E + m->nghost) * 5 * d->n * d->n);
+    if (!mixed) {
+        // the face fluxes are dead once the stage kernel has run, which is when the limiter's
+        // summaries (50 doubles per element, at most the 15 n^2 of its faces) are formed
+        st = st ? st : cudaMalloc(&m->Fs, sizeof(double) * (size_t)(3 * E + m->nghost) * 5 * d->n * d->n);
+        m->S = m->Fs;
+    }
     st = st ? st : cudaMalloc(&m->unphys, (size_t)E);
     st = st ? st : cudaMalloc(&m->lam, sizeof(unsigned long long));
     st = st ? st : cudaMalloc(&m->dt, sizeof(double));
@@ -1006,8 +1011,10 @@ dg_status dg_rk3_step(dg_mesh *m, double *U, double dt, double cfl, double *dt_u
     a.dt_ptr = cflmode ? m->dt : nullptr;
     LamGuard lam{cflmode ? m : nullptr, s};
 
-    double *ins[3] = {U, m->W1, m->W2};
-    double *outs[3] = {m->W1, m->W2, U};
+    // with the face fluxes in memory, the stage kernel reads and writes an element's state
+    // only in that element's CTA, node by node: stage 2 runs in place
+    double *ins[3] = {U, m->W1, m->W1};
+    double *outs[3] = {m->W1, m->W1, U};
     const double ca[3] = {0.0, 0.75, 1.0 / 3.0};
     const double cb[3] = {1.0, 0.25, 2.0 / 3.0};
     const double ct[3] = {0.0, 1.0, 0.5};  // stage times t + ct dt (analytic boundaries)

@@ -110,7 +110,7 @@ struct StageArgs {
     const double *P;       // primitives (vx, vy, vz, p) of Us, [e][4][node]
     const double *Fs;      // numerical fluxes of Us at the face points (FaceArgs)
     long long E;
-    double *out;           // U_{s+1} (mode 1) or dU/dt (mode 0)
+    double *out;           // U_{s+1} (mode 1; may be Us) or dU/dt (mode 0)
     double *Pout;          // Newtonian primitives of U_{s+1} for the next stage (may be P), or nullptr
     double gamma;          // (with Pout)
     const double *dt_ptr;  // device dt (CFL mode) or nullptr
@@ -173,10 +173,10 @@ struct dg_mesh {
     double dxmin;    // smallest node gap
     dg::Tables T;
     // library-owned device scratch
-    double *W1, *W2;         // stage states
+    double *W1, *W2;         // stage states (FP64 path: W1 only)
     double *P;               // primitives [e][4][node]
     double *Fs;              // FP64 path: numerical fluxes at the face points [3 E + nghost][5][n^2]
-    double *S;               // limiter summaries [e][5][10]
+    double *S;               // limiter summaries [e][5][10] (FP64 path: in Fs, between a stage and the next faces)
     unsigned char *unphys;   // per-element SR flags (bit 0: an unphysical node; mixed path bit 1: a node needs the fix)
     unsigned long long *lam; // max wave speed (bit pattern of a non-negative double); 0 between steps
     double *dt;              // device step
