@@ -68,7 +68,10 @@ __host__ __device__ __forceinline__ uint32_t lo32(uint64_t b) { return (uint32_t
 __host__ __device__ __forceinline__ uint64_t mk64(uint32_t h, uint32_t l) { return ((uint64_t)h << 32) | l; }
 __host__ __device__ __forceinline__ uint64_t mulw(uint32_t a, uint32_t b) { return (uint64_t)a * b; }
 
-// 1/x and 1/sqrt(x) in FP32 to about 2^-22 (any estimate within 2^-21.5 does)
+// 1/x and 1/sqrt(x) in FP32.  What the digits below are exact for: 1/x within 2^-22 absolute for x
+// in [1, 2] (divisor() takes that much off, to stay below), 1/sqrt(x) within 2^-22.5 relative
+// (root_fast's second remainder then stays within 2^53).  The PTX manual gives the instructions'
+// largest errors as 2^-23 on that range, and 2^-22.9 relative.
 __host__ __device__ __forceinline__ float rcp_est(float x)
 {
 #ifdef __CUDA_ARCH__
@@ -215,8 +218,8 @@ __host__ __device__ __forceinline__ Divisor divisor(double b)
     d.h = hi32(bb);
     const uint32_t Bh = (d.h & 0xfffffu) | 0x100000u, Bl = lo32(bb);
     d.B = mk64(Bh, Bl);
-    // reciprocal of B's significand rounded up to FP32, y in [0.5, 1), as 2^32 y less
-    // 2^10 (more than the estimate's error): r0 <= 2^84 / B
+    // reciprocal of B's significand rounded up to FP32, y in [0.5, 1], as 2^32 y less
+    // 2^10 (2^-22 of it, no less than the estimate's error): r0 <= 2^84 / B
     const uint32_t c = (Bh << 11) | (Bl >> 21);  // B 2^-21, in [2^31, 2^32)
     const float y = rcp_est(bflt((c >> 8) + 0x3f000001u));
     const uint32_t r0 = (fbits(y) << 8) + 0x7ffffc00u;

@@ -31,15 +31,40 @@ extern "C" void run2(long n, const double *a, const double *b, double *h, int *h
 """
 
 
-@pytest.fixture(scope="module")
-def lib(tmp_path_factory):
-    d = tmp_path_factory.mktemp("intfp64")
+def _compile(d, header_dir, *flags):
     src, so = str(d / "t.cpp"), str(d / "t.so")
     with open(src, "w") as f:
         f.write(SRC)
-    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC, src, "-o", so],
-                   check=True)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", *flags, "-I", header_dir, src,
+                    "-o", so], check=True)
     return ctypes.CDLL(so)
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return _compile(tmp_path_factory.mktemp("intfp64"), CSRC)
+
+
+# The estimates that the division and the root start from, off by RCP (absolute) and RSQRT
+# (relative) on top of their own rounding to FP32.
+NUDGED = (("return 1.0f / x;", "return (float)(1.0 / (double)x + RCP);"),
+          ("return 1.0f / std::sqrt(x);", "return (float)((1.0 + RSQRT) / std::sqrt((double)x));"))
+
+
+@pytest.fixture(scope="module", params=[(r, q) for r in (-1, 1) for q in (-1, 1)])
+def nudged(request, tmp_path_factory):
+    """The operations with both estimates at the ends of the ranges that they are exact for."""
+    d = tmp_path_factory.mktemp("intfp64_nudged")
+    with open(os.path.join(CSRC, "dg_intfp64.cuh")) as f:
+        text = f.read()
+    for old, new in NUDGED:
+        assert text.count(old) == 1
+        text = text.replace(old, new)
+    with open(d / "dg_intfp64.cuh", "w") as f:
+        f.write(text)
+    r, q = request.param
+    # 2^-22 and 2^-22.5, less the rounding of the estimate itself (half an FP32 ulp below 1)
+    return _compile(d, str(d), f"-DRCP=({r * (2.0 ** -22 - 2.0 ** -25)!r})", f"-DRSQRT=({q * (2.0 ** -22.5 - 2.0 ** -24)!r})")
 
 
 def _operands(kind):
@@ -50,6 +75,9 @@ def _operands(kind):
     if kind == "sparse":      # significands with few bits at either end: exact results, carries, halves
         k = r.randint(0, 52, n).astype(np.uint64)
         mant = np.where(r.rand(n) < 0.5, mant >> k << k, mant | ((np.uint64(1) << k) - np.uint64(1)))
+    if kind == "ends":        # significands near 1 and 2, where the estimates' slack is smallest
+        k = (bits >> np.uint64(2)) & np.uint64((1 << 30) - 1)
+        mant = np.where(r.rand(n) < 0.5, k, np.uint64((1 << 52) - 1) - k)
     exp = r.randint(0, 2048, n) if kind == "any" else r.randint(960, 1087, n)
     sign = r.randint(0, 2, n).astype(np.uint64) << np.uint64(63)
     x = (sign | (exp.astype(np.uint64) << np.uint64(52)) | mant).view(np.float64)
@@ -60,9 +88,7 @@ def _operands(kind):
     return x
 
 
-@pytest.mark.parametrize("ka", ["near", "sparse", "any", "special"])
-@pytest.mark.parametrize("kb", ["near", "sparse", "any", "special"])
-def test_same_bits(lib, ka, kb):
+def _same_bits(lib, ka, kb):
     a, b = _operands(ka), np.roll(_operands(kb), 7)
     m, d, s = (np.empty_like(a) for _ in range(3))
     p = [x.ctypes.data_as(ctypes.c_void_p) for x in (a, b, m, d, s)]
@@ -72,6 +98,18 @@ def test_same_bits(lib, ka, kb):
             nan = np.isnan(ref)
             assert np.array_equal(np.isnan(got), nan)
             assert np.array_equal(got[~nan].view(np.uint64), ref[~nan].view(np.uint64))
+
+
+@pytest.mark.parametrize("ka", ["near", "sparse", "any", "special"])
+@pytest.mark.parametrize("kb", ["near", "sparse", "any", "special"])
+def test_same_bits(lib, ka, kb):
+    _same_bits(lib, ka, kb)
+
+
+@pytest.mark.parametrize("ka", ["near", "sparse", "ends"])
+@pytest.mark.parametrize("kb", ["near", "sparse", "ends"])
+def test_same_bits_from_the_worst_estimates(nudged, ka, kb):
+    _same_bits(nudged, ka, kb)
 
 
 @pytest.mark.parametrize("ka", ["near", "sparse", "any", "special"])
