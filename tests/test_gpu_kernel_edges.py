@@ -76,6 +76,53 @@ def test_newtonian_steps_bitwise(pkg, n, scale, K):
         assert np.array_equal(Ug.cpu().numpy(), U), (limiter, flux)
 
 
+@pytest.mark.parametrize("system", [0, 1])
+@pytest.mark.parametrize("n,K", [(2, (11, 9, 9)), (3, (11, 9, 9)), (4, (11, 9, 9)), (5, (11, 9, 9)), (6, (11, 9, 7)),
+                                 (7, (7, 5, 11)), (8, (7, 5, 11)), (2, (31, 5, 1)), (5, (31, 5, 1)), (8, (31, 5, 1))])
+def test_summaries_of_several_elements_per_cta(pkg, n, K, system):
+    """The summaries take ceil(E / 152) elements per CTA up to a largest group (6 for n <= 5, 4 for n = 6, 3
+    for n = 7, 8): that group with a short last CTA (891 = 6 * 148 + 3, 693 = 4 * 173 + 1, 385 = 3 * 128
+    + 1) and two elements with one left over (155), unphysical states in the last element among them,
+    against the oracle."""
+    import torch
+    kw = dict(system=system, K=K, n=n, flux=1, limiter=1, gamma=G, lo=(0,) * 3, hi=(1,) * 3)
+    om, gm = oracle.Mesh(oracle.MeshSpec(**kw)), pkg.Mesh(**kw)
+    xyz = om.coords()
+    U = om.from_prim(di.blast_sr(xyz, seed=3) if system else di.kh_ne(xyz - 0.5, seed=3))
+    assert np.array_equal(gm.summaries(_gpu(U)).cpu().numpy(), om.summaries(U))
+    V = U.copy()
+    if system:
+        V[[0, om.E // 2, om.E - 1], 4, n] *= -1.0  # every variable of these elements is replaced
+    Ug, t = _gpu(V), torch.zeros(om.E, dtype=torch.uint8, device="cuda")
+    V, to = om.limit(V)
+    gm.limit(Ug, t)
+    assert np.array_equal(t.cpu().numpy(), to) and np.array_equal(Ug.cpu().numpy(), V)
+    if system:
+        assert (to[[0, om.E // 2, om.E - 1]] == 31).all()
+
+
+@pytest.mark.parametrize("system,n,limiter", [(0, 4, 0), (0, 6, 1), (1, 5, 1), (1, 4, 0)])
+def test_captured_steps_bitwise(pkg, system, n, limiter):
+    """FP64 steps captured into a CUDA graph (their launches' programmatic edges with them) and replayed."""
+    import torch
+    kw = dict(system=system, K=(5, 3, 4), n=n, flux=1, limiter=limiter, gamma=G, lo=(-0.5,) * 3, hi=(0.5,) * 3)
+    om, gm = oracle.Mesh(oracle.MeshSpec(**kw)), pkg.Mesh(**kw)
+    xyz = om.coords()
+    U = om.from_prim(di.blast_sr(xyz + 0.5, seed=2) if system else di.kh_ne(xyz, seed=2))
+    Ug, dt = _gpu(U), torch.zeros(1, dtype=torch.float64, device="cuda")
+    g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=s):
+        for _ in range(2):
+            gm.rk3_step(Ug, cfl=0.2, dt_used=dt)
+    for _ in range(2):
+        g.replay()
+        for _ in range(2):
+            h = om.cfl_dt(U, 0.2)
+            U = om.rk3_step(U, h)
+        torch.cuda.synchronize()
+        assert np.array_equal(Ug.cpu().numpy(), U) and dt.item() == h
+
+
 @pytest.mark.parametrize("n", [2, 4, 6, 7, 8])
 def test_relativistic_steps_bitwise(pkg, n):
     for limiter, flux in ((0, 1), (1, 0)):
