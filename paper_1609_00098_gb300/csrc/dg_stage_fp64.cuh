@@ -23,12 +23,13 @@ struct StageShape64 {
     static constexpr int EPB = NP == 2 ? 4 : NP == 3 ? 2 : 1;
     static constexpr int THREADS = NP == 2 || NP == 4 ? 256 : NP == 3 || NP == 6 ? 288 : NP == 8 ? 512 : 384;
     static constexpr size_t SMEM = sizeof(double) * (15 * NN + 30 * N2) * EPB;
-    // CTAs that must fit on an SM, which caps the registers (36 for n = 2, 3, 40 for n = 5,
-    // 64 for n = 4, 80 for n = 7): more warps to hide the FP64 latency.  Step without a limiter at
-    // about 0.5 M nodes (KH, LLF), us, unbounded and so: n = 2 801, 646; n = 3 1000, 883; n
-    // = 4 1026, 979; n = 5 1080, 1045; n = 7 (one CTA per SM before) 1562, 1217.  n = 6 had
-    // four CTAs anyway, but spills less (24^3, limiter: 4225, 4106).  n = 8 keeps its own
-    // choice (64 registers, two CTAs: 1129; with 320 threads 1130 to 1224).
+    // CTAs that must fit on an SM, which caps the registers (32 for n = 2, 3, 40 for n = 5,
+    // 56 for n = 6, 64 for n = 4, 80 for n = 7, with up to 320, 84, 4, 0 and 104 bytes of
+    // spills): more warps to hide the FP64 latency.  Step without a limiter at about 0.5 M
+    // nodes (KH, LLF), us, unbounded and so: n = 2 801, 646; n = 3 1000, 883; n = 4 1026,
+    // 979; n = 5 1080, 1045; n = 7 (one CTA per SM before) 1562, 1217.  n = 6 had four CTAs
+    // anyway, but spills less (24^3, limiter: 4225, 4106).  n = 8 keeps its own choice (64
+    // registers, two CTAs: 1129; with 320 threads 1130 to 1224).
     static constexpr int MIN_CTAS = NP == 2 ? 7 : NP == 3 ? 6 : NP == 7 ? 2 : NP <= 6 ? 4 : 0;
 };
 
