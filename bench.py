@@ -403,12 +403,12 @@ def _con2prim_bench(pkg, torch, reps=3):
 # The same capture's pipe utilisation (ncu, % of peak sustained while active, mean
 # of the three launches) is reported beside the flop fractions.
 SR_STAGE_FLOPS = {"fp64": 18772488, "fp32": 358819649}
-SR_STAGE_PIPES = {"fp64_pipe_pct": 36.5, "fma_pipe_pct": 17.8, "alu_pipe_pct": 24.8, "tensor_pipe_pct": 5.1,
-                  "issue_active_pct": 47.4}
+SR_STAGE_PIPES = {"fp64_pipe_pct": 36.5, "fma_pipe_pct": 17.8, "alu_pipe_pct": 24.9, "tensor_pipe_pct": 5.1,
+                  "issue_active_pct": 47.3}
 SR_STAGE_SOURCES = ("paper_1609_00098_gb300/csrc/dg_mixed.cuh", "paper_1609_00098_gb300/csrc/dg_physics.cuh",
                     "paper_1609_00098_gb300/csrc/dg_c2p_net.cuh", "paper_1609_00098_gb300/csrc/dg_intfp64.cuh",
                     "paper_1609_00098_gb300/csrc/dg_polish64.cuh", "paper_1609_00098_gb300/csrc/dg_internal.h")
-SR_STAGE_SOURCES_SHA256 = "67b38175ec278a909c9615c0f60062441332c6a6086c8dd712239b5848948606"
+SR_STAGE_SOURCES_SHA256 = "4883ee8d1a24eb41ee0bc02acbb8499aa0bd827e602bc88d296e4cd04e47d7f2"
 # FMA throughput of this GPU (independent dependent-FMA chains, every SM busy;
 # flops count an FMA as two): FP64 1.20 TFLOP/s, FP32 75.0 TFLOP/s.
 FP64_PEAK_TFLOPS = 1.20

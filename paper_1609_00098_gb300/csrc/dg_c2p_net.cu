@@ -614,11 +614,12 @@ __global__ void __launch_bounds__(32 * NET_SLICES) k_net_reduce(const float *par
     if (k >= OFF_W2 && k < OFF_W2 + 4096) W2b[k - OFF_W2] = __float2bfloat16_rn(pk);
 }
 
-// An epoch (or NET_LAUNCH_BATCHES mini-batches of it) in one launch, by one cluster of CTAs that
-// keep the weights in shared memory: per mini-batch every CTA takes its tiles and writes its gradient into the
-// owners' shared memory (CTA r owns the parameters [r NET_OWN, (r + 1) NET_OWN)), a cluster
-// barrier, every owner sums its parameters' gradients in CTA order, takes the Adam step
-// and writes the new values into every CTA's copy of the weights, a second barrier.
+// An epoch (or NET_LAUNCH_BATCHES mini-batches of it) in one launch, by one cluster of CTAs
+// that keep the weights in shared memory: per mini-batch CTA r takes tile r and writes its
+// gradient into the owners' shared memory (CTA r owns the parameters [r NET_OWN, (r + 1)
+// NET_OWN)), a cluster barrier, every owner sums its parameters' gradients in the order of the
+// tiles, takes the Adam step and writes the new values into every CTA's copy of the weights,
+// a second barrier.
 //
 // Bound by the serial chain of a mini-batch (a tile's forward and backward, two
 // barriers and the exchange).  Launched per mini-batch, the same work is two launches

@@ -20,7 +20,7 @@ namespace dg {
 
 constexpr int NET_PARAMS = 4481;
 constexpr int OFF_W1 = 0, OFF_B1 = 192, OFF_W2 = 256, OFF_B2 = 4352, OFF_W3 = 4416, OFF_B3 = 4480;
-constexpr int NET_PARTIAL = NET_PARAMS + 1;  // gradient + loss per CTA
+constexpr int NET_PARTIAL = NET_PARAMS + 1;  // gradient + loss of a tile
 
 struct NetTileArgs {
     const float *P;              // FP32 parameters
@@ -28,7 +28,7 @@ struct NetTileArgs {
     const double *cons;          // 5 rows of `count`
     const double *p;             // true pressures (training) or nullptr
     double *guess;               // output guesses (inference) or nullptr
-    float *partial;              // [gridDim.x][NET_PARTIAL] gradient partials (training)
+    float *partial;              // [tile][NET_PARTIAL] gradients of the tiles (training)
     long long count;             // rows of cons
     long long first;             // first sample of this launch
     long long nsamp;             // samples in this launch (batch)
